@@ -35,6 +35,13 @@ struct BIdx {
 };
 __device__ __forceinline__ BIdx bidx(const Batch& b) {
   BIdx r;
+  if (b.n == 1) {   // a single solve: no divisions
+    r.nz = gridDim.z;
+    r.p = 0;
+    r.z = blockIdx.z;
+    r.off = 0;
+    return r;
+  }
   r.nz = gridDim.z / static_cast<unsigned>(b.n);
   r.p = static_cast<int>(blockIdx.z / r.nz);
   r.z = blockIdx.z % r.nz;

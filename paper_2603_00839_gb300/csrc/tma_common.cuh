@@ -33,9 +33,11 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(bar)));
   asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
 }
-// An mbarrier that completes its phase after `count` plain arrivals.
-__device__ __forceinline__ void mbar_init_n(uint64_t* bar, uint32_t count) {
+// Several barriers: initialise each, then one fence.
+__device__ __forceinline__ void mbar_init_raw(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(count));
+}
+__device__ __forceinline__ void mbar_init_fence() {
   asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
 }
 // One arrival (release semantics: this thread's earlier writes are visible
@@ -100,17 +102,21 @@ __device__ __forceinline__ void bulk_s2g_commit_and_wait_read() {
   asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
 }
 
+// One try: whether phase `parity` has completed.
+__device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(done)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return done != 0;
+}
+
 // Waits for phase `parity`; gives up after a bounded number of polls.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-  for (int it = 0; it < (1 << 22); ++it) {
-    uint32_t done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    if (done) return true;
-  }
+  for (int it = 0; it < (1 << 22); ++it)
+    if (mbar_try(bar, parity)) return true;
   return false;
 }
 

@@ -1,0 +1,62 @@
+"""Kernel variants that a size or an alignment selects, at the sizes where the choice changes.
+
+Each test compares a variant with the oracle or with the other variant on the
+same values, at the edges of its tiles: the last size of one rule, the first of
+the next, remainders of every tile dimension and the smallest tensors.
+"""
+import numpy as np
+import pytest
+
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def api():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2603_00839_gb300 import api as a
+    return a
+
+
+@pytest.fixture(scope="module")
+def h(api):
+    return api.Handle(0)
+
+
+def _rel(a, b):
+    return np.linalg.norm(a - b) / np.linalg.norm(b)
+
+
+# ------------------------------------------------------------------------ first sketch stage
+
+# 304 groups of 32 columns is the most a CTA per group takes; beyond, a CTA takes two
+@pytest.mark.parametrize("dims,sk", [
+    ((72, 9728), (20, 12)),        # 304 groups: one per CTA
+    ((72, 9729), (20, 12)),        # 305: two per CTA, the last CTA with one column
+    ((37, 9770), (37 - 1, 12)),    # rows that start on no 16-byte boundary (4-byte copies)
+    ((72, 21, 500), (20, 5, 30)),  # CTAs whose columns fall into several slabs of the next stage
+    ((40, 7, 1501), (8, 7, 20)),   # an unsketched mode between the two sketched ones
+    ((129, 33), (129 - 1, 7)),     # a K block of one value
+    ((66, 40), (1, 40)),           # one row of Theta, nothing after the first stage
+])
+def test_first_stage_column_groups(api, h, dims, sk):
+    X = np.random.default_rng(len(dims) + dims[1]).standard_normal(dims).astype(np.float32)
+    ref = oracle.sketch(X.astype(np.float64), oracle.sketch_matrices(dims, sk, 3, problem_id=0))
+    got = h.sketch(api.to_device(X), sk, 3)
+    torch.cuda.synchronize()
+    # the longest chain here: 1501 / 16 products per limb in the second stage, over eight warps, each sum
+    # truncated at 2^-23 of its size
+    assert _rel(got.cpu().double().numpy(), ref) < 1e-5
+
+
+def test_first_stage_does_not_depend_on_the_grouping(api, h):
+    """Mode-1 sketches of 10 000 columns at once and 1 000 at a time are the same bits."""
+    X = torch.randn((10000, 70), device="cuda", generator=torch.Generator("cuda").manual_seed(1)).t()
+    whole = h.sketch(X, (24, 10000), 5)
+    for c in range(0, 10000, 1000):
+        part = h.sketch(X[:, c:c + 1000], (24, 1000), 5)
+        torch.cuda.synchronize()
+        assert torch.equal(part, whole[:, c:c + 1000])
