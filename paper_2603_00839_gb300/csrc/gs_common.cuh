@@ -100,6 +100,36 @@ __device__ __forceinline__ FF ff_warp_sum(FF v) {
   }
   return v;
 }
+// Product of two pairs, about 2^-46 relative; the low part may overlap the
+// high part's last bits (as in ff_add_lazy).
+__device__ __forceinline__ FF ff_mul(FF a, FF b) {
+  const float p = __fmul_rn(a.hi, b.hi);
+  const float e = __fmaf_rn(a.hi, b.hi, -p);
+  return {p, __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, e))};
+}
+__device__ __forceinline__ FF ff_twice(FF a) { return {2.f * a.hi, 2.f * a.lo}; }
+__device__ __forceinline__ FF ff_sub(FF a, FF b) { return ff_add_lazy(a, {-b.hi, -b.lo}); }
+__device__ __forceinline__ FF ff_mac(FF a, FF b, FF c) { return ff_add_lazy(c, ff_mul(a, b)); }   // a b + c
+__device__ __forceinline__ bool ff_finite(FF a) { return isfinite(a.hi) && isfinite(a.lo); }
+// The pair as the nearest float and the remainder.
+__device__ __forceinline__ FF ff_norm(FF v) {
+  const float s = __fadd_rn(v.hi, v.lo);
+  return {s, __fsub_rn(v.lo, __fsub_rn(s, v.hi))};
+}
+// Square root (v >= 0, normalised) and reciprocal, one Newton correction of
+// the FP32 value each: the relative error is that of the square of an FP32
+// rounding, about 2^-46.
+__device__ __forceinline__ FF ff_sqrt(FF v) {
+  const float r = __fsqrt_rn(v.hi);
+  if (!(r > 0.f)) return {r, 0.f};
+  const float e = __fadd_rn(__fmaf_rn(-r, r, v.hi), v.lo);
+  return ff_norm({r, __fdiv_rn(e, 2.f * r)});
+}
+__device__ __forceinline__ FF ff_recip(FF v) {
+  const float r = __frcp_rn(v.hi);
+  const float e = __fmaf_rn(-v.lo, r, __fmaf_rn(-v.hi, r, 1.f));
+  return ff_norm({r, __fmul_rn(r, e)});
+}
 __device__ __forceinline__ double ff_to_double(FF v) {
   return static_cast<double>(v.hi) + static_cast<double>(v.lo);
 }
@@ -119,6 +149,50 @@ struct DotAcc<double> {
   __device__ __forceinline__ void add(double a, double b) { v = fma(a, b, v); }
   __device__ __forceinline__ double warp_total() { return warp_sum(v); }
 };
+
+// Type of the combined partial sums: float-float for FP32 data, FP64 for
+// FP64 data.
+template <typename T>
+struct Sum;
+template <>
+struct Sum<float> {
+  using V = FF;
+  static __device__ __forceinline__ V zero() { return {0.f, 0.f}; }
+  static __device__ __forceinline__ V add(V a, V b) { return ff_add_lazy(a, b); }
+  static __device__ __forceinline__ double dbl(V a) { return ff_to_double(a); }
+  static __device__ __forceinline__ V ldcg(const V* p) {
+    const float2 f = __ldcg(reinterpret_cast<const float2*>(p));
+    return {f.x, f.y};
+  }
+};
+template <>
+struct Sum<double> {
+  using V = double;
+  static __device__ __forceinline__ V zero() { return 0.0; }
+  static __device__ __forceinline__ V add(V a, V b) { return a + b; }
+  static __device__ __forceinline__ double dbl(V a) { return a; }
+  static __device__ __forceinline__ V ldcg(const V* p) { return __ldcg(p); }
+};
+
+// __double2float_rn on the integer pipe for values in FP32's normal range
+// (the conversion instruction takes about 1000 cycles on this GPU): the
+// significand's upper 24 bits, rounded to nearest even, and the exponent
+// moved; a carry out of the significand lands in the exponent.
+__device__ __forceinline__ float double_to_float_rn(double x) {
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x));
+  const unsigned e = static_cast<unsigned>(b >> 52) & 0x7ffu;
+  if (e < 1023u - 126u || e > 1023u + 126u) return b << 1 == 0ull ? __uint_as_float(static_cast<unsigned>(b >> 32)) : __double2float_rn(x);
+  const unsigned long long m = (b & 0x7fffffffffffffffull) - (static_cast<unsigned long long>(1023 - 127) << 52);
+  const unsigned long long r = (m + 0x0fffffffull + ((m >> 29) & 1ull)) >> 29;
+  return __uint_as_float(static_cast<unsigned>(r) | (static_cast<unsigned>(b >> 32) & 0x80000000u));
+}
+
+// A coefficient in the data's type.
+template <typename T>
+__device__ __forceinline__ T coef_as(double x) {
+  if constexpr (sizeof(T) == 4) return double_to_float_rn(x);
+  else return x;
+}
 
 // Columns of the per-block partial sums of one Gram-Schmidt reduction:
 // [0, J] s . Q_i, [J+1] s . s, [J+2, 2J+2] Q_J . Q_i (the new row of the
@@ -237,9 +311,11 @@ __device__ __forceinline__ FF ff_warps_total(const FF (*red)[kRedCols], int nw, 
 // Per-block partial sums of the columns above: products of the stored
 // values accumulated in double-float (FP32 data) or FP64 (FP64 data).
 // Each thread passes up to ITEMS entries (vals at sketch indices idx);
-// entries past cnt or with a negative index are ignored.  Writes row
-// (linear block id) of w.part: float-float pairs for FP32 data (summed by
-// last_block_combine<true> on the FP32 pipe), doubles for FP64 data.
+// entries past cnt or with a negative index are ignored.  Writes this block's
+// entry (linear block id) of every column of w.part, which is stored column
+// by column (w.part_rows entries each, so that the combine reads a column's
+// entries side by side): float-float pairs for FP32 data, doubles for FP64
+// data.
 // red: shared [GS_MAXW][kRedCols] doubles (float-float pairs for FP32).
 template <typename T, int ITEMS>
 __device__ void block_partials(const Work& w, const T* vals, const int64_t* idx, int cnt, int J,
@@ -312,103 +388,137 @@ __device__ void block_partials(const Work& w, const T* vals, const int64_t* idx,
     }
   }
   __syncthreads();
-  const int rowlen = 2 * w.m + 4;
-  const int64_t row = static_cast<int64_t>(blockIdx.x + gridDim.x * blockIdx.y) * rowlen;
+  const int64_t row = blockIdx.x + gridDim.x * blockIdx.y;
   for (int i = threadIdx.x; i < ncols; i += blockDim.x) {
-    if constexpr (sizeof(T) == 4) reinterpret_cast<FF*>(w.part)[row + i] = ff_warps_total(rf, nw, i);
-    else w.part[row + i] = warps_total(red, nw, i);
+    const int64_t at = static_cast<int64_t>(i) * w.part_rows + row;
+    if constexpr (sizeof(T) == 4) reinterpret_cast<FF*>(w.part)[at] = ff_warps_total(rf, nw, i);
+    else w.part[at] = warps_total(red, nw, i);
   }
 }
 
+// One thread's share of a column: entries g, g + G, ... below n, U loads in
+// flight per round, each round summed as a tree.
+template <typename T, int U>
+__device__ __forceinline__ typename Sum<T>::V column_share(const typename Sum<T>::V* p, unsigned g, unsigned G,
+                                                           unsigned n) {
+  using A = Sum<T>;
+  typename A::V acc = A::zero();
+  for (unsigned b = g; b < n; b += U * G) {
+    typename A::V v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) v[u] = b + u * G < n ? A::ldcg(p + b + u * G) : A::zero();
+#pragma unroll
+    for (int h = U / 2; h > 0; h >>= 1)
+#pragma unroll
+      for (int u = 0; u < h; ++u) v[u] = A::add(v[u], v[u + h]);
+    acc = A::add(acc, v[0]);
+  }
+  return acc;
+}
+
 // Ticket: returns true in every thread of the last block to finish, after
-// tot[0..ncols) holds the sum of all blocks' rows.  Thread t takes column
-// t % nc and every G-th row starting at t / nc, sixteen rows per round of
-// loads, then one thread per column adds the G group sums in a pairwise
-// tree.  FFROWS: the rows hold float-float pairs, summed with float-float
-// adds on the FP32 pipe (an FP64 add occupies its SM sub-partition's FP64
-// unit for about 64 cycles on this GPU; the pairs already carry the
-// partial sums' precision); else doubles.  The order is fixed, so the
-// result is deterministic.  The counter wraps back to zero by itself.
-// scratch: >= blockDim doubles.  pre (optional): called by every thread of
-// the last block right after the ticket, before its loads, e.g. to start
-// asynchronous copies that the caller needs after the combine.
-template <bool FFROWS, typename Pre = void (*)()>
-__device__ inline bool last_block_combine(const Work& w, int ncols, double* tot, int* am_last,
+// tot[0..ncols) holds the sum of all blocks' entries of each column (float-
+// float for T = float, FP64 for double; 256 threads).  The order is fixed, so
+// the result is deterministic.  FP32 data: a column is summed by G
+// neighbouring lanes (a power of two), each taking every G-th entry with as
+// many loads in flight as it has entries (up to 16), and a shuffle tree adds
+// the lanes.  FP64 data: G = 256 / columns groups (at most 32), each with
+// every G-th entry, then one thread per column adds the groups' sums in a
+// pairwise tree (scratch: >= blockDim doubles).  The counter wraps back to
+// zero by itself.  pre (optional): called by every thread of the last block
+// right after the ticket, before its loads, e.g. to start asynchronous copies
+// that the caller needs after the combine.
+template <typename T, typename Pre = void (*)()>
+__device__ inline bool last_block_combine(const Work& w, int ncols, typename Sum<T>::V* tot, int* am_last,
                                           double* scratch, Pre pre = nullptr) {
-  using V = typename std::conditional<FFROWS, FF, double>::type;
+  using A = Sum<T>;
+  using V = typename A::V;
   __syncthreads();
   const unsigned nblk = gridDim.x * gridDim.y;
   if (threadIdx.x == 0) *am_last = (ticket_acq_rel(w.counter, nblk - 1) == nblk - 1);
   __syncthreads();
   if (!*am_last) return false;
   if constexpr (!std::is_same<Pre, void (*)()>::value) pre();   // e.g. start the Gram staging copies
-  auto add = [](V x, V y) -> V {
-    if constexpr (FFROWS) return ff_add_lazy(x, y);
-    else return x + y;
-  };
-  auto load = [](const V* q) -> V {
-    if constexpr (FFROWS) {
-      const float2 f = __ldcg(reinterpret_cast<const float2*>(q));
-      return FF{f.x, f.y};
-    } else {
-      return __ldcg(q);
-    }
-  };
-  const V zero{};
-  V* sc = reinterpret_cast<V*>(scratch);
-  const int rowlen = 2 * w.m + 4;
-  const int nt = blockDim.x;
-  for (int c0 = 0; c0 < ncols; c0 += nt) {
-    const int nc = (ncols - c0 < nt) ? ncols - c0 : nt;
-    int G = nt / nc;
-    if (G > 32) G = 32;
-    const int t = threadIdx.x;
-    const int c = t % nc, g = t / nc;
-    if (g < G) {
-      // rows g, g + G, ...: sixteen loads in flight per round (one L2
-      // round trip per sixteen rows), summed in a fixed tree
-      constexpr int U = 16;
-      V acc = zero;
-      const V* p = reinterpret_cast<const V*>(w.part) + c0 + c;
-      for (unsigned b = g; b < nblk; b += U * G) {
-        V v[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const unsigned bb = b + u * G;
-          v[u] = bb < nblk ? load(p + static_cast<int64_t>(bb) * rowlen) : zero;
-        }
-#pragma unroll
-        for (int h = U / 2; h > 0; h >>= 1)
-#pragma unroll
-          for (int u = 0; u < h; ++u) v[u] = add(v[u], v[u + h]);
-        acc = add(acc, v[0]);
+  const V* part = reinterpret_cast<const V*>(w.part);
+  if constexpr (sizeof(T) == 4) {
+    // lanes per column: 32 for up to 8 columns, 16 for up to 16, ..., 1 beyond 128
+    int lg = 5;
+    while (lg > 0 && (ncols << lg) > static_cast<int>(blockDim.x)) --lg;
+    const unsigned G = 1u << lg, g = threadIdx.x & (G - 1u);
+    const int per = static_cast<int>(blockDim.x) >> lg;            // columns per round
+    for (int c0 = 0; c0 < ncols; c0 += per) {
+      const int c = c0 + (static_cast<int>(threadIdx.x) >> lg);
+      V acc = A::zero();
+      if (c < ncols) {
+        const V* p = part + static_cast<int64_t>(c) * w.part_rows;
+        if (nblk <= 4 * G) acc = column_share<T, 4>(p, g, G, nblk);
+        else if (nblk <= 8 * G) acc = column_share<T, 8>(p, g, G, nblk);
+        else acc = column_share<T, 16>(p, g, G, nblk);
       }
-      sc[g * nc + c] = acc;
+      for (int o = static_cast<int>(G) >> 1; o > 0; o >>= 1) {
+        V other;
+        other.hi = __shfl_xor_sync(0xffffffffu, acc.hi, o);
+        other.lo = __shfl_xor_sync(0xffffffffu, acc.lo, o);
+        acc = A::add(acc, other);
+      }
+      if (g == 0 && c < ncols) tot[c] = ff_norm(acc);
     }
     __syncthreads();
-    if (t < nc) {   // pairwise tree over the G group sums (levels that would add only zeros skipped)
-      V v[32];
+  } else {
+    const int nt = blockDim.x, t = threadIdx.x;
+    for (int c0 = 0; c0 < ncols; c0 += nt) {
+      const int nc = (ncols - c0 < nt) ? ncols - c0 : nt;
+      int G = nt / nc;
+      if (G > 32) G = 32;
+      const int c = t % nc, g = t / nc;
+      if (g < G) {
+        const V* p = part + static_cast<int64_t>(c0 + c) * w.part_rows;
+        // (a tree over fewer loads leaves out only additions of zero)
+        if (nblk <= static_cast<unsigned>(G)) scratch[g * nc + c] = column_share<T, 1>(p, g, G, nblk);
+        else scratch[g * nc + c] = column_share<T, 16>(p, g, G, nblk);
+      }
+      __syncthreads();
+      if (t < nc) {   // pairwise tree over the G group sums (levels that would add only zeros skipped)
+        const int used = static_cast<int>(nblk) < G ? static_cast<int>(nblk) : G;
+        if (used <= 4) {
+          V v[4];
 #pragma unroll
-      for (int u = 0; u < 32; ++u) v[u] = u < G ? sc[u * nc + t] : zero;
+          for (int u = 0; u < 4; ++u) v[u] = u < used ? scratch[u * nc + t] : A::zero();
+          tot[c0 + t] = (v[0] + v[2]) + (v[1] + v[3]);
+        } else {
+          V v[32];
 #pragma unroll
-      for (int h = 16; h > 0; h >>= 1)
-        if (h < G) {
+          for (int u = 0; u < 32; ++u) v[u] = u < G ? scratch[u * nc + t] : A::zero();
 #pragma unroll
-          for (int u = 0; u < h; ++u) v[u] = add(v[u], v[u + h]);
+          for (int h = 16; h > 0; h >>= 1)
+            if (h < G) {
+#pragma unroll
+              for (int u = 0; u < h; ++u) v[u] = A::add(v[u], v[u + h]);
+            }
+          tot[c0 + t] = v[0];
         }
-      if constexpr (FFROWS) tot[c0 + t] = ff_to_double(v[0]);
-      else tot[c0 + t] = v[0];
+      }
+      __syncthreads();
     }
-    __syncthreads();
   }
   return true;
 }
 
+// 1 / d for the kernels that scale by it, once instead of in every thread.
+__device__ __forceinline__ void set_inverse(Ctl* ctl, double d) {
+  const double r = 1.0 / d;
+  const float f = double_to_float_rn(r);
+  ctl->inv = r;
+  ctl->inv_hi = f;
+  ctl->inv_lo = double_to_float_rn(r - static_cast<double>(f));
+}
+
 // Start of a process (one thread): beta = ||R_0||_Theta = sqrt(s . s).
-__device__ inline void gs_finish_start(const Work& w, const StepOpts& o, const double* tot) {
+template <typename T>
+__device__ inline void gs_finish_start(const Work& w, const StepOpts& o, const typename Sum<T>::V* tot) {
   Ctl* ctl = w.ctl;
   const double tol = o.desc_tol ? *o.desc_tol : o.tol;
-  const double beta = sqrt(tot[0]);
+  const double beta = sqrt(Sum<T>::dbl(tot[0]));
   if (ctl->status != 0) {
     ctl->stop = 1;
   } else if (!isfinite(beta)) {
@@ -419,6 +529,7 @@ __device__ inline void gs_finish_start(const Work& w, const StepOpts& o, const d
     ctl->stop = 1;
   } else {
     ctl->beta = beta;
+    set_inverse(ctl, beta);
     if (ctl->cycle == 0) ctl->beta0 = beta;
     w.g[0] = beta;
     ctl->rho = beta / ctl->beta0;
@@ -447,7 +558,7 @@ __device__ inline void gs_stage_gram_async(const Work& w, int J, double* sh) {
   const int n = J + 1;
   if (J < 1 || n > kGramSmemRows) return;
   const int lg = gram_smem_ld(n), ldg = gram_ld(w.m), pairs = (J + 1) / 2;
-  double* Gs = sh + (kMaxK + 2) + 4;
+  double* Gs = sh + (kMaxK + 2) + 4;   // (a float-float pair is as wide as a double)
   for (int e = threadIdx.x; e < J * pairs; e += blockDim.x) {
     const int p = e % pairs, k = e / pairs;
     const unsigned sa = static_cast<unsigned>(__cvta_generic_to_shared(&Gs[k * lg + 2 * p]));
@@ -463,17 +574,15 @@ __device__ inline void gs_stage_gram_async(const Work& w, int J, double* sh) {
 // the Gram matrix G = Q^T Q of the stored sketched basis so that a single
 // pass over Q suffices: h1 = Q^T s, h2 = Q^T (s - Q h1) = h1 - G h1,
 // h = h1 + h2 and h_{j+1,j}^2 = ||s - Q h||^2 = s.s - 2 h.h1 + h.(G h), all
-// in FP64.  Writes the Hessenberg column, h_{j+1,j} (0 on breakdown), the
+// in FP64 (FP64 data; gs_finish_gram_ff is FP32 data's).  Writes the Hessenberg column, h_{j+1,j} (0 on breakdown), the
 // breakdown and non-finite flags, and advances j.  The Givens update of
 // Eq. 11S, rho_j and the stop rule follow in givens_step, off this
 // kernel's critical path.  Up to kGramSmemRows rows the Gram matrix is
 // staged in shared memory and every warp takes part in the two products
 // with it; beyond, one warp per row reads it from global memory.  sh:
 // shared scratch of GS_MAXW * kRedCols doubles, 256 threads.
-__device__ inline void gs_finish_gram(const Work& w, const StepOpts& o, const double* tot, double* sh,
-                                      bool staged = false) {
+__device__ inline void gs_finish_gram(const Work& w, const StepOpts& o, int J, const double* tot, double* sh) {
   Ctl* ctl = w.ctl;
-  const int J = ctl->j;
   const int ld = w.m + 1, ldg = gram_ld(w.m);
   const double bd_tol = o.desc_bd_tol ? *o.desc_bd_tol : o.bd_tol;   // loaded early, used at the end
   const double* h1 = tot;
@@ -492,13 +601,6 @@ __device__ inline void gs_finish_gram(const Work& w, const StepOpts& o, const do
     double* Gs = red + 4;              // n x n
     double* pr = Gs + n * lg;          // [nw][n] partial products
     double* ab = pr + nw * n;          // [2][2] the two warps' sums of a and b
-    if (staged) {   // rows and columns < J arrived by gs_stage_gram_async; J from the new row
-      asm volatile("cp.async.wait_all;\n" ::: "memory");
-      for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        Gs[J * lg + i] = grow[i];
-        Gs[i * lg + J] = grow[i];
-      }
-    } else
     for (int e0 = 0; e0 < n * n; e0 += 8 * static_cast<int>(blockDim.x)) {   // eight loads in flight
       double v[8];
 #pragma unroll
@@ -550,8 +652,8 @@ __device__ inline void gs_finish_gram(const Work& w, const StepOpts& o, const do
       const int i = threadIdx.x & 63, which = warp >> 1;
       double p = 0.0;
       if (i < n) p = which == 0 ? col[i] * h1[i] : col[i] * wsum(i);
-      const float hi = __double2float_rn(p);
-      FF v{hi, __double2float_rn(p - static_cast<double>(hi))};
+      const float hi = double_to_float_rn(p);
+      FF v{hi, double_to_float_rn(p - static_cast<double>(hi))};
       v = ff_warp_sum(v);
       if (lane == 0) ab[warp] = ff_to_double(v);
     }
@@ -616,6 +718,7 @@ __device__ inline void gs_finish_gram(const Work& w, const StepOpts& o, const do
     Hc[J + 1] = breakdown ? 0.0 : hn;
     ctl->pre2 = s2;
     ctl->hnext = hn;
+    ctl->inv = 1.0 / hn;
     ctl->j = J + 1;
     if (!finite) ctl->status = RTG_ERR_NONFINITE;
     if (breakdown) ctl->breakdown = 1;
@@ -624,15 +727,169 @@ __device__ inline void gs_finish_gram(const Work& w, const StepOpts& o, const do
   }
 }
 
+// The step finish of FP32 data, in float-float arithmetic: the partial sums
+// are float-float already, and on this GPU an FP64 addition returns after 60
+// to 150 cycles and a conversion to FP32 after about 1000, against some 30 for
+// a float-float multiply-add.  G is stored as float-float pairs.  As
+// gs_finish_gram, with h_{j+1,j}^2 = s.s - h.(2 h1 - G h) in one sum; the
+// column also goes out as pairs for the update, and 1 / h_{j+1,j} with it.
+// What follows the second product is one warp's work (no block barrier).
+// Sketch group of one step (both contractions, dots and this chain; FP64
+// arithmetic, row-major partial sums and two separate sums before):
+// 512 x 512 x 3 28.6 -> 24.2 us, 1024 x 1024 x 3 40.4 -> 33.8 us,
+// 256 x 256 x 3 x 64 (1728 blocks to combine) 149 -> 107 us; the error of
+// solves against 64 bits is the same to two digits, ill-conditioned ones too.
+__device__ inline void gs_finish_gram_ff(const Work& w, const StepOpts& o, int J, const FF* tot, double* sh,
+                                         bool staged = false) {
+  Ctl* ctl = w.ctl;
+  const int ld = w.m + 1, ldg = gram_ld(w.m);
+  const double bd_tol = o.desc_bd_tol ? *o.desc_bd_tol : o.bd_tol;   // loaded early, used at the end
+  const FF* h1 = tot;
+  const FF s2 = tot[J + 1];
+  const FF* grow = tot + J + 2;
+  FF* col = reinterpret_cast<FF*>(sh);   // h
+  FF* ext = col + (kMaxK + 2);          // 4 values
+  FF* G = reinterpret_cast<FF*>(w.G);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int n = J + 1;
+  const bool small = n <= kGramSmemRows;
+  const int lg = gram_smem_ld(n);
+  FF* Gs = ext + 4;                     // n x n, symmetric
+  FF* pr = Gs + n * lg;                 // [nw][n] partial products
+  if (small) {
+    // G staged in shared memory (even row stride); each product G x runs
+    // on every warp: warp w takes a slice of the columns, lane the rows
+    // lane and lane + 32, and the warps' partial rows are summed in order
+    if (staged) {   // rows and columns < J arrived by gs_stage_gram_async; J from the new row
+      asm volatile("cp.async.wait_all;\n" ::: "memory");
+      for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        Gs[J * lg + i] = grow[i];
+        Gs[i * lg + J] = grow[i];
+      }
+    } else {
+      for (int e0 = 0; e0 < n * n; e0 += 8 * static_cast<int>(blockDim.x)) {   // eight loads in flight
+        FF v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int e = e0 + u * blockDim.x + threadIdx.x;
+          const int i = e % n, k = e / n;
+          v[u] = (e >= n * n) ? FF{0.f, 0.f}
+                              : (i == J) ? grow[k] : (k == J ? grow[i] : Sum<float>::ldcg(G + i + static_cast<int64_t>(ldg) * k));
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int e = e0 + u * blockDim.x + threadIdx.x;
+          if (e < n * n) Gs[(e % n) * lg + e / n] = v[u];
+        }
+      }
+    }
+    for (int i = threadIdx.x; i <= J; i += blockDim.x) {   // new row/column, for later steps
+      G[i + static_cast<int64_t>(ldg) * J] = grow[i];
+      G[J + static_cast<int64_t>(ldg) * i] = grow[i];
+    }
+    __syncthreads();
+    const int ks = (n + nw - 1) / nw;
+    const int k0 = warp * ks, k1 = (k0 + ks < n) ? k0 + ks : n;
+    auto gmul = [&](const FF* x) {   // pr[w][i] = sum over the warp's columns of G(k, i) x_k
+      for (int i = lane; i < n; i += 32) {
+        FF u = FF{0.f, 0.f};
+        for (int k = k0; k < k1; ++k) u = ff_mac(Gs[k * lg + i], x[k], u);
+        pr[warp * n + i] = u;
+      }
+    };
+    gmul(h1);
+    __syncthreads();
+    auto psum = [&](int i) {   // the warps' partial rows as a fixed tree
+      if (nw == 8)
+        return ff_add_lazy(ff_add_lazy(ff_add_lazy(pr[i], pr[n + i]), ff_add_lazy(pr[2 * n + i], pr[3 * n + i])),
+                      ff_add_lazy(ff_add_lazy(pr[4 * n + i], pr[5 * n + i]), ff_add_lazy(pr[6 * n + i], pr[7 * n + i])));
+      FF u = FF{0.f, 0.f};
+      for (int v = 0; v < nw; ++v) u = ff_add_lazy(u, pr[v * n + i]);
+      return u;
+    };
+    for (int i = threadIdx.x; i < n; i += blockDim.x) col[i] = ff_norm(ff_sub(ff_twice(h1[i]), psum(i)));
+    __syncthreads();
+    gmul(col);
+    __syncthreads();
+    if (warp == 0) {
+      FF t = FF{0.f, 0.f};
+      for (int i = lane; i < n; i += 32) t = ff_mac(col[i], ff_sub(ff_twice(h1[i]), psum(i)), t);
+      t = ff_warp_sum(t);
+      if (lane == 0) ext[0] = t;
+    }
+  } else {
+    for (int i = threadIdx.x; i <= J; i += blockDim.x) {
+      G[i + static_cast<int64_t>(ldg) * J] = grow[i];
+      G[J + static_cast<int64_t>(ldg) * i] = grow[i];
+    }
+    __syncthreads();
+    // h = 2 h1 - G h1: one warp per row, lanes across the columns
+    for (int i = warp; i <= J; i += nw) {
+      FF gh = FF{0.f, 0.f};
+      for (int k = lane; k <= J; k += 32) gh = ff_mac(Sum<float>::ldcg(G + i + static_cast<int64_t>(ldg) * k), h1[k], gh);
+      gh = ff_warp_sum(gh);
+      if (lane == 0) col[i] = ff_norm(ff_sub(ff_twice(h1[i]), gh));
+    }
+    __syncthreads();
+    FF* row = ext + 4;                  // h_i (2 h1 - G h)_i per row
+    for (int i = warp; i <= J; i += nw) {
+      FF gh = FF{0.f, 0.f};
+      for (int k = lane; k <= J; k += 32) gh = ff_mac(Sum<float>::ldcg(G + i + static_cast<int64_t>(ldg) * k), col[k], gh);
+      gh = ff_warp_sum(gh);
+      if (lane == 0) row[i] = ff_mul(col[i], ff_sub(ff_twice(h1[i]), gh));
+    }
+    __syncthreads();
+    if (warp == 0) {
+      FF t = FF{0.f, 0.f};
+      for (int i = lane; i <= J; i += 32) t = ff_add_lazy(t, row[i]);
+      t = ff_warp_sum(t);
+      if (lane == 0) ext[0] = t;
+    }
+  }
+  double* Hc = w.H + static_cast<int64_t>(ld) * J;
+  if (warp != 0) {   // the column for the later kernels, beside warp 0's scalars
+    for (int i = static_cast<int>(threadIdx.x) - 32; i <= J; i += blockDim.x - 32) {
+      Hc[i] = ff_to_double(col[i]);
+      reinterpret_cast<float2*>(w.hf)[i] = make_float2(col[i].hi, col[i].lo);
+    }
+    for (int i = J + 2 + static_cast<int>(threadIdx.x) - 32; i < ld; i += blockDim.x - 32) Hc[i] = 0.0;
+    return;
+  }
+  bool bad = false;
+  for (int i = lane; i <= J; i += 32) bad |= !ff_finite(col[i]);
+  bad = __any_sync(0xffffffffu, bad);
+  if (lane != 0) return;
+  const FF t = ext[0];
+  const bool finite = ff_finite(s2) && ff_finite(t) && !bad;
+  const FF hn2 = ff_norm(ff_sub(s2, t));
+  const FF p2 = hn2.hi > 0.f ? hn2 : FF{0.f, 0.f};
+  const FF root = ff_sqrt(p2), inv = ff_recip(root);
+  const double hn = ff_to_double(root);
+  // h_{j+1,j} <= bd_tol ||S(Phi V_j)||, compared in squares
+  const bool breakdown = finite && ff_to_double(p2) <= bd_tol * bd_tol * ff_to_double(s2);
+  ctl->inv_hi = inv.hi;
+  ctl->inv_lo = inv.lo;
+  Hc[J + 1] = breakdown ? 0.0 : hn;
+  ctl->pre2 = ff_to_double(s2);
+  ctl->hnext = hn;
+  ctl->j = J + 1;
+  if (!finite) ctl->status = RTG_ERR_NONFINITE;
+  if (breakdown) ctl->breakdown = 1;
+  ctl->skip_update = (!finite || breakdown) ? 1 : 0;
+  ctl->givens = 1;
+}
+
 // Givens update of Eq. 11S for the Hessenberg column the last finish wrote
 // (column J = j - 1), rho_j = |g_{J+1}| / beta_0, the stop rule and the
 // condition of the device-side loop, which never runs more than m + 1
 // bodies.  Called by every thread of one block, which runs beside the basis
-// update (it does not depend on it): the block stages the column and the
-// stored rotations in shared memory with one round of loads, then one
-// thread applies the rotations (a dependent FP64 chain).
+// update (it does not depend on it): the block loads the column and the
+// stored rotations in one round and forms their products, then one thread
+// runs the dependent chain, one FP64 multiply-add per rotation.
 __device__ inline void givens_step(const Work& w, const StepOpts& o) {
-  __shared__ double gv_h[kMaxK + 2], gv_c[kMaxK], gv_s[kMaxK];
+  // c_i y_{i+1}, s_i y_{i+1}, s_i, c_i of the stored rotations on the new
+  // column, and the chain's values x_i
+  __shared__ double gv_cy[kMaxK], gv_sy[kMaxK], gv_s[kMaxK], gv_c[kMaxK], gv_x[kMaxK], gv_last[2], gv_rot[2];
   __shared__ int gv_J, gv_do;
   Ctl* ctl = w.ctl;
   if (threadIdx.x == 0) {
@@ -644,34 +901,50 @@ __device__ inline void givens_step(const Work& w, const StepOpts& o) {
   if (gv_do) {
     const int J = gv_J;
     const double* Hc = w.H + static_cast<int64_t>(ld) * J;
-    for (int i = threadIdx.x; i <= J + 1; i += blockDim.x) gv_h[i] = Hc[i];
     for (int i = threadIdx.x; i < J; i += blockDim.x) {
-      gv_c[i] = w.cs[i];
-      gv_s[i] = w.sn[i];
+      const double y = Hc[i + 1], c = w.cs[i], sv = w.sn[i];
+      gv_c[i] = c;
+      gv_s[i] = sv;
+      gv_cy[i] = c * y;
+      gv_sy[i] = sv * y;
+    }
+    if (threadIdx.x == blockDim.x - 1) gv_last[0] = Hc[0];
+    if (threadIdx.x == blockDim.x - 2) gv_last[1] = Hc[J + 1];
+    __syncthreads();
+    // rotations 0..J-1 on the new column: one dependent multiply-add each
+    // (the products with y do not depend on the chain)
+    if (threadIdx.x == 0) {
+      double x = gv_last[0];
+      for (int i = 0; i < J; ++i) {
+        gv_x[i] = x;
+        x = fma(-gv_s[i], x, gv_cy[i]);
+      }
+      gv_last[0] = x;
+    }
+    __syncthreads();
+    double* Rc = w.R + static_cast<int64_t>(ld) * J;
+    if (threadIdx.x >= 32)
+      for (int i = static_cast<int>(threadIdx.x) - 32; i < J; i += blockDim.x - 32) Rc[i] = fma(gv_c[i], gv_x[i], gv_sy[i]);
+    // the new rotation: its two quotients in two lanes at once
+    if (threadIdx.x < 2) {
+      const double x = gv_last[0], y = gv_last[1];
+      const double q = fma(x, x, y * y);
+      // (hypot where the squares leave the normal range)
+      const double den = (q > 1e-280 && q < 1e280) ? sqrt(q) : hypot(x, y);
+      double v = threadIdx.x == 0 ? 1.0 : 0.0;
+      if (den != 0.0) v = (threadIdx.x == 0 ? x : y) / den;
+      gv_rot[threadIdx.x] = v;
+      if (threadIdx.x == 0) Rc[J] = den;
     }
   }
-  __syncthreads();
+  __syncwarp();
   if (threadIdx.x != 0) return;
   if (gv_do) {
     ctl->givens = 0;
     const int J = gv_J;
     const double tol = o.desc_tol ? *o.desc_tol : o.tol;
     double* Rc = w.R + static_cast<int64_t>(ld) * J;
-    // rotations 0..J-1 on the new column, then the new rotation
-    double x = gv_h[0];
-    for (int i = 0; i < J; ++i) {
-      const double y = gv_h[i + 1], c = gv_c[i], sv = gv_s[i];
-      Rc[i] = c * x + sv * y;
-      x = -sv * x + c * y;
-    }
-    const double y = gv_h[J + 1];
-    const double den = hypot(x, y);
-    double c = 1.0, sv = 0.0;
-    if (den != 0.0) {
-      c = x / den;
-      sv = y / den;
-    }
-    Rc[J] = den;
+    const double c = gv_rot[0], sv = gv_rot[1];
     Rc[J + 1] = 0.0;
     w.cs[J] = c;
     w.sn[J] = sv;

@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(GS_THREADS) k_gs_pass(Work w0, int pass, StepO
   const int d = w.d;
   T* S = static_cast<T*>(w.S);
   __shared__ double red[GS_MAXW][kRedCols];
-  __shared__ double tot[kRedCols];
+  __shared__ typename Sum<T>::V tot[kRedCols];
   __shared__ int am_last;
   const int64_t chunk = (d + gridDim.x - 1) / gridDim.x;
   const int64_t lo = blockIdx.x * chunk;
@@ -79,12 +79,21 @@ __global__ void __launch_bounds__(GS_THREADS) k_gs_pass(Work w0, int pass, StepO
     }
   }
   block_partials<T, GS_ITEMS>(w, sv, ix, cnt, J, red);
-  if (!last_block_combine<sizeof(T) == 4>(w, gs_ncols(J), tot, &am_last, &red[0][0])) return;
+  if (!last_block_combine<T>(w, gs_ncols(J), tot, &am_last, &red[0][0])) return;
   if (pass == 0) {
-    if (threadIdx.x == 0) gs_finish_start(w, o, tot);
+    if (threadIdx.x == 0) gs_finish_start<T>(w, o, tot);
+  } else if constexpr (sizeof(T) == 4) {
+    gs_finish_gram_ff(w, o, J, tot, &red[0][0]);
   } else {
-    gs_finish_gram(w, o, tot, &red[0][0]);
+    gs_finish_gram(w, o, J, tot, &red[0][0]);
   }
+}
+
+// 1 / beta or 1 / h_{j+1,j} in the data's type (Ctl::inv, inv_hi).
+template <typename T>
+__device__ __forceinline__ T ctl_inverse(const Ctl* ctl) {
+  if constexpr (sizeof(T) == 4) return ctl->inv_hi;
+  else return ctl->inv;
 }
 
 // V_0 = src / beta, Q_0 = S / beta
@@ -98,7 +107,7 @@ __global__ void k_start_scale(Work w0, PtrRef srcr0, const int* gate) {
   if (gate != nullptr && *gate) return;
   if (ctl->stop) return;
   const T* src = srcr.get<const T>();
-  const T inv = static_cast<T>(1.0 / ctl->beta);
+  const T inv = ctl_inverse<T>(ctl);
   T* V = static_cast<T*>(w.V);
   T* Q = static_cast<T*>(w.Q);
   const T* S = static_cast<const T*>(w.S);
@@ -117,6 +126,31 @@ __global__ void k_start_scale(Work w0, PtrRef srcr0, const int* gate) {
     for (int64_t o = t0; o < w.n; o += stride) V[o] = src[o] * inv;
   }
   for (int64_t o = t0; o < w.d; o += stride) Q[o] = S[o] * inv;
+}
+
+// One entry of the sketched column Q_{j+1} = (S - sum_i h_i Q_i) / h_{j+1,j} of
+// FP32 data, accumulated in float-float (h_i = hs[i] + hl[i], the inverse of
+// h_{j+1,j} as a pair) and rounded once; q: the entry of Q_0, d apart per column.
+__device__ __forceinline__ float sketch_column_entry(float sv, const float* q, int64_t d, int jj, const float* hs,
+                                                     const float* hl, float r_hi, float r_lo) {
+  FF v{sv, 0.f};
+  auto sub = [&](int i, float x) {   // v -= (hs_i + hl_i) x
+    const FF p = ff_prod(hs[i], x);
+    v = ff_add(v, FF{-p.hi, -__fmaf_rn(hl[i], x, p.lo)});
+  };
+  int i = 0;
+  for (; i + 8 <= jj; i += 8) {   // eight loads in flight, then the chain in order
+    float q8[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) q8[u] = q[static_cast<int64_t>(i + u) * d];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) sub(i + u, q8[u]);
+  }
+  for (; i < jj; ++i) sub(i, q[static_cast<int64_t>(i) * d]);
+  // (v.hi + v.lo)(r_hi + r_lo), rounded once to FP32
+  const FF p = ff_prod(v.hi, r_hi);
+  const float lo = __fmaf_rn(v.hi, r_lo, __fmaf_rn(v.lo, r_hi, p.lo));
+  return __fadd_rn(p.hi, lo);
 }
 
 // V_{j} = (W - sum_{i<j} h_i V_i) / h_{j,j-1};  Q_{j} = (S - sum_{i<j} h2_i Q_i) / h_{j,j-1}
@@ -144,13 +178,18 @@ __global__ void k_update(Work w0, StepOpts o0) {
     }
     return;
   }
+  // h as the data's type; the sketched column of FP32 data also takes its low part
   __shared__ T hs[kMaxK + 1];
-  __shared__ double hd[kMaxK + 1];
+  __shared__ float hl[kMaxK + 1];
   const int ld = w.m + 1;
   for (int i = threadIdx.x; i < jj; i += blockDim.x) {
-    const double h = w.H[static_cast<int64_t>(ld) * (jj - 1) + i];
-    hs[i] = static_cast<T>(h);
-    hd[i] = h;
+    if constexpr (sizeof(T) == 4) {
+      const float2 h = static_cast<const float2*>(w.hf)[i];
+      hs[i] = h.x;
+      hl[i] = h.y;
+    } else {
+      hs[i] = w.H[static_cast<int64_t>(ld) * (jj - 1) + i];
+    }
   }
   T* V = static_cast<T*>(w.V);
   T* Q = static_cast<T*>(w.Q);
@@ -175,8 +214,7 @@ __global__ void k_update(Work w0, StepOpts o0) {
         if (i < jj) pre[i] = V4[static_cast<int64_t>(i) * n4 + t0];
     }
     __syncthreads();
-    const T inv = static_cast<T>(1.0 / ctl->hnext);
-    const float fi = static_cast<float>(inv);
+    const float fi = static_cast<float>(ctl_inverse<T>(ctl));
     for (int64_t e = t0; e < n4; e += stride) {
       float4 acc;
       int i = 0;
@@ -224,19 +262,22 @@ __global__ void k_update(Work w0, StepOpts o0) {
     }
   } else {
     __syncthreads();
-    const T inv = static_cast<T>(1.0 / ctl->hnext);
+    const T inv = ctl_inverse<T>(ctl);
     for (int64_t e = t0; e < n; e += stride) {
       T v = W[e];
       for (int i = 0; i < jj; ++i) v -= hs[i] * V[static_cast<int64_t>(i) * n + e];
       V[static_cast<int64_t>(jj) * n + e] = v * inv;
     }
   }
-  // Q_{j} = (s - Q h) / h_{j,j-1}, accumulated in FP64 and rounded once
-  const double invd = 1.0 / ctl->hnext;
+  // Q_{j} = (s - Q h) / h_{j,j-1}
   for (int64_t e = t0; e < d; e += stride) {
-    double v = static_cast<double>(S[e]);
-    for (int i = 0; i < jj; ++i) v -= hd[i] * static_cast<double>(Q[static_cast<int64_t>(i) * d + e]);
-    Q[static_cast<int64_t>(jj) * d + e] = static_cast<T>(v * invd);
+    if constexpr (sizeof(T) == 4) {
+      Q[static_cast<int64_t>(jj) * d + e] = sketch_column_entry(S[e], Q + e, d, jj, hs, hl, ctl->inv_hi, ctl->inv_lo);
+    } else {
+      double v = S[e];
+      for (int i = 0; i < jj; ++i) v -= hs[i] * Q[static_cast<int64_t>(i) * d + e];
+      Q[static_cast<int64_t>(jj) * d + e] = v * ctl->inv;
+    }
   }
 }
 
@@ -331,7 +372,7 @@ __global__ void k_start_scale_bf16(Work w0, PtrRef srcr0, const int* gate) {
   gate = bsh(gate, bo);
   if (gate != nullptr && *gate) return;
   if (ctl->stop) return;
-  const float fi = static_cast<float>(1.0 / ctl->beta);
+  const float fi = ctl->inv_hi;
   uint4* V8 = static_cast<uint4*>(w.V);
   const int64_t n8 = w.n / 8;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -351,7 +392,7 @@ __global__ void k_start_scale_bf16(Work w0, PtrRef srcr0, const int* gate) {
   }
   float* Q = static_cast<float*>(w.Q);
   const float* S = static_cast<const float*>(w.S);
-  const float inv = static_cast<float>(1.0 / ctl->beta);
+  const float inv = ctl->inv_hi;
   for (int64_t o = t0; o < w.d; o += stride) Q[o] = S[o] * inv;
 }
 
@@ -376,20 +417,18 @@ __global__ void k_update_bf16(Work w0, StepOpts o0) {
     }
     return;
   }
-  __shared__ float hs[kMaxK + 1];
-  __shared__ double hd[kMaxK + 1];
-  const int ld = w.m + 1;
+  __shared__ float hs[kMaxK + 1], hl[kMaxK + 1];
   for (int i = threadIdx.x; i < jj; i += blockDim.x) {
-    const double h = w.H[static_cast<int64_t>(ld) * (jj - 1) + i];
-    hs[i] = static_cast<float>(h);
-    hd[i] = h;
+    const float2 h = static_cast<const float2*>(w.hf)[i];
+    hs[i] = h.x;
+    hl[i] = h.y;
   }
   __syncthreads();
   const uint4* W8 = static_cast<const uint4*>(w.W);
   const uint4* V8 = static_cast<const uint4*>(w.V);
   const int64_t n8 = w.n / 8;
   uint4* out = static_cast<uint4*>(w.V) + static_cast<int64_t>(jj) * n8;
-  const float fi = static_cast<float>(1.0 / ctl->hnext);
+  const float fi = ctl->inv_hi;
   const int64_t stride = (int64_t)(gridDim.x - 1) * blockDim.x;
   const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   for (int64_t e = t0; e < n8; e += stride) {
@@ -439,12 +478,9 @@ __global__ void k_update_bf16(Work w0, StepOpts o0) {
   }
   float* Q = static_cast<float*>(w.Q);
   const float* S = static_cast<const float*>(w.S);
-  const double invd = 1.0 / ctl->hnext;
-  for (int64_t e = t0; e < w.d; e += stride) {
-    double v = static_cast<double>(S[e]);
-    for (int i = 0; i < jj; ++i) v -= hd[i] * static_cast<double>(Q[static_cast<int64_t>(i) * w.d + e]);
-    Q[static_cast<int64_t>(jj) * w.d + e] = static_cast<float>(v * invd);
-  }
+  for (int64_t e = t0; e < w.d; e += stride)
+    Q[static_cast<int64_t>(jj) * w.d + e] =
+        sketch_column_entry(S[e], Q + e, w.d, jj, hs, hl, ctl->inv_hi, ctl->inv_lo);
 }
 
 // Basis update streamed through shared memory (FP32 or BF16 storage, FP32
@@ -494,51 +530,27 @@ __global__ void __launch_bounds__(UP_THREADS) k_update_ring(Work w0, StepOpts o0
     }
     return;
   }
-  // h_{i,j} as FP32 (hs) and, for the sketched column, as float-float
-  // hs + hl; 1/h_{j+1,j} likewise, computed once per CTA (an FP64 division
-  // in every thread would load the slow FP64 pipe).
+  // h_{i,j} as float-float pairs hs + hl and 1/h_{j+1,j} likewise, formed
+  // once by the step finish: FP64 conversions and divisions here cost every
+  // CTA some 3000 cycles before its first subtraction
   __shared__ float hs[kMaxK + 1];
   __shared__ float hl[kMaxK + 1];
-  __shared__ float rinv[2];
   __shared__ __align__(8) uint64_t full[UP_STAGES];
-  const int ld = w.m + 1;
   const bool qcta = static_cast<int>(blockIdx.x) >= nchunks;
-  for (int i = threadIdx.x; i < jj; i += blockDim.x) {
-    const double h = w.H[static_cast<int64_t>(ld) * (jj - 1) + i];
-    const float f = static_cast<float>(h);
-    hs[i] = f;
-    if (qcta) hl[i] = static_cast<float>(h - static_cast<double>(f));
+  // (thread 0 goes straight to the first copies)
+  for (int i = static_cast<int>(threadIdx.x) - 32; i < jj; i += blockDim.x - 32) {
+    if (i < 0) break;
+    const float2 h = static_cast<const float2*>(w.hf)[i];
+    hs[i] = h.x;
+    hl[i] = h.y;
   }
-  if (threadIdx.x == blockDim.x - 1) {
-    const double r = 1.0 / ctl->hnext;
-    const float f = static_cast<float>(r);
-    rinv[0] = f;
-    rinv[1] = static_cast<float>(r - static_cast<double>(f));
-  }
-  if (qcta) {   // Q_{j+1} = (S - sum_i h_i Q_i) / h_{j+1,j}, accumulated in float-float
+  if (qcta) {
     __syncthreads();
     float* Q = static_cast<float*>(w.Q);
-    const float* S = static_cast<const float*>(w.S);
     const int64_t e = static_cast<int64_t>(blockIdx.x - nchunks) * blockDim.x + threadIdx.x;
     if (e >= w.d) return;
-    FF v{S[e], 0.f};
-    auto sub = [&](int i, float q) {   // v -= (hs_i + hl_i) q
-      const FF p = ff_prod(hs[i], q);
-      v = ff_add(v, FF{-p.hi, -__fmaf_rn(hl[i], q, p.lo)});
-    };
-    int i = 0;
-    for (; i + 8 <= jj; i += 8) {   // eight loads in flight, then the chain in order
-      float q8[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) q8[u] = Q[static_cast<int64_t>(i + u) * w.d + e];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) sub(i + u, q8[u]);
-    }
-    for (; i < jj; ++i) sub(i, Q[static_cast<int64_t>(i) * w.d + e]);
-    // (v.hi + v.lo)(r0 + r1), rounded once to FP32
-    const FF p = ff_prod(v.hi, rinv[0]);
-    const float lo = __fmaf_rn(v.hi, rinv[1], __fmaf_rn(v.lo, rinv[0], p.lo));
-    Q[static_cast<int64_t>(jj) * w.d + e] = __fadd_rn(p.hi, lo);
+    Q[static_cast<int64_t>(jj) * w.d + e] = sketch_column_entry(static_cast<const float*>(w.S)[e], Q + e, w.d, jj, hs,
+                                                                hl, ctl->inv_hi, ctl->inv_lo);
     return;
   }
   extern __shared__ __align__(128) unsigned char smem[];
@@ -603,7 +615,7 @@ __global__ void __launch_bounds__(UP_THREADS) k_update_ring(Work w0, StepOpts o0
         mbar_wait(&full[u % UP_STAGES], static_cast<uint32_t>((u / UP_STAGES) & 1));
     return;
   }
-  const float fi = rinv[0];
+  const float fi = ctl->inv_hi;
   TV* out = static_cast<TV*>(w.V) + static_cast<int64_t>(jj) * n + c0;
 #pragma unroll
   for (int k = 0; k < NV; ++k) {

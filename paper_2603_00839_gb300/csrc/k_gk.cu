@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(GK_THREADS) k_gk_norm(Work w, int phase, StepO
   __shared__ int am_last;
   const T* S = static_cast<const T*>(w.S);
   const T* q = static_cast<const T*>(w.Q) + (phase == 3 ? w.d : 0);
-  const T c = static_cast<T>(gk_coef(w, phase));
+  const T c = coef_as<T>(gk_coef(w, phase));
   const int64_t d = w.d;
   DotAcc<T> a, b;
   const int64_t chunk = (d + gridDim.x - 1) / gridDim.x;
@@ -64,11 +64,10 @@ __global__ void __launch_bounds__(GK_THREADS) k_gk_norm(Work w, int phase, StepO
     red[warp][1] = tb;
   }
   __syncthreads();
-  const int rowlen = 2 * w.m + 4;
   if (threadIdx.x < 2)
-    w.part[static_cast<int64_t>(blockIdx.x) * rowlen + threadIdx.x] =
+    w.part[static_cast<int64_t>(threadIdx.x) * w.part_rows + blockIdx.x] =
         warps_total(red, blockDim.x >> 5, threadIdx.x);
-  if (!last_block_combine<false>(w, 2, tot, &am_last, &red[0][0])) return;
+  if (!last_block_combine<double>(w, 2, tot, &am_last, &red[0][0])) return;
   if (threadIdx.x != 0) return;
   const double nrm = sqrt(tot[0] > 0.0 ? tot[0] : 0.0);
   const double pre = sqrt(tot[1] > 0.0 ? tot[1] : 0.0);
@@ -88,7 +87,7 @@ __global__ void __launch_bounds__(GK_THREADS) k_gk_norm(Work w, int phase, StepO
       ctl->beta = ctl->beta0 = nrm;
       w.g[0] = nrm;
       ctl->rho = 1.0;
-      ctl->gk_scale = nrm;
+      set_inverse(ctl, nrm);
     }
     set_cond(o, !ctl->stop);
   } else if (phase == 1) {     // alpha_0
@@ -98,7 +97,7 @@ __global__ void __launch_bounds__(GK_THREADS) k_gk_norm(Work w, int phase, StepO
       ctl->stop = 1;
     } else {
       w.H[0] = nrm;
-      ctl->gk_scale = nrm;
+      set_inverse(ctl, nrm);
     }
     set_cond(o, !ctl->stop);
   } else if (phase == 2) {     // beta_{J+1}: column J of the bidiagonal is complete
@@ -111,7 +110,7 @@ __global__ void __launch_bounds__(GK_THREADS) k_gk_norm(Work w, int phase, StepO
     if (breakdown) ctl->breakdown = 1;
     ctl->pre2 = pre * pre;
     ctl->hnext = nrm;
-    ctl->gk_scale = nrm;
+    set_inverse(ctl, nrm);
     ctl->skip_update = breakdown ? 1 : 0;
     ctl->j = J + 1;
     ctl->givens = 1;
@@ -124,7 +123,7 @@ __global__ void __launch_bounds__(GK_THREADS) k_gk_norm(Work w, int phase, StepO
       set_cond(o, 0);
     } else {
       if (J + 1 < w.m) w.H[(J + 1) + static_cast<int64_t>(ld) * (J + 1)] = nrm;
-      ctl->gk_scale = nrm;
+      set_inverse(ctl, nrm);
     }
   }
 }
@@ -173,8 +172,8 @@ __global__ void k_gk_update(Work w, int phase, PtrRef srcr, StepOpts o) {
   double cprev = 0.0;
   if (phase == 2) cprev = w.H[(Jn - 1) + static_cast<int64_t>(ld) * (Jn - 1)];
   if (phase == 3) cprev = w.H[Jn + static_cast<int64_t>(ld) * (Jn - 1)];
-  const double inv = 1.0 / ctl->gk_scale;
-  const T ci = static_cast<T>(cprev), si = static_cast<T>(inv);
+  const double inv = ctl->inv;
+  const T ci = coef_as<T>(cprev), si = coef_as<T>(inv);
   const int64_t stride = static_cast<int64_t>(nblk) * blockDim.x;
   const int64_t t0 = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (sizeof(T) == 4 && (n % 4) == 0 && (reinterpret_cast<uintptr_t>(src) % 16) == 0) {

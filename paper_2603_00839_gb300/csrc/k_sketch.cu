@@ -791,7 +791,7 @@ k_sk_first_umma(PtrRef Xr, float* __restrict__ out, int64_t I, int64_t R, int64_
 // blocked input) during the contraction, then the reduction scratch of the
 // fused Gram-Schmidt pass (GS_MAXW rows of partial sums and the totals).
 template <int CH>
-constexpr size_t inner_smem() {
+__host__ __device__ constexpr size_t inner_smem() {
   constexpr size_t mma = size_t(CH) * N_NT * 32 * 8 + size_t(CH) * 16 * XA * 4;
   constexpr size_t red = size_t(GS_MAXW + 1) * kRedCols * 8;
   return mma > red ? mma : red;
@@ -902,15 +902,18 @@ k_sk_inner_tc(PtrRef Xr, int in_blocked, float* __restrict__ out, int64_t L, int
       for (int c = 0; c < 4; ++c) acc[nt][c] = fill;
   }
   __syncthreads();
-  float* red = reinterpret_cast<float*>(smem);               // [8][16][N_NT*8]
+  // the warps' partial tiles, [8][q][XA]: a row of 16 values of l and 4 pad, so
+  // that neither the fragments' stores nor the sums' loads meet in a bank
+  float* red = reinterpret_cast<float*>(smem);
   constexpr int TW = N_NT * 8;
+  static_assert(size_t(8) * TW * XA * 4 <= inner_smem<CH>(), "partial tiles fit the operands' space");
 #pragma unroll
   for (int nt = 0; nt < N_NT; ++nt)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int l = gid + h * 8, q = nt * 8 + tig * 2;
-      red[(warp * 16 + l) * TW + q] = acc[nt][2 * h];
-      red[(warp * 16 + l) * TW + q + 1] = acc[nt][2 * h + 1];
+      red[(warp * TW + q) * XA + l] = acc[nt][2 * h];
+      red[(warp * TW + q + 1) * XA + l] = acc[nt][2 * h + 1];
     }
   __syncthreads();
   constexpr int ITEMS = (16 * TW + TC_THREADS - 1) / TC_THREADS;
@@ -927,7 +930,7 @@ k_sk_inner_tc(PtrRef Xr, int in_blocked, float* __restrict__ out, int64_t L, int
     if (gl >= L || gq >= s) continue;
     float v = 0.f;
 #pragma unroll
-    for (int wv = 0; wv < 8; ++wv) v += red[(wv * 16 + l) * TW + q];
+    for (int wv = 0; wv < 8; ++wv) v += red[(wv * TW + q) * XA + l];
     v *= scale;
     const int64_t g = out_pos(om, gl, gq, r);
     out[g] = v;
@@ -939,15 +942,15 @@ k_sk_inner_tc(PtrRef Xr, int in_blocked, float* __restrict__ out, int64_t L, int
   // the reduction scratch reuses the dynamic shared memory
   __syncthreads();
   double(*red2)[kRedCols] = reinterpret_cast<double(*)[kRedCols]>(smem);
-  double* tot = reinterpret_cast<double*>(smem) + GS_MAXW * kRedCols;
+  FF* tot = reinterpret_cast<FF*>(smem) + GS_MAXW * kRedCols;
   block_partials<float, ITEMS>(w, vals, ix, ITEMS, J, red2);
   double* fin_sh = &red2[0][0];
   auto stage = [&]() { if (dots_pass > 0) gs_stage_gram_async(w, J, fin_sh); };
-  if (!last_block_combine<true>(w, gs_ncols(J), tot, &am_last, &red2[0][0], stage)) return;
+  if (!last_block_combine<float>(w, gs_ncols(J), tot, &am_last, fin_sh, stage)) return;
   if (dots_pass == 0) {
-    if (tid == 0) gs_finish_start(w, o, tot);
+    if (tid == 0) gs_finish_start<float>(w, o, tot);
   } else {
-    gs_finish_gram(w, o, tot, &red2[0][0], true);
+    gs_finish_gram_ff(w, o, J, tot, fin_sh, true);
   }
 }
 

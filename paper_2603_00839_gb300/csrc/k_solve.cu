@@ -244,7 +244,7 @@ __global__ void k_assemble(Work w0, PtrRef X0r0, PtrRef Xr0, const int* gate) {
   if (gate != nullptr && *gate) return;
   const int k = w.ctl->j;
   __shared__ T ys[kMaxK];
-  for (int i = threadIdx.x; i < k; i += blockDim.x) ys[i] = static_cast<T>(w.y[i]);
+  for (int i = threadIdx.x; i < k; i += blockDim.x) ys[i] = coef_as<T>(w.y[i]);
   __syncthreads();
   T* X = Xr.get<T>();
   const T* X0 = w.ctl->cycle > 0 ? X : X0r.get<const T>();
@@ -336,7 +336,7 @@ __global__ void k_assemble_bf16(Work w0, PtrRef X0r0, PtrRef Xr0, const int* gat
   if (gate != nullptr && *gate) return;
   const int k = w.ctl->j;
   __shared__ float ys[kMaxK];
-  for (int i = threadIdx.x; i < k; i += blockDim.x) ys[i] = static_cast<float>(w.y[i]);
+  for (int i = threadIdx.x; i < k; i += blockDim.x) ys[i] = coef_as<float>(w.y[i]);
   __syncthreads();
   float* X = Xr.get<float>();
   const float* X0 = w.ctl->cycle > 0 ? X : X0r.get<const float>();

@@ -395,6 +395,7 @@ size_t carve_work(void* mem, int dtype, int64_t n, const SketchPlan& sp, int m, 
   w.counter = c.take<unsigned>(8);
   w.ctl = c.take<Ctl>(1);
   w.H = c.take<double>(size_t(m + 1) * m);
+  w.hf = c.take<double>(size_t(m + 1));
   w.R = c.take<double>(size_t(m + 1) * m);
   w.cs = c.take<double>(m);
   w.sn = c.take<double>(m);
@@ -1193,6 +1194,8 @@ static rtg_status tune_update(SolvePlan& P, std::map<std::string, int>* cache, i
     Ctl c{};
     c.j = js[q];
     c.hnext = 1.0;
+    c.inv = 1.0;
+    c.inv_hi = 1.f;
     c.rs_skip = 1;
     for (int p = 0; p < w.b.n; ++p)
       CK(cudaMemcpyAsync(reinterpret_cast<char*>(w.ctl) + int64_t(p) * w.b.stride, &c, sizeof(Ctl),

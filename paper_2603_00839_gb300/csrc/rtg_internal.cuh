@@ -118,7 +118,8 @@ struct Ctl {
   double hnext;     // h_{j+1,j}
   double mu;        // chosen regularisation
   double gcv_best;
-  double gk_scale;  // Golub-Kahan: the norm the next update divides by
+  double inv;       // 1 / beta (start), 1 / h_{j+1,j} (FP64 step), 1 / gk_scale (Golub-Kahan)
+  float inv_hi, inv_lo;   // the same as a float-float pair (set for FP32 data)
   double true_rr;   // ||C - Phi(X)||_F / ||C||_F of the returned X (true-residual epilogue)
   double true_th;   // ||C - Phi(X)||_Theta / ||R_0||_Theta of the first cycle
 };
@@ -185,21 +186,22 @@ struct Work {
   void* tmp0;                  // sketch chain intermediates
   void* tmp1;
   void* Q;                     // (m+1) * d sketched basis
-  double* part;                // partial sums: blocks x (2m+4)
+  double* part;                // partial sums: (2m+4) columns of part_rows entries, one per block
   unsigned* counter;           // last-block counters (several)
   Ctl* ctl;
   double* H;                   // (m+1) x m Hessenberg, column-major
+  void* hf;                    // (m+1) float-float pairs: the newest Hessenberg column (FP32 data)
   double* R;                   // (m+1) x m rotated Hessenberg (upper triangular part)
   double* cs;                  // Givens cosines (m)
   double* sn;                  // Givens sines (m)
   double* g;                   // rotated right-hand side (m+1)
   double* G;                   // (m+1) x (m+1) Gram matrix of the stored sketched basis, leading
-                               // dimension gram_ld(m)
+                               // dimension gram_ld(m) (float-float pairs for FP32 data)
   double* rho_hist;            // (m) per cycle
   double* y;                   // solution coefficients (m)
   double* gcv;                 // GCV values (kMaxMu)
   double* ysel;                // per-mu coefficient candidates (kMaxMu * m)
-  int part_rows;               // rows available in part
+  int part_rows;               // entries of a column of part
   Batch b;                     // lock-step batch of identical workspaces
 #ifdef __CUDACC__
   // this workspace moved to the problem `off` bytes further
@@ -217,6 +219,7 @@ struct Work {
     r.counter = bsh(counter, off);
     r.ctl = bsh(ctl, off);
     r.H = bsh(H, off);
+    r.hf = bsh(hf, off);
     r.R = bsh(R, off);
     r.cs = bsh(cs, off);
     r.sn = bsh(sn, off);
