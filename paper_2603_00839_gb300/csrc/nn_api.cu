@@ -14,6 +14,7 @@
 // copy for the tensor-core products; accumulation is FP32.  The flat
 // parameter order is, per layer e1..e4, d3, d2, d1, out: weights
 // (c_out, 3, 3, c_in) then biases; then the head's weights and bias.
+#include <algorithm>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -94,10 +95,10 @@ struct rtg_warmstart {
   int adam_t = 0;
   // activations and their gradients, sized for the last (N, H, W)
   int N = 0, H = 0, W = 0;
-  Buf act, grad, col, dA, part, dzf, dzb, z, small;
-  float *x0, *e1, *e2, *e3, *e4, *u4, *r3, *d3, *u3, *r2, *d2, *u2, *r1, *d1, *zo, *g, *loglam;
-  float *gd1, *gu2, *gd2, *gu3, *gd3, *gu4, *ge4, *ge3, *ge2, *ge1, *gtmp, *dout, *dll;
-  double* loss;
+  Buf act, grad, slices, part, dzb, small;
+  float *x0, *e1, *e2, *e3, *e4, *r3, *d3, *r2, *d2, *r1, *d1, *zo, *g, *loglam;
+  float *gd1, *gd2, *gd3, *ge4, *ge3, *ge2, *ge1, *dout, *dll;
+  double* loss;      // the loss, then the loss kernels' scratch
 };
 
 namespace {
@@ -123,11 +124,10 @@ rtg_status shape_buffers(rtg_warmstart* ws, int N, int H, int W) {
   const int c = ws->base;
   const int64_t p1 = int64_t(N) * H * W, p2 = p1 / 4, p4 = p1 / 16, p8 = p1 / 64;
   // activation sizes in floats (order matters: pointers are carved in this order)
-  const int64_t sz[] = {p1 * 3, p1 * c, p2 * 2 * c, p4 * 4 * c, p8 * 4 * c, p4 * 4 * c, p4 * 4 * c, p4 * 4 * c,
-                        p2 * 4 * c, p2 * 2 * c, p2 * 2 * c, p1 * 2 * c, p1 * c, p1 * c, p1 * 3,
-                        int64_t(N) * 4 * c, int64_t(N)};
-  float** ptr[] = {&ws->x0, &ws->e1, &ws->e2, &ws->e3, &ws->e4, &ws->u4, &ws->r3, &ws->d3, &ws->u3, &ws->r2,
-                   &ws->d2, &ws->u2, &ws->r1, &ws->d1, &ws->zo, &ws->g, &ws->loglam};
+  const int64_t sz[] = {p1 * 3, p1 * c, p2 * 2 * c, p4 * 4 * c, p8 * 4 * c, p4 * 4 * c, p4 * 4 * c,
+                        p2 * 2 * c, p2 * 2 * c, p1 * c, p1 * c, p1 * 3, int64_t(N) * 4 * c, int64_t(N)};
+  float** ptr[] = {&ws->x0, &ws->e1, &ws->e2, &ws->e3, &ws->e4, &ws->r3, &ws->d3, &ws->r2,
+                   &ws->d2, &ws->r1, &ws->d1, &ws->zo, &ws->g, &ws->loglam};
   int64_t tot = 0;
   for (int64_t v : sz) tot += (v + 63) / 64 * 64;
   NRK(ws->act.ensure(size_t(tot) * 4));
@@ -136,10 +136,8 @@ rtg_status shape_buffers(rtg_warmstart* ws, int N, int H, int W) {
     *ptr[i] = ws->act.as<float>() + o;
     o += (sz[i] + 63) / 64 * 64;
   }
-  const int64_t gs[] = {p1 * c, p1 * 2 * c, p2 * 2 * c, p2 * 4 * c, p4 * 4 * c, p4 * 4 * c, p8 * 4 * c,
-                        p4 * 4 * c, p2 * 2 * c, p1 * c, p1 * 2 * c, p1 * 3, int64_t(N)};
-  float** gp[] = {&ws->gd1, &ws->gu2, &ws->gd2, &ws->gu3, &ws->gd3, &ws->gu4, &ws->ge4, &ws->ge3, &ws->ge2,
-                  &ws->ge1, &ws->gtmp, &ws->dout, &ws->dll};
+  const int64_t gs[] = {p1 * c, p2 * 2 * c, p4 * 4 * c, p8 * 4 * c, p4 * 4 * c, p2 * 2 * c, p1 * c, p1 * 3, int64_t(N)};
+  float** gp[] = {&ws->gd1, &ws->gd2, &ws->gd3, &ws->ge4, &ws->ge3, &ws->ge2, &ws->ge1, &ws->dout, &ws->dll};
   tot = 0;
   for (int64_t v : gs) tot += (v + 63) / 64 * 64;
   NRK(ws->grad.ensure(size_t(tot) * 4));
@@ -148,23 +146,19 @@ rtg_status shape_buffers(rtg_warmstart* ws, int N, int H, int W) {
     *gp[i] = ws->grad.as<float>() + o;
     o += (gs[i] + 63) / 64 * 64;
   }
-  // largest im2col (rows x 9 c_in) and GEMM output over the layers
-  int64_t mk = 0, mn = 0;
-  const int hs[NLAYER] = {H, H / 2, H / 4, H / 8, H / 4, H / 2, H, H};
-  const int wsz[NLAYER] = {W, W / 2, W / 4, W / 8, W / 4, W / 2, W, W};
+  // largest layer output, and the scratch of the layers that split K
+  int64_t mn = 0, sl = int64_t(N) * 32 * 4 * c;   // (the pooling partial sums)
+  const int hs[NLAYER] = {H, H, H / 2, H / 4, H / 4, H / 2, H, H};   // grid the layer reads
+  const int wsz[NLAYER] = {W, W, W / 2, W / 4, W / 4, W / 2, W, W};
   for (int l = 0; l < NLAYER; ++l) {
-    const int64_t M = int64_t(N) * hs[l] * wsz[l];
-    mk = std::max<int64_t>(mk, M * 9 * ws->L[l].cin);
-    mn = std::max<int64_t>(mn, M * ws->L[l].cout);
+    const Layer& L = ws->L[l];
+    mn = std::max<int64_t>(mn, int64_t(N) * (hs[l] / L.stride) * (wsz[l] / L.stride) * L.cout);
+    sl = std::max<int64_t>(sl, nn::conv_fwd_scratch(N, hs[l], wsz[l], L.cin, L.stride, L.cout));
   }
-  mk = std::max<int64_t>(mk, int64_t(N) * 32 * 4 * c);   // dA also holds the pooling partial sums
-  NRK(ws->col.ensure(size_t(mk) * 2));
-  NRK(ws->dA.ensure(size_t(mk) * 4));
-  NRK(ws->z.ensure(size_t(mn) * 4));
-  NRK(ws->dzf.ensure(size_t(mn) * 4));
+  NRK(ws->slices.ensure(size_t(sl) * 4));
   NRK(ws->dzb.ensure(size_t(mn) * 2));
   NRK(ws->part.ensure(size_t(64) * 4 * ws->base * 9 * 4 * ws->base * 4 + 1024));
-  NRK(ws->small.ensure(64));
+  NRK(ws->small.ensure(size_t(nn::loss_scratch_doubles(N) + 8) * sizeof(double)));
   ws->loss = ws->small.as<double>();
   ws->N = N;
   ws->H = H;
@@ -176,27 +170,20 @@ const float* Bf(const rtg_warmstart* ws, int l) { return ws->P.as<float>() + ws-
 const __nv_bfloat16* Wb(const rtg_warmstart* ws, int l) { return ws->Pb.as<__nv_bfloat16>() + ws->L[l].w; }
 
 // Backward of layer l: dy is the gradient of its output (after the ReLU when
-// mask != null); x its input (N, h, w, cin).  Writes the parameter gradients
-// and, if dx != null, the input gradient.
-rtg_status conv_bwd(rtg_warmstart* ws, int l, const float* x, int h, int w, const float* dy, const float* mask,
-                    float* dx, cudaStream_t s) {
+// mask != null); x its input on the h x w grid (up: stored at half resolution).
+// Writes the parameter gradients and, if dx != null, the input gradient
+// (plus addend, if given): on the stored grid of x.
+rtg_status conv_bwd(rtg_warmstart* ws, int l, const float* x, int h, int w, bool up, const float* dy,
+                    const float* mask, const float* addend, float* dx, cudaStream_t s) {
   const Layer& L = ws->L[l];
-  const int ho = h / L.stride, wo = w / L.stride;
-  const int M = ws->N * ho * wo, K = 9 * L.cin;
-  NCK(nn::mask_grad(dy, mask, ws->dzf.as<float>(), ws->dzb.as<__nv_bfloat16>(), int64_t(M) * L.cout, s));
+  const int64_t M = int64_t(ws->N) * (h / L.stride) * (w / L.stride);
   float* G = ws->G.as<float>();
-  NCK(nn::colsum(ws->dzf.as<float>(), G + L.b, M, L.cout, s));
-  NCK(nn::im2col(x, ws->col.as<__nv_bfloat16>(), ws->N, h, w, L.cin, L.stride, s));
-  int splits = M / 2048;
-  if (splits < 1) splits = 1;
-  if (splits > 64) splits = 64;
-  NCK(nn::gemm(true, false, ws->dzb.as<__nv_bfloat16>(), ws->col.as<__nv_bfloat16>(), G + L.w, nullptr, L.cout, K,
-               M, L.cout, K, splits, ws->part.as<float>(), s));
-  if (dx != nullptr) {
-    NCK(nn::gemm(false, false, ws->dzb.as<__nv_bfloat16>(), Wb(ws, l), ws->dA.as<float>(), nullptr, M, K, L.cout,
-                 L.cout, K, 1, nullptr, s));
-    NCK(nn::col2im(ws->dA.as<float>(), dx, ws->N, h, w, L.cin, L.stride, s));
-  }
+  __nv_bfloat16* dzb = ws->dzb.as<__nv_bfloat16>();
+  float* part = ws->part.as<float>();
+  NCK(nn::mask_grad(dy, mask, dzb, G + L.b, part, M, L.cout, s));
+  NCK(nn::conv_dw(x, dzb, G + L.w, ws->N, h, w, L.cin, L.stride, L.cout, up, part, int64_t(ws->part.bytes / 4), s));
+  if (dx != nullptr)
+    NCK(nn::conv_dx(dzb, Wb(ws, l), addend, dx, ws->N, h, w, L.cin, L.stride, L.cout, up, s));
   return RTG_OK;
 }
 
@@ -207,12 +194,13 @@ rtg_status layer_fwd(rtg_warmstart* ws, int l, const float* x, int h, int w, boo
                      float* out, cudaStream_t s) {
   const Layer& L = ws->L[l];
   NCK(nn::conv_fwd(x, Wb(ws, l), Bf(ws, l), r, skip, out, ws->N, h, w, L.cin, L.stride, L.cout, l != OUT, up,
-                   ws->dA.as<float>(), int64_t(ws->dA.bytes / 4), s));
+                   ws->slices.as<float>(), int64_t(ws->slices.bytes / 4), s));
   return RTG_OK;
 }
 
-// training: the up-sampled decoder inputs are materialised (the backward
-// pass reads them); inference reads them through the convolution's gather.
+// training: the activations before the skip sums are kept (the backward pass
+// takes its ReLU masks from them).  The up-sampled decoder inputs are read
+// through the convolutions' gather.
 rtg_status forward(rtg_warmstart* ws, const float* C, float* X0, float* loglam_out, bool training, cudaStream_t s) {
   const int N = ws->N, H = ws->H, W = ws->W, c = ws->base;
   NCK(nn::to_nhwc(C, ws->x0, N, H, W, 3, s));
@@ -220,53 +208,35 @@ rtg_status forward(rtg_warmstart* ws, const float* C, float* X0, float* loglam_o
   NRK(layer_fwd(ws, E2, ws->e1, H, W, false, nullptr, nullptr, ws->e2, s));
   NRK(layer_fwd(ws, E3, ws->e2, H / 2, W / 2, false, nullptr, nullptr, ws->e3, s));
   NRK(layer_fwd(ws, E4, ws->e3, H / 4, W / 4, false, nullptr, nullptr, ws->e4, s));
-  if (training) {
-    NCK(nn::up2(ws->e4, ws->u4, N, H / 8, W / 8, 4 * c, s));
-    NRK(layer_fwd(ws, D3, ws->u4, H / 4, W / 4, false, ws->r3, ws->e3, ws->d3, s));
-    NCK(nn::up2(ws->d3, ws->u3, N, H / 4, W / 4, 4 * c, s));
-    NRK(layer_fwd(ws, D2, ws->u3, H / 2, W / 2, false, ws->r2, ws->e2, ws->d2, s));
-    NCK(nn::up2(ws->d2, ws->u2, N, H / 2, W / 2, 2 * c, s));
-    NRK(layer_fwd(ws, D1, ws->u2, H, W, false, ws->r1, ws->e1, ws->d1, s));
-  } else {
-    NRK(layer_fwd(ws, D3, ws->e4, H / 4, W / 4, true, nullptr, ws->e3, ws->d3, s));
-    NRK(layer_fwd(ws, D2, ws->d3, H / 2, W / 2, true, nullptr, ws->e2, ws->d2, s));
-    NRK(layer_fwd(ws, D1, ws->d2, H, W, true, nullptr, ws->e1, ws->d1, s));
-  }
+  NRK(layer_fwd(ws, D3, ws->e4, H / 4, W / 4, true, training ? ws->r3 : nullptr, ws->e3, ws->d3, s));
+  NRK(layer_fwd(ws, D2, ws->d3, H / 2, W / 2, true, training ? ws->r2 : nullptr, ws->e2, ws->d2, s));
+  NRK(layer_fwd(ws, D1, ws->d2, H, W, true, training ? ws->r1 : nullptr, ws->e1, ws->d1, s));
   NRK(layer_fwd(ws, OUT, ws->d1, H, W, false, nullptr, nullptr, ws->zo, s));
   NCK(nn::from_nhwc_add(ws->zo, C, X0, N, H, W, 3, s));
   const float* Pf = ws->P.as<float>();
-  NCK(nn::pool_head(ws->e4, Pf + ws->head_w, Pf + ws->head_b, ws->g, loglam_out, ws->dA.as<float>(), N,
+  NCK(nn::pool_head(ws->e4, Pf + ws->head_w, Pf + ws->head_b, ws->g, loglam_out, ws->slices.as<float>(), N,
                     (H / 8) * (W / 8), 4 * c, s));
   return RTG_OK;
 }
 
 rtg_status backward(rtg_warmstart* ws, cudaStream_t s) {
   const int N = ws->N, H = ws->H, W = ws->W, c = ws->base;
-  const int64_t p1 = int64_t(N) * H * W, p2 = p1 / 4, p4 = p1 / 16;
   float* G = ws->G.as<float>();
   // out (no ReLU): input d1
-  NRK(conv_bwd(ws, OUT, ws->d1, H, W, ws->dout, nullptr, ws->gd1, s));
-  // d1 = relu(conv(u2)) + e1
-  NRK(conv_bwd(ws, D1, ws->u2, H, W, ws->gd1, ws->r1, ws->gu2, s));
-  NCK(nn::up2_back(ws->gu2, ws->gd2, N, H / 2, W / 2, 2 * c, false, s));
-  // d2 = relu(conv(u3)) + e2
-  NRK(conv_bwd(ws, D2, ws->u3, H / 2, W / 2, ws->gd2, ws->r2, ws->gu3, s));
-  NCK(nn::up2_back(ws->gu3, ws->gd3, N, H / 4, W / 4, 4 * c, false, s));
-  // d3 = relu(conv(u4)) + e3
-  NRK(conv_bwd(ws, D3, ws->u4, H / 4, W / 4, ws->gd3, ws->r3, ws->gu4, s));
-  NCK(nn::up2_back(ws->gu4, ws->ge4, N, H / 8, W / 8, 4 * c, false, s));
+  NRK(conv_bwd(ws, OUT, ws->d1, H, W, false, ws->dout, nullptr, nullptr, ws->gd1, s));
+  // d_k = relu(conv(up(.))) + e_k: the input gradients are summed over the up-sampling's 2 x 2 blocks
+  NRK(conv_bwd(ws, D1, ws->d2, H, W, true, ws->gd1, ws->r1, nullptr, ws->gd2, s));
+  NRK(conv_bwd(ws, D2, ws->d3, H / 2, W / 2, true, ws->gd2, ws->r2, nullptr, ws->gd3, s));
+  NRK(conv_bwd(ws, D3, ws->e4, H / 4, W / 4, true, ws->gd3, ws->r3, nullptr, ws->ge4, s));
   // lambda head
   const float* Pf = ws->P.as<float>();
   NCK(nn::head_back(ws->g, ws->dll, Pf + ws->head_w, G + ws->head_w, G + ws->head_b, ws->ge4, N,
                     (H / 8) * (W / 8), 4 * c, s));
   // encoder: each e_k feeds the next level and a skip sum
-  NRK(conv_bwd(ws, E4, ws->e3, H / 4, W / 4, ws->ge4, ws->e4, ws->gtmp, s));
-  NCK(nn::add(ws->gd3, ws->gtmp, ws->ge3, p4 * 4 * c, s));
-  NRK(conv_bwd(ws, E3, ws->e2, H / 2, W / 2, ws->ge3, ws->e3, ws->gtmp, s));
-  NCK(nn::add(ws->gd2, ws->gtmp, ws->ge2, p2 * 2 * c, s));
-  NRK(conv_bwd(ws, E2, ws->e1, H, W, ws->ge2, ws->e2, ws->gtmp, s));
-  NCK(nn::add(ws->gd1, ws->gtmp, ws->ge1, p1 * c, s));
-  NRK(conv_bwd(ws, E1, ws->x0, H, W, ws->ge1, ws->e1, nullptr, s));
+  NRK(conv_bwd(ws, E4, ws->e3, H / 4, W / 4, false, ws->ge4, ws->e4, ws->gd3, ws->ge3, s));
+  NRK(conv_bwd(ws, E3, ws->e2, H / 2, W / 2, false, ws->ge3, ws->e3, ws->gd2, ws->ge2, s));
+  NRK(conv_bwd(ws, E2, ws->e1, H, W, false, ws->ge2, ws->e2, ws->gd1, ws->ge1, s));
+  NRK(conv_bwd(ws, E1, ws->x0, H, W, false, ws->ge1, ws->e1, nullptr, nullptr, s));
   return RTG_OK;
 }
 
@@ -360,7 +330,8 @@ rtg_status rtg_ws_train_step(rtg_ws ws, int32_t n_img, int32_t I1, int32_t I2, c
     return nfail(RTG_ERR_INVALID_ARG, "NULL argument");
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   NRK(forward(ws, C, X0_scratch, ws->loglam, true, s));
-  NCK(nn::loss(X0_scratch, Xstar, ws->loglam, logmu, ws->dout, ws->dll, ws->loss, ws->N, ws->H, ws->W, 3, s));
+  NCK(nn::loss(X0_scratch, Xstar, ws->loglam, logmu, ws->dout, ws->dll, ws->loss, ws->loss + 8, ws->N, ws->H,
+               ws->W, 3, s));
   NRK(backward(ws, s));
   if (lr > 0.f) {
     ws->adam_t += 1;
@@ -385,34 +356,24 @@ rtg_status rtg_nn_conv3x3(int32_t device, int32_t N, int32_t H, int32_t W, int32
   if (dy == nullptr && y == nullptr) return nfail(RTG_ERR_INVALID_ARG, "give y (forward) or dy (backward)");
   DevGuard dg(device);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  const int ho = H / stride, wo = W / stride;
-  const int M = N * ho * wo, K = 9 * cin;
-  Buf wb, col, zf, zb, dA, part;
+  const int64_t M = int64_t(N) * (H / stride) * (W / stride);
+  const int K = 9 * cin;
+  Buf wb, zb, part;
   NRK(wb.ensure(size_t(cout) * K * 2));
-  NRK(col.ensure(size_t(M) * K * 2));
   NCK(nn::to_bf16(w, wb.as<__nv_bfloat16>(), int64_t(cout) * K, s));
-  NCK(nn::im2col(x, col.as<__nv_bfloat16>(), N, H, W, cin, stride, s));
   if (y != nullptr)
     NCK(nn::conv_fwd(x, wb.as<__nv_bfloat16>(), b, nullptr, nullptr, y, N, H, W, cin, stride, cout, false, false,
                      nullptr, 0, s));
   if (dy != nullptr) {
-    NRK(zf.ensure(size_t(M) * cout * 4));
+    const int64_t splits = nn::conv_dw_splits(N, H, W, cin, stride, cout, int64_t(1) << 62);
+    const int64_t pf = std::max<int64_t>(int64_t(nn::mask_grad_blocks(M)) * cout, splits * cout * K);
     NRK(zb.ensure(size_t(M) * cout * 2));
-    NCK(nn::mask_grad(dy, nullptr, zf.as<float>(), zb.as<__nv_bfloat16>(), int64_t(M) * cout, s));
-    if (db != nullptr) NCK(nn::colsum(zf.as<float>(), db, M, cout, s));
-    if (dw != nullptr) {
-      int splits = M / 2048;
-      splits = splits < 1 ? 1 : (splits > 64 ? 64 : splits);
-      NRK(part.ensure(size_t(splits) * cout * K * 4 + 64));
-      NCK(nn::gemm(true, false, zb.as<__nv_bfloat16>(), col.as<__nv_bfloat16>(), dw, nullptr, cout, K, M, cout, K,
-                   splits, part.as<float>(), s));
-    }
-    if (dx != nullptr) {
-      NRK(dA.ensure(size_t(M) * K * 4));
-      NCK(nn::gemm(false, false, zb.as<__nv_bfloat16>(), wb.as<__nv_bfloat16>(), dA.as<float>(), nullptr, M, K,
-                   cout, cout, K, 1, nullptr, s));
-      NCK(nn::col2im(dA.as<float>(), dx, N, H, W, cin, stride, s));
-    }
+    NRK(part.ensure(size_t(pf) * 4 + 64));
+    NCK(nn::mask_grad(dy, nullptr, zb.as<__nv_bfloat16>(), db, part.as<float>(), M, cout, s));
+    if (dw != nullptr)
+      NCK(nn::conv_dw(x, zb.as<__nv_bfloat16>(), dw, N, H, W, cin, stride, cout, false, part.as<float>(), pf, s));
+    if (dx != nullptr)
+      NCK(nn::conv_dx(zb.as<__nv_bfloat16>(), wb.as<__nv_bfloat16>(), nullptr, dx, N, H, W, cin, stride, cout, false, s));
   }
   NCK(cudaStreamSynchronize(s));
   return RTG_OK;

@@ -8,19 +8,21 @@
 namespace rtg {
 namespace nn {
 
-// C = op(A) op(B) (+ bias), BF16 operands, FP32 result; a_cm: A stored
-// transposed; b_t: B stored N x K.  splits > 1 splits K (part: splits*M*N floats).
-cudaError_t gemm(bool a_cm, bool b_t, const __nv_bfloat16* A, const __nv_bfloat16* B, float* C,
-                 const float* bias, int M, int N, int K, int lda, int ldb, int splits, float* part,
-                 cudaStream_t s);
-cudaError_t im2col(const float* x, __nv_bfloat16* A, int N, int H, int W, int C, int stride, cudaStream_t s);
-cudaError_t col2im(const float* dA, float* dx, int N, int H, int W, int C, int stride, cudaStream_t s);
-cudaError_t relu_skip(const float* z, float* r, const float* skip, float* out, int64_t n, cudaStream_t s);
-cudaError_t mask_grad(const float* dy, const float* mask, float* dz, __nv_bfloat16* dzb, int64_t n, cudaStream_t s);
-cudaError_t colsum(const float* dz, float* db, int64_t rows, int cols, cudaStream_t s);
-cudaError_t up2(const float* x, float* y, int N, int H, int W, int C, cudaStream_t s);
-cudaError_t up2_back(const float* dy, float* dx, int N, int H, int W, int C, bool acc, cudaStream_t s);
-cudaError_t add(const float* a, const float* b, float* out, int64_t n, cudaStream_t s);
+// dz = dy * (mask > 0) (mask null: dz = dy) in BF16, db[c] = its FP32 column
+// sums over the rows (db null: none; part: mask_grad_blocks(rows) * cols floats).
+cudaError_t mask_grad(const float* dy, const float* mask, __nv_bfloat16* dzb, float* db, float* part, int64_t rows,
+                      int cols, cudaStream_t s);
+int mask_grad_blocks(int64_t rows);
+// Gradients of a 3x3 convolution on an H x W grid (padding 1).  Weights: dw
+// (cout, 3, 3, C); x as for conv_fwd (up: stored at half resolution); part:
+// conv_dw_splits(..., part_floats) * cout * 9 C floats when that is over 1.
+// Data: dx (N, H, W, C) = addend + gradient (addend may be null); up2: the 2 x 2
+// block sums of the gradient instead, (N, H / 2, W / 2, C).
+int conv_dw_splits(int N, int H, int W, int C, int stride, int cout, int64_t part_floats);
+cudaError_t conv_dw(const float* x, const __nv_bfloat16* dzb, float* dw, int N, int H, int W, int C, int stride,
+                    int cout, bool up, float* part, int64_t part_floats, cudaStream_t s);
+cudaError_t conv_dx(const __nv_bfloat16* dzb, const __nv_bfloat16* w, const float* addend, float* dx, int N, int H,
+                    int W, int C, int stride, int cout, bool up2, cudaStream_t s);
 cudaError_t to_nhwc(const float* src, float* dst, int N, int H, int W, int C, cudaStream_t s);
 cudaError_t from_nhwc_add(const float* src, const float* base, float* dst, int N, int H, int W, int C,
                           cudaStream_t s);
@@ -35,8 +37,12 @@ cudaError_t pool_head(const float* e, const float* w, const float* b, float* g, 
 cudaError_t conv_fwd(const float* x, const __nv_bfloat16* w, const float* bias, float* r, const float* skip,
                      float* out, int N, int H, int W, int C, int stride, int cout, bool relu, bool up,
                      float* part, int64_t part_floats, cudaStream_t s);
+// floats of scratch that lets conv_fwd split K as far as it would
+int64_t conv_fwd_scratch(int N, int H, int W, int C, int stride, int cout);
+// scratch: loss_scratch_doubles(N)
 cudaError_t loss(const float* X0, const float* Xs, const float* loglam, const float* logmu, float* dout,
-                 float* dloglam, double* out, int N, int H, int W, int C, cudaStream_t s);
+                 float* dloglam, double* out, double* scratch, int N, int H, int W, int C, cudaStream_t s);
+int64_t loss_scratch_doubles(int N);
 cudaError_t head_back(const float* g, const float* dll, const float* w, float* dw, float* db, float* de, int N,
                       int HW, int C, cudaStream_t s);
 cudaError_t adam(float* p, const float* g, float* m, float* v, __nv_bfloat16* pb, int64_t n, float lr, float b1,

@@ -60,3 +60,41 @@ def test_first_stage_does_not_depend_on_the_grouping(api, h):
         part = h.sketch(X[:, c:c + 1000], (24, 1000), 5)
         torch.cuda.synchronize()
         assert torch.equal(part, whole[:, c:c + 1000])
+
+
+# ------------------------------------------------------------------------ convolution gradients
+
+def _bf16_exact(shape, seed):
+    g = torch.Generator("cuda").manual_seed(seed)
+    return torch.randn(shape, device="cuda", generator=g).to(torch.bfloat16).float()
+
+
+@pytest.mark.parametrize("N,H,W,cin,cout,stride", [
+    (1, 1, 1, 1, 1, 1),          # one pixel
+    (2, 9, 17, 3, 33, 1),        # ragged tiles, three channels, two tiles of output channels
+    (1, 16, 34, 24, 64, 2),      # parity classes with ragged tiles
+    (1, 10, 18, 130, 129, 1),    # channels past 128 on both sides: two chunks of K
+    (2, 6, 6, 64, 200, 2),
+    (1, 40, 40, 32, 3, 1),       # the output layer's shape, several slices of pixels
+])
+def test_convolution_gradients(api, N, H, W, cin, cout, stride):
+    x, wt = _bf16_exact((N, H, W, cin), 1), _bf16_exact((cout, 3, 3, cin), 2)
+    dy = _bf16_exact((N, H // stride, W // stride, cout), 3)
+    dx, dw, db = api.conv3x3(x, wt, None, stride=stride, dy=dy)
+    xr = x.double().permute(0, 3, 1, 2).requires_grad_(True)
+    wr = wt.double().permute(0, 3, 1, 2).requires_grad_(True)
+    y = torch.nn.functional.conv2d(xr, wr, stride=stride, padding=1)
+    gx, gw = torch.autograd.grad(y, (xr, wr), dy.double().permute(0, 3, 1, 2))
+    # operands are exact in BF16, so only FP32 sums of at most 9 * 200 (data) or 1600 (weights) products differ
+    for got, ref in ((dx, gx.permute(0, 2, 3, 1)), (dw, gw.permute(0, 2, 3, 1)), (db, dy.double().sum(dim=(0, 1, 2)))):
+        assert float((got.double() - ref).norm()) <= 5e-6 * float(ref.norm()) + 1e-12
+
+
+def test_convolution_gradients_of_unaligned_input(api):
+    """x on no 16-byte boundary takes the scalar gather: the same bits as the aligned copy."""
+    buf = _bf16_exact((1 * 12 * 20 * 16 + 1,), 4)
+    x = buf[1:].view(1, 12, 20, 16)
+    wt, dy = _bf16_exact((8, 3, 3, 16), 5), _bf16_exact((1, 12, 20, 8), 6)
+    a = api.conv3x3(x, wt, None, dy=dy)
+    b = api.conv3x3(x.clone(), wt, None, dy=dy)
+    assert all(torch.equal(p, q) for p, q in zip(a, b))
