@@ -57,7 +57,7 @@ k_conv_fwd(const float* __restrict__ x, const __nv_bfloat16* __restrict__ wt, co
   const int Hs = up ? H / 2 : H, Ws = up ? W / 2 : W, sh = up ? 1 : 0;   // stored input grid
   const int m0 = blockIdx.x * CBM, n0 = blockIdx.y * BN;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, gid = lane >> 2, tig = lane & 3;
-  const bool fastA = (C % 32) == 0;
+  const bool fastA = (C % 32) == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
   const bool fastB = (Kfull % 8) == 0;
   float4 ra[4];
   float rs[16];
@@ -243,10 +243,16 @@ int64_t conv_fwd_scratch(int N, int H, int W, int C, int stride, int cout) {
 
 cudaError_t conv_fwd(const float* x, const __nv_bfloat16* w, const float* bias, float* r, const float* skip,
                      float* out, int N, int H, int W, int C, int stride, int cout, bool relu, bool up,
-                     float* part, int64_t part_floats, cudaStream_t s) {
+                     float* part, int64_t part_floats, cudaStream_t s, bool planar_in, const float* planar_add) {
   const int M = N * (H / stride) * (W / stride);
   const FwdSplit f = fwd_split(N, H, W, C, stride, cout, part != nullptr, part_floats);
   const int bn = f.bn, mtiles = f.mtiles, ntiles = f.ntiles, splits = f.splits, kchunk = f.kchunk;
+  // the tile kernels read an input tile once for all taps; they cut K where the
+  // slices would, so the choice does not change the result
+  if (const int kind = conv_tile_kind(x, w, H, W, C, stride, bn, up))
+    return conv_tile(kind, x, w, bias, r, skip, out, planar_add, planar_in, N, H, W, C, stride, cout, relu, up, bn,
+                     kchunk, s);
+  if (planar_in || planar_add != nullptr) return cudaErrorInvalidValue;
   dim3 grid(mtiles, ntiles, splits);
   const int rl = relu ? 1 : 0, u = up ? 1 : 0;
 #define RTG_CONV_CASE(B_)                                                                                   \
@@ -263,15 +269,11 @@ cudaError_t conv_fwd(const float* x, const __nv_bfloat16* w, const float* bias, 
 
 // ------------------------------------------------------------------ elementwise
 // solver layout (per image x fastest, then y, then channel) <-> channels last
-__global__ void k_to_nhwc(const float* __restrict__ src, float* __restrict__ dst, int N, int H, int W, int C) {
-  const int64_t total = static_cast<int64_t>(N) * H * W * C;
-  for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < total;
-       e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int x = static_cast<int>(e % W);
-    const int y = static_cast<int>((e / W) % H);
-    const int c = static_cast<int>((e / (static_cast<int64_t>(W) * H)) % C);
-    const int n = static_cast<int>(e / (static_cast<int64_t>(W) * H * C));
-    dst[((static_cast<int64_t>(n) * H + y) * W + x) * C + c] = src[e];
+__global__ void k_to_nhwc(const float* __restrict__ src, float* __restrict__ dst, int64_t pixels, int HW, int C) {
+  for (int64_t p = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; p < pixels;
+       p += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+    const int64_t n = p / HW;
+    for (int c = 0; c < C; ++c) dst[p * C + c] = src[(n * (C - 1) + c) * HW + p];   // image n starts at n C HW
   }
 }
 
@@ -300,6 +302,7 @@ __global__ void k_pool_part(const float* __restrict__ e, float* __restrict__ par
   const int p1 = static_cast<int>((static_cast<int64_t>(HW) * (b + 1)) / POOL_SLICES);
   for (int c = threadIdx.x; c < C; c += blockDim.x) {
     float v = 0.f;
+#pragma unroll 16
     for (int p = p0; p < p1; ++p) v += e[(static_cast<int64_t>(n) * HW + p) * C + c];
     part[(static_cast<int64_t>(n) * POOL_SLICES + b) * C + c] = v;
   }
@@ -383,7 +386,7 @@ __global__ void k_to_bf16(const float* __restrict__ x, __nv_bfloat16* __restrict
   } while (0)
 
 cudaError_t to_nhwc(const float* src, float* dst, int N, int H, int W, int C, cudaStream_t s) {
-  NN_EW(k_to_nhwc, int64_t(N) * H * W * C, src, dst, N, H, W, C);
+  NN_EW(k_to_nhwc, int64_t(N) * H * W, src, dst, int64_t(N) * H * W, H * W, C);
 }
 cudaError_t from_nhwc_add(const float* src, const float* base, float* dst, int N, int H, int W, int C,
                           cudaStream_t s) {

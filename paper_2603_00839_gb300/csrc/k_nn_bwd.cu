@@ -11,133 +11,105 @@
 #include <cuda_bf16.h>
 
 #include "nn_internal.cuh"
+#include "nn_mma.cuh"
 #include "rtg_internal.cuh"
 
 namespace rtg {
 namespace nn {
 
-__device__ __forceinline__ uint32_t smem_addr(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-__device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], uint32_t a) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];\n"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(a)
-               : "memory");
-}
-__device__ __forceinline__ void ldsm_x4_t(uint32_t (&r)[4], uint32_t a) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];\n"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(a)
-               : "memory");
-}
-__device__ __forceinline__ void mma_k16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-      "{%0,%1,%2,%3};\n"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-  return *reinterpret_cast<const uint32_t*>(&h);
-}
-
 // ------------------------------------------------------------------ output gradient
-// dzb = bf16(dz), dz = dy * (mask > 0) (mask null: dz = dy), and this block's
-// column sums of dz into part[block][cols] (part null: none).  A block takes
-// `rows_per` rows; consecutive threads take V consecutive columns each, so the
-// loads are whole lines and each thread's sums stay in its own columns.
-// blockIdx.y: column chunk of `cw` columns.
-template <int V>
+// dzb = bf16(dz), dz = dy * (mask > 0) (mask null: dz = dy), and with `part`
+// the column sums of dz: block t takes the rows t, t + 256, ..., all threads
+// load (U rows of a column each, in flight together) and one thread per column
+// adds them in row order; part[t][cols], then k_colsum_tree.  The order is kept
+// whatever the parallelism: Adam divides by the gradients' size, so a change
+// of rounding in an entry near zero would change its first step's sign.
+// blockIdx.y: column chunk of `cw` <= 256 columns.
+constexpr int MG_U = 8;
 __global__ void __launch_bounds__(256)
 k_mask_grad_db(const float* __restrict__ dy, const float* __restrict__ mask, __nv_bfloat16* __restrict__ dzb,
-               float* __restrict__ part, int64_t rows, int cols, int cw, int64_t rows_per) {
-  __shared__ float red[256 * V];
-  const int c0 = blockIdx.y * cw;
-  const int width = min(cw, cols - c0), tpr = width / V, rpb = 256 / tpr;
-  const int rr = threadIdx.x / tpr, col = c0 + (threadIdx.x % tpr) * V;
-  const int64_t r0 = blockIdx.x * rows_per, r1 = min(rows, r0 + rows_per);
-  float sum[V];
+               float* __restrict__ part, int64_t rows, int cols, int cw) {
+  __shared__ float sh[MG_U * 256];
+  const int c0 = blockIdx.y * cw, width = min(cw, cols - c0);
+  const int lpc = 256 / width;                       // rows loaded side by side
+  const int kk = threadIdx.x / width, col = c0 + threadIdx.x % width;
+  const int64_t nk = blockIdx.x < rows ? (rows - blockIdx.x + 255) / 256 : 0;   // this block's rows
+  float sum = 0.f;
+  for (int64_t k0 = 0; k0 < nk; k0 += MG_U * lpc) {
+    float g[MG_U], m[MG_U];
 #pragma unroll
-  for (int v = 0; v < V; ++v) sum[v] = 0.f;
-  if (rr < rpb)
-    for (int64_t r = r0 + rr; r < r1; r += rpb) {
-      const int64_t at = r * cols + col;
-      float g[V], m[V];
-      if constexpr (V == 4) {
-        const float4 q = *reinterpret_cast<const float4*>(dy + at);
-        g[0] = q.x; g[1] = q.y; g[2] = q.z; g[3] = q.w;
-        if (mask != nullptr) {
-          const float4 k = *reinterpret_cast<const float4*>(mask + at);
-          m[0] = k.x; m[1] = k.y; m[2] = k.z; m[3] = k.w;
-        }
-      } else {
-        g[0] = dy[at];
-        if (mask != nullptr) m[0] = mask[at];
-      }
-#pragma unroll
-      for (int v = 0; v < V; ++v) {
-        if (mask != nullptr && !(m[v] > 0.f)) g[v] = 0.f;
-        sum[v] += g[v];
-      }
-      if constexpr (V == 4) {
-        *reinterpret_cast<uint2*>(dzb + at) = make_uint2(pack_bf16(g[0], g[1]), pack_bf16(g[2], g[3]));
-      } else {
-        dzb[at] = __float2bfloat16(g[0]);
+    for (int u = 0; u < MG_U; ++u) {
+      const int64_t k = k0 + u * lpc + kk;
+      g[u] = 0.f;
+      m[u] = 1.f;
+      if (kk < lpc && k < nk) {
+        const int64_t at = (blockIdx.x + 256 * k) * cols + col;
+        g[u] = dy[at];
+        if (mask != nullptr) m[u] = mask[at];
       }
     }
-  if (part == nullptr) return;
 #pragma unroll
-  for (int v = 0; v < V; ++v) red[rr < rpb ? (rr * tpr + threadIdx.x % tpr) * V + v : 256 * V - 1] = sum[v];
-  __syncthreads();
-  for (int c = threadIdx.x; c < width; c += 256) {
-    float s = 0.f;
-    for (int q = 0; q < rpb; ++q) s += red[q * width + c];
-    part[static_cast<int64_t>(blockIdx.x) * cols + c0 + c] = s;
+    for (int u = 0; u < MG_U; ++u) {
+      const int64_t k = k0 + u * lpc + kk;
+      if (!(m[u] > 0.f)) g[u] = 0.f;
+      if (kk < lpc && k < nk) dzb[(blockIdx.x + 256 * k) * cols + col] = __float2bfloat16(g[u]);
+      if (kk < lpc) sh[(u * lpc + kk) * width + threadIdx.x % width] = g[u];
+    }
+    if (part == nullptr) continue;
+    __syncthreads();
+    if (threadIdx.x < width) {
+      const int64_t left = nk - k0;
+      const int cnt = static_cast<int>(left < MG_U * lpc ? left : MG_U * lpc);
+#pragma unroll 16
+      for (int q = 0; q < cnt; ++q) sum += sh[q * width + threadIdx.x];
+    }
+    __syncthreads();
   }
+  if (part != nullptr && threadIdx.x < width) part[static_cast<int64_t>(blockIdx.x) * cols + c0 + threadIdx.x] = sum;
 }
 
-// out[i] = sum over z < nz of part[z * len + i], fixed order: 64 entries and
-// four interleaved groups of slices per block.
-__global__ void __launch_bounds__(256)
-k_sum_parts(const float* __restrict__ part, float* __restrict__ out, int64_t len, int nz) {
-  __shared__ float red[4][64];
-  const int e = threadIdx.x & 63, g = threadIdx.x >> 6;
-  const int64_t i = static_cast<int64_t>(blockIdx.x) * 64 + e;
-  float v = 0.f;
-  if (i < len) {
-#pragma unroll 8
-    for (int z = g; z < nz; z += 4) v += part[static_cast<int64_t>(z) * len + i];
-  }
-  red[g][e] = v;
+// db[c] = tree over the 256 partial sums of column c.
+__global__ void __launch_bounds__(256) k_colsum_tree(const float* __restrict__ part, float* __restrict__ db, int cols) {
+  __shared__ float red[256];
+  red[threadIdx.x] = part[static_cast<int64_t>(threadIdx.x) * cols + blockIdx.x];
   __syncthreads();
-  if (g == 0 && i < len) out[i] = (red[0][e] + red[1][e]) + (red[2][e] + red[3][e]);
+  for (int o = 128; o > 0; o >>= 1) {
+    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) db[blockIdx.x] = red[0];
+}
+
+// out[i] = sum over z < nz of part[z * len + i], in order (as above): up to 16
+// loads in flight per thread.
+__global__ void __launch_bounds__(128)
+k_sum_slices(const float* __restrict__ part, float* __restrict__ out, int64_t len, int nz) {
+  const int64_t i = static_cast<int64_t>(blockIdx.x) * 128 + threadIdx.x;
+  if (i >= len) return;
+  float v = 0.f;
+  int z = 0;
+  for (; z + 16 <= nz; z += 16) {
+    float t[16];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) t[u] = part[static_cast<int64_t>(z + u) * len + i];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) v += t[u];
+  }
+#pragma unroll 4
+  for (; z < nz; ++z) v += part[static_cast<int64_t>(z) * len + i];
+  out[i] = v;
 }
 
 static bool aligned16(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }
 
-int mask_grad_blocks(int64_t rows) {
-  int64_t b = (rows + 63) / 64;
-  return static_cast<int>(b > 456 ? 456 : (b < 1 ? 1 : b));
-}
-
 cudaError_t mask_grad(const float* dy, const float* mask, __nv_bfloat16* dzb, float* db, float* part, int64_t rows,
                       int cols, cudaStream_t s) {
-  const int nb = mask_grad_blocks(rows);
-  const int64_t rows_per = (rows + nb - 1) / nb;
   float* pt = db != nullptr ? part : nullptr;
-  // four columns per thread where 16-byte accesses fit
-  if (cols % 4 == 0 && aligned16(dy) && (mask == nullptr || aligned16(mask)) && aligned16(dzb)) {
-    const int cw = cols < 1024 ? cols : 1024;
-    k_mask_grad_db<4><<<dim3(nb, (cols + cw - 1) / cw), 256, 0, s>>>(dy, mask, dzb, pt, rows, cols, cw, rows_per);
-  } else {
-    const int cw = cols < 255 ? cols : 255;
-    k_mask_grad_db<1><<<dim3(nb, (cols + cw - 1) / cw), 256, 0, s>>>(dy, mask, dzb, pt, rows, cols, cw, rows_per);
-  }
+  const int cw = cols < 256 ? cols : 256;
+  k_mask_grad_db<<<dim3(256, (cols + cw - 1) / cw), 256, 0, s>>>(dy, mask, dzb, pt, rows, cols, cw);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || pt == nullptr) return e;
-  k_sum_parts<<<(cols + 63) / 64, 256, 0, s>>>(part, db, cols, nb);
+  k_colsum_tree<<<cols, 256, 0, s>>>(part, db, cols);
   return cudaGetLastError();
 }
 
@@ -279,35 +251,33 @@ k_conv_dw(const float* __restrict__ x, const __nv_bfloat16* __restrict__ dzb, fl
       }
 }
 
-// Slices of the pixels: enough CTAs for three per SM, at least 256 pixels each.
-int conv_dw_splits(int N, int H, int W, int C, int stride, int cout, int64_t part_floats) {
-  const int64_t M = int64_t(N) * (H / stride) * (W / stride), len = int64_t(cout) * 9 * C;
-  const int bm = cout <= 32 ? 32 : (cout <= 64 ? 64 : 128);
-  const int64_t tiles = ((9 * C + DW_BN - 1) / DW_BN) * ((cout + bm - 1) / bm);
-  int64_t sp = (456 + tiles - 1) / tiles;
-  if (sp > M / 256) sp = M / 256;
-  if (sp > part_floats / len) sp = part_floats / len;
-  return static_cast<int>(sp < 1 ? 1 : sp);
+// Slices of the pixels: about 2048 each, at most 64.
+int conv_dw_splits(int N, int H, int W, int stride) {
+  const int64_t sp = int64_t(N) * (H / stride) * (W / stride) / 2048;
+  return static_cast<int>(sp < 1 ? 1 : (sp > 64 ? 64 : sp));
 }
 
 cudaError_t conv_dw(const float* x, const __nv_bfloat16* dzb, float* dw, int N, int H, int W, int C, int stride,
-                    int cout, bool up, float* part, int64_t part_floats, cudaStream_t s) {
+                    int cout, bool up, float* part, cudaStream_t s) {
   const int64_t M = int64_t(N) * (H / stride) * (W / stride), len = int64_t(cout) * 9 * C;
-  int splits = conv_dw_splits(N, H, W, C, stride, cout, part_floats);
+  int splits = conv_dw_splits(N, H, W, stride);
   int64_t kchunk = (M + splits - 1) / splits;
   kchunk = (kchunk + DW_BK - 1) / DW_BK * DW_BK;
   splits = static_cast<int>((M + kchunk - 1) / kchunk);
   float* dst = splits > 1 ? part : dw;
   const int vecx = C % 8 == 0 && aligned16(x) ? 1 : 0, u = up ? 1 : 0;
-  const int bm = cout <= 32 ? 32 : (cout <= 64 ? 64 : 128);
-  const dim3 grid((9 * C + DW_BN - 1) / DW_BN, (cout + bm - 1) / bm, splits);
+  // fewer output channels per CTA where the tiles and slices leave SMs idle
+  const int64_t ntile = (9 * C + DW_BN - 1) / DW_BN;
+  int bm = cout <= 32 ? 32 : (cout <= 64 ? 64 : 128);
+  while (bm > 32 && ntile * ((cout + bm - 1) / bm) * splits < 152) bm /= 2;
+  const dim3 grid(static_cast<unsigned>(ntile), (cout + bm - 1) / bm, splits);
   const int kc = static_cast<int>(kchunk);
   if (bm == 32) k_conv_dw<32><<<grid, 256, 0, s>>>(x, dzb, dst, N, H, W, C, stride, cout, u, kc, vecx);
   else if (bm == 64) k_conv_dw<64><<<grid, 256, 0, s>>>(x, dzb, dst, N, H, W, C, stride, cout, u, kc, vecx);
   else k_conv_dw<128><<<grid, 256, 0, s>>>(x, dzb, dst, N, H, W, C, stride, cout, u, kc, vecx);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || splits == 1) return e;
-  k_sum_parts<<<static_cast<unsigned>((len + 63) / 64), 256, 0, s>>>(part, dw, len, splits);
+  k_sum_slices<<<static_cast<unsigned>((len + 127) / 128), 128, 0, s>>>(part, dw, len, splits);
   return cudaGetLastError();
 }
 

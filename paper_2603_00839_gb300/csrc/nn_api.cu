@@ -181,15 +181,15 @@ rtg_status conv_bwd(rtg_warmstart* ws, int l, const float* x, int h, int w, bool
   __nv_bfloat16* dzb = ws->dzb.as<__nv_bfloat16>();
   float* part = ws->part.as<float>();
   NCK(nn::mask_grad(dy, mask, dzb, G + L.b, part, M, L.cout, s));
-  NCK(nn::conv_dw(x, dzb, G + L.w, ws->N, h, w, L.cin, L.stride, L.cout, up, part, int64_t(ws->part.bytes / 4), s));
+  NCK(nn::conv_dw(x, dzb, G + L.w, ws->N, h, w, L.cin, L.stride, L.cout, up, part, s));
   if (dx != nullptr)
     NCK(nn::conv_dx(dzb, Wb(ws, l), addend, dx, ws->N, h, w, L.cin, L.stride, L.cout, up, s));
   return RTG_OK;
 }
 
-// One forward layer through the implicit-GEMM kernel: r = relu(conv(x) + b)
-// (when r), out = r + skip (skip may be null); the output layer has no ReLU.
-// up: x is the half-resolution tensor, read through its x2 up-sampling.
+// One forward layer: r = relu(conv(x) + b) (when r), out = r + skip (skip may
+// be null).  up: x is the half-resolution tensor, read through its x2
+// up-sampling.
 rtg_status layer_fwd(rtg_warmstart* ws, int l, const float* x, int h, int w, bool up, float* r, const float* skip,
                      float* out, cudaStream_t s) {
   const Layer& L = ws->L[l];
@@ -203,16 +203,24 @@ rtg_status layer_fwd(rtg_warmstart* ws, int l, const float* x, int h, int w, boo
 // through the convolutions' gather.
 rtg_status forward(rtg_warmstart* ws, const float* C, float* X0, float* loglam_out, bool training, cudaStream_t s) {
   const int N = ws->N, H = ws->H, W = ws->W, c = ws->base;
-  NCK(nn::to_nhwc(C, ws->x0, N, H, W, 3, s));
-  NRK(layer_fwd(ws, E1, ws->x0, H, W, false, nullptr, nullptr, ws->e1, s));
+  // the input layer reads the solver's planar images; the backward pass wants them channels last
+  if (training) NCK(nn::to_nhwc(C, ws->x0, N, H, W, 3, s));
+  NCK(nn::conv_fwd(C, Wb(ws, E1), Bf(ws, E1), nullptr, nullptr, ws->e1, N, H, W, 3, 1, c, true, false, nullptr, 0, s,
+                   true));
   NRK(layer_fwd(ws, E2, ws->e1, H, W, false, nullptr, nullptr, ws->e2, s));
   NRK(layer_fwd(ws, E3, ws->e2, H / 2, W / 2, false, nullptr, nullptr, ws->e3, s));
   NRK(layer_fwd(ws, E4, ws->e3, H / 4, W / 4, false, nullptr, nullptr, ws->e4, s));
   NRK(layer_fwd(ws, D3, ws->e4, H / 4, W / 4, true, training ? ws->r3 : nullptr, ws->e3, ws->d3, s));
   NRK(layer_fwd(ws, D2, ws->d3, H / 2, W / 2, true, training ? ws->r2 : nullptr, ws->e2, ws->d2, s));
   NRK(layer_fwd(ws, D1, ws->d2, H, W, true, training ? ws->r1 : nullptr, ws->e1, ws->d1, s));
-  NRK(layer_fwd(ws, OUT, ws->d1, H, W, false, nullptr, nullptr, ws->zo, s));
-  NCK(nn::from_nhwc_add(ws->zo, C, X0, N, H, W, 3, s));
+  // X_0 = C + out: in the output layer's epilogue where the tile kernel runs it
+  if (nn::conv_tile_kind(ws->d1, Wb(ws, OUT), H, W, c, 1, 8, false)) {
+    NCK(nn::conv_fwd(ws->d1, Wb(ws, OUT), Bf(ws, OUT), nullptr, nullptr, X0, N, H, W, c, 1, 3, false, false,
+                     ws->slices.as<float>(), int64_t(ws->slices.bytes / 4), s, false, C));
+  } else {
+    NRK(layer_fwd(ws, OUT, ws->d1, H, W, false, nullptr, nullptr, ws->zo, s));
+    NCK(nn::from_nhwc_add(ws->zo, C, X0, N, H, W, 3, s));
+  }
   const float* Pf = ws->P.as<float>();
   NCK(nn::pool_head(ws->e4, Pf + ws->head_w, Pf + ws->head_b, ws->g, loglam_out, ws->slices.as<float>(), N,
                     (H / 8) * (W / 8), 4 * c, s));
@@ -365,13 +373,13 @@ rtg_status rtg_nn_conv3x3(int32_t device, int32_t N, int32_t H, int32_t W, int32
     NCK(nn::conv_fwd(x, wb.as<__nv_bfloat16>(), b, nullptr, nullptr, y, N, H, W, cin, stride, cout, false, false,
                      nullptr, 0, s));
   if (dy != nullptr) {
-    const int64_t splits = nn::conv_dw_splits(N, H, W, cin, stride, cout, int64_t(1) << 62);
-    const int64_t pf = std::max<int64_t>(int64_t(nn::mask_grad_blocks(M)) * cout, splits * cout * K);
+    const int64_t splits = nn::conv_dw_splits(N, H, W, stride);
+    const int64_t pf = std::max<int64_t>(int64_t(256) * cout, splits * cout * K);
     NRK(zb.ensure(size_t(M) * cout * 2));
     NRK(part.ensure(size_t(pf) * 4 + 64));
     NCK(nn::mask_grad(dy, nullptr, zb.as<__nv_bfloat16>(), db, part.as<float>(), M, cout, s));
     if (dw != nullptr)
-      NCK(nn::conv_dw(x, zb.as<__nv_bfloat16>(), dw, N, H, W, cin, stride, cout, false, part.as<float>(), pf, s));
+      NCK(nn::conv_dw(x, zb.as<__nv_bfloat16>(), dw, N, H, W, cin, stride, cout, false, part.as<float>(), s));
     if (dx != nullptr)
       NCK(nn::conv_dx(zb.as<__nv_bfloat16>(), wb.as<__nv_bfloat16>(), nullptr, dx, N, H, W, cin, stride, cout, false, s));
   }

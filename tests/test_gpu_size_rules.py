@@ -90,6 +90,33 @@ def test_convolution_gradients(api, N, H, W, cin, cout, stride):
         assert float((got.double() - ref).norm()) <= 5e-6 * float(ref.norm()) + 1e-12
 
 
+@pytest.mark.parametrize("N,H,W,cin,cout,stride", [
+    (1, 1, 1, 3, 1, 1),          # the three-channel kernel's smallest
+    (2, 18, 34, 3, 40, 2),       # and its stride 2, ragged, 64 output channels at a time
+    (1, 9, 17, 16, 8, 1),        # the tile kernel: one step of channels per tap, ragged tiles
+    (2, 20, 36, 48, 129, 2),     # two tiles of output channels, stride 2
+    (1, 8, 16, 128, 3, 1),       # one tile, the output layer's channel count
+    (1, 7, 5, 20, 33, 1),        # channels in no step of 16: the general kernel
+])
+def test_convolution_forward(api, N, H, W, cin, cout, stride):
+    x, wt = _bf16_exact((N, H, W, cin), 7), _bf16_exact((cout, 3, 3, cin), 8)
+    b = torch.randn(cout, device="cuda", generator=torch.Generator("cuda").manual_seed(9))
+    y = api.conv3x3(x, wt, b, stride=stride)
+    ref = torch.nn.functional.conv2d(x.double().permute(0, 3, 1, 2), wt.double().permute(0, 3, 1, 2), b.double(),
+                                     stride=stride, padding=1).permute(0, 2, 3, 1)
+    # exact products, FP32 sums of at most 9 * 128 of them
+    assert float((y.double() - ref).norm()) <= 5e-6 * float(ref.norm())
+
+
+@pytest.mark.parametrize("cin", [16, 48])
+def test_convolution_kernels_agree(api, cin):
+    """An input on no 16-byte boundary runs the general kernel: the tile kernel's bits."""
+    buf = _bf16_exact((2 * 13 * 21 * cin + 1,), 10) * 1.001
+    x = buf[1:].view(2, 13, 21, cin)
+    wt, b = _bf16_exact((24, 3, 3, cin), 11), _bf16_exact((24,), 12)
+    assert torch.equal(api.conv3x3(x, wt, b), api.conv3x3(x.clone(), wt, b))
+
+
 def test_convolution_gradients_of_unaligned_input(api):
     """x on no 16-byte boundary takes the scalar gather: the same bits as the aligned copy."""
     buf = _bf16_exact((1 * 12 * 20 * 16 + 1,), 4)
