@@ -116,25 +116,31 @@ cudaError_t mask_grad(const float* dy, const float* mask, __nv_bfloat16* dzb, fl
 // ------------------------------------------------------------------ weight gradient
 // dw[o, tap, c] = sum over output pixels p of dz[p, o] x[p + tap, c], as a GEMM
 // with M = output channels, N = (tap, input channel) and K = pixels.  CTA tile
-// BM x 64, K in stages of 32 pixels, double buffered: dz rows arrive with
+// BM x 64, K in stages of 128 pixels (64 for BM = 128), double buffered (with
+// stages of 32 the loads' latency was most of a stage): dz rows arrive with
 // 16-byte loads, the patch entries are gathered from x (FP32, rounded to BF16
 // on the way) while the stage before is multiplied; both operands lie [k][.]
 // in shared memory and are read with transposing ldmatrix.  gridDim.z splits
 // the pixels; slice z writes part[z].  16 x 128 x 128, all eight layers: 2.93
 // ms of GEMM (scalar loads) and 2.16 ms of im2col before.
-constexpr int DW_BN = 64, DW_BK = 32;
+constexpr int DW_BN = 64;
+template <int BM>
+__host__ __device__ constexpr int dw_bk() { return BM >= 128 ? 64 : 128; }
+template <int BM>
+constexpr size_t dw_smem() { return size_t(2) * dw_bk<BM>() * (BM + 8 + DW_BN + 8) * 2; }
 
 template <int BM>
 __global__ void __launch_bounds__(256)
 k_conv_dw(const float* __restrict__ x, const __nv_bfloat16* __restrict__ dzb, float* __restrict__ part, int N, int H,
           int W, int C, int stride, int cout, int up, int kchunk, int vecx) {
-  constexpr int PA = BM + 8, PB = DW_BN + 8;
-  __shared__ __align__(16) __nv_bfloat16 As[2][DW_BK][PA];
-  __shared__ __align__(16) __nv_bfloat16 Bs[2][DW_BK][PB];
+  constexpr int BK = dw_bk<BM>(), PA = BM + 8, PB = DW_BN + 8;
+  extern __shared__ __align__(16) unsigned char dw_sm[];
+  __nv_bfloat16(*As)[BK][PA] = reinterpret_cast<__nv_bfloat16(*)[BK][PA]>(dw_sm);
+  __nv_bfloat16(*Bs)[BK][PB] = reinterpret_cast<__nv_bfloat16(*)[BK][PB]>(dw_sm + size_t(2) * BK * PA * 2);
   constexpr int WM = BM >= 64 ? 4 : 2, WN = 8 / WM;          // warps along M and N
   constexpr int MT = BM / (16 * WM), NT = DW_BN / (8 * WN);  // m16 and n8 tiles per warp
-  constexpr int ACH = DW_BK * BM / 8;                        // 16-byte pieces of an A stage
-  constexpr int AP = (ACH + 255) / 256;
+  constexpr int ACH = BK * BM / 8;                        // 16-byte pieces of an A stage
+  constexpr int AP = (ACH + 255) / 256, BP = BK / 32;        // pieces per thread
   const int Ho = H / stride, Wo = W / stride;
   const int M = N * Ho * Wo, K9 = 9 * C;
   const int n0 = blockIdx.x * DW_BN, m0 = blockIdx.y * BM;
@@ -143,9 +149,16 @@ k_conv_dw(const float* __restrict__ x, const __nv_bfloat16* __restrict__ dzb, fl
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, gid = lane >> 2, tig = lane & 3;
   const int wm = (warp % WM) * 16 * MT, wn = (warp / WM) * 8 * NT;
   const bool veca = cout % 8 == 0;
-  // this thread's piece of a B stage: one pixel, eight columns
+  // this thread's pieces of a B stage: eight columns of every 32nd pixel
   const int brow = tid >> 3, j0 = n0 + (tid & 7) * 8;
-  uint4 ra[AP], rb;
+  const int tap0 = j0 / C, ch0 = j0 - tap0 * C, ky0 = tap0 / 3, kx0 = tap0 - 3 * ky0;   // (vecx: all eight)
+  int ent[8];   // otherwise: channel, ky and kx of each (negative: past K9)
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int jj = j0 + k, tap = jj / C;
+    ent[k] = jj < K9 ? (jj - tap * C) << 4 | (tap / 3) << 2 | tap % 3 : -1;
+  }
+  uint4 ra[AP], rb[BP];
   auto load = [&](int k0) {
 #pragma unroll
     for (int q = 0; q < AP; ++q) {
@@ -163,31 +176,43 @@ k_conv_dw(const float* __restrict__ x, const __nv_bfloat16* __restrict__ dzb, fl
         ra[q] = make_uint4(h[0] | h[1] << 16, h[2] | h[3] << 16, h[4] | h[5] << 16, h[6] | h[7] << 16);
       }
     }
-    rb = make_uint4(0u, 0u, 0u, 0u);
-    const int p = k0 + brow;
-    if (p >= kend || j0 >= K9) return;
-    const int j = p % Wo, t1 = p / Wo, i = t1 % Ho, n = t1 / Ho;
     if (vecx) {   // eight channels of one tap
-      const int tap = j0 / C, c = j0 - tap * C, ky = tap / 3, kx = tap - 3 * ky;
-      const int yy = stride * i + ky - 1, xx = stride * j + kx - 1;
-      if (yy < 0 || yy >= H || xx < 0 || xx >= W) return;
-      const float4* s4 = reinterpret_cast<const float4*>(
-          x + ((static_cast<int64_t>(n) * Hs + (yy >> up)) * Ws + (xx >> up)) * C + c);
-      const float4 a = s4[0], b = s4[1];
-      rb = make_uint4(pack_bf16(a.x, a.y), pack_bf16(a.z, a.w), pack_bf16(b.x, b.y), pack_bf16(b.z, b.w));
-    } else {
+      float4 fa[BP], fb[BP];
+#pragma unroll
+      for (int q = 0; q < BP; ++q) {
+        fa[q] = fb[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+        const int p = k0 + brow + 32 * q;
+        if (p >= kend || j0 >= K9) continue;
+        const int j = p % Wo, t1 = p / Wo, i = t1 % Ho, n = t1 / Ho;
+        const int yy = stride * i + ky0 - 1, xx = stride * j + kx0 - 1;
+        if (yy < 0 || yy >= H || xx < 0 || xx >= W) continue;
+        const float4* s4 = reinterpret_cast<const float4*>(
+            x + ((static_cast<int64_t>(n) * Hs + (yy >> up)) * Ws + (xx >> up)) * C + ch0);
+        fa[q] = s4[0];
+        fb[q] = s4[1];
+      }
+#pragma unroll
+      for (int q = 0; q < BP; ++q)
+        rb[q] = make_uint4(pack_bf16(fa[q].x, fa[q].y), pack_bf16(fa[q].z, fa[q].w), pack_bf16(fb[q].x, fb[q].y),
+                           pack_bf16(fb[q].z, fb[q].w));
+      return;
+    }
+#pragma unroll
+    for (int q = 0; q < BP; ++q) {
+      const int p = k0 + brow + 32 * q;
       float v[8];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        v[k] = 0.f;
-        const int jj = j0 + k;
-        if (jj >= K9) continue;
-        const int tap = jj / C, c = jj - tap * C, ky = tap / 3, kx = tap - 3 * ky;
-        const int yy = stride * i + ky - 1, xx = stride * j + kx - 1;
-        if (yy >= 0 && yy < H && xx >= 0 && xx < W)
-          v[k] = x[((static_cast<int64_t>(n) * Hs + (yy >> up)) * Ws + (xx >> up)) * C + c];
+      for (int k = 0; k < 8; ++k) v[k] = 0.f;
+      if (p < kend) {
+        const int j = p % Wo, t1 = p / Wo, i = t1 % Ho, n = t1 / Ho;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const int yy = stride * i + (ent[k] >> 2 & 3) - 1, xx = stride * j + (ent[k] & 3) - 1;
+          if (ent[k] >= 0 && yy >= 0 && yy < H && xx >= 0 && xx < W)
+            v[k] = x[((static_cast<int64_t>(n) * Hs + (yy >> up)) * Ws + (xx >> up)) * C + (ent[k] >> 4)];
+        }
       }
-      rb = make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+      rb[q] = make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
     }
   };
   auto store = [&](int buf) {
@@ -196,7 +221,8 @@ k_conv_dw(const float* __restrict__ x, const __nv_bfloat16* __restrict__ dzb, fl
       const int e = tid + q * 256;
       if (e < ACH) *reinterpret_cast<uint4*>(&As[buf][e / (BM / 8)][(e % (BM / 8)) * 8]) = ra[q];
     }
-    *reinterpret_cast<uint4*>(&Bs[buf][brow][(tid & 7) * 8]) = rb;
+#pragma unroll
+    for (int q = 0; q < BP; ++q) *reinterpret_cast<uint4*>(&Bs[buf][brow + 32 * q][(tid & 7) * 8]) = rb[q];
   };
   float acc[MT][NT][4];
 #pragma unroll
@@ -210,11 +236,11 @@ k_conv_dw(const float* __restrict__ x, const __nv_bfloat16* __restrict__ dzb, fl
   __syncthreads();
   const int mi = lane >> 3, r8 = lane & 7;
   int buf = 0;
-  for (int k0 = kbeg; k0 < kend; k0 += DW_BK) {
-    const bool more = k0 + DW_BK < kend;
-    if (more) load(k0 + DW_BK);
-#pragma unroll
-    for (int kk = 0; kk < DW_BK; kk += 16) {
+  for (int k0 = kbeg; k0 < kend; k0 += BK) {
+    const bool more = k0 + BK < kend;
+    if (more) load(k0 + BK);
+#pragma unroll 2
+    for (int kk = 0; kk < BK; kk += 16) {
       uint32_t a[MT][4];
 #pragma unroll
       for (int mt = 0; mt < MT; ++mt)
@@ -262,7 +288,7 @@ cudaError_t conv_dw(const float* x, const __nv_bfloat16* dzb, float* dw, int N, 
   const int64_t M = int64_t(N) * (H / stride) * (W / stride), len = int64_t(cout) * 9 * C;
   int splits = conv_dw_splits(N, H, W, stride);
   int64_t kchunk = (M + splits - 1) / splits;
-  kchunk = (kchunk + DW_BK - 1) / DW_BK * DW_BK;
+  kchunk = (kchunk + 31) / 32 * 32;
   splits = static_cast<int>((M + kchunk - 1) / kchunk);
   float* dst = splits > 1 ? part : dw;
   const int vecx = C % 8 == 0 && aligned16(x) ? 1 : 0, u = up ? 1 : 0;
@@ -272,10 +298,16 @@ cudaError_t conv_dw(const float* x, const __nv_bfloat16* dzb, float* dw, int N, 
   while (bm > 32 && ntile * ((cout + bm - 1) / bm) * splits < 152) bm /= 2;
   const dim3 grid(static_cast<unsigned>(ntile), (cout + bm - 1) / bm, splits);
   const int kc = static_cast<int>(kchunk);
-  if (bm == 32) k_conv_dw<32><<<grid, 256, 0, s>>>(x, dzb, dst, N, H, W, C, stride, cout, u, kc, vecx);
-  else if (bm == 64) k_conv_dw<64><<<grid, 256, 0, s>>>(x, dzb, dst, N, H, W, C, stride, cout, u, kc, vecx);
-  else k_conv_dw<128><<<grid, 256, 0, s>>>(x, dzb, dst, N, H, W, C, stride, cout, u, kc, vecx);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = cudaSuccess;
+#define RTG_DW_CASE(B_)                                                                                       \
+  if (bm == B_) {                                                                                             \
+    e = set_smem(k_conv_dw<B_>, dw_smem<B_>());                                                               \
+    if (e != cudaSuccess) return e;                                                                           \
+    k_conv_dw<B_><<<grid, 256, dw_smem<B_>(), s>>>(x, dzb, dst, N, H, W, C, stride, cout, u, kc, vecx);       \
+  }
+  RTG_DW_CASE(32) RTG_DW_CASE(64) RTG_DW_CASE(128)
+#undef RTG_DW_CASE
+  e = cudaGetLastError();
   if (e != cudaSuccess || splits == 1) return e;
   k_sum_slices<<<static_cast<unsigned>((len + 127) / 128), 128, 0, s>>>(part, dw, len, splits);
   return cudaGetLastError();
