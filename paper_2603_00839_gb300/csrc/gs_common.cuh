@@ -187,6 +187,25 @@ __device__ __forceinline__ float double_to_float_rn(double x) {
   return __uint_as_float(static_cast<unsigned>(r) | (static_cast<unsigned>(b >> 32) & 0x80000000u));
 }
 
+// x as the FP32 value nearest to it and the FP32 value nearest to the rest, as
+// the two conversions would give them, without the FP64 pipe's round trips:
+// the rest of a 53-bit significand after its rounding to 24 bits is an
+// integer of at most 29 bits.
+__device__ __forceinline__ FF double_split_rn(double x) {
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x));
+  const int e = static_cast<int>(b >> 52) & 0x7ff;
+  if (e < 1023 - 60 || e > 1023 + 126) {
+    const float hi = double_to_float_rn(x);
+    return {hi, double_to_float_rn(x - static_cast<double>(hi))};
+  }
+  const float hi = double_to_float_rn(x);
+  const unsigned long long m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
+  const unsigned long long top = (m + 0x0fffffffull + ((m >> 29) & 1ull)) >> 29;   // as rounded (up to 2^24)
+  const int rest = static_cast<int>(static_cast<long long>(m) - static_cast<long long>(top << 29));
+  const float lo = static_cast<float>(rest) * __int_as_float((e - 1023 - 52 + 127) << 23);   // exact scaling
+  return {hi, b >> 63 ? -lo : lo};
+}
+
 // A coefficient in the data's type.
 template <typename T>
 __device__ __forceinline__ T coef_as(double x) {
@@ -317,6 +336,9 @@ __device__ __forceinline__ FF ff_warps_total(const FF (*red)[kRedCols], int nw, 
 // entries side by side): float-float pairs for FP32 data, doubles for FP64
 // data.
 // red: shared [GS_MAXW][kRedCols] doubles (float-float pairs for FP32).
+// FP64 data: blocks with the same entries may share the columns, block y of
+// gridDim.y taking the columns y, y + gridDim.y, ... (and s . s by block 0):
+// the FP64 work of a column is some 2000 cycles of its SM.
 template <typename T, int ITEMS>
 __device__ void block_partials(const Work& w, const T* vals, const int64_t* idx, int cnt, int J,
                                double (*red)[kRedCols]) {
@@ -333,12 +355,15 @@ __device__ void block_partials(const Work& w, const T* vals, const int64_t* idx,
     qJ[k] = (ok && J >= 0) ? Q[static_cast<int64_t>(J) * d + idx[k]] : static_cast<T>(0);
   }
   FF (*rf)[kRedCols] = reinterpret_cast<FF (*)[kRedCols]>(red);
-  {   // s . s
+  if (sizeof(T) == 4 || blockIdx.y == 0) {   // s . s
     DotAcc<T> a;
     if constexpr (sizeof(T) == 4) a.v = ff_prod(sv[0], sv[0]);
     else a.add(sv[0], sv[0]);
 #pragma unroll
-    for (int k = 1; k < ITEMS; ++k) a.add(sv[k], sv[k]);
+    for (int k = 1; k < ITEMS; ++k) {
+      if (sizeof(T) == 8 && k >= cnt) break;   // (the entries past it are zero)
+      a.add(sv[k], sv[k]);
+    }
     if constexpr (sizeof(T) == 4) {
       const FF t = ff_warp_sum(a.v);
       if (lane == 0) rf[warp][J + 1] = t;
@@ -359,37 +384,45 @@ __device__ void block_partials(const Work& w, const T* vals, const int64_t* idx,
       else ff_dot_group<1, ITEMS>(Q, d, sv, qJ, idx, cnt, i0, J, rf, warp, lane);
     }
   } else {
-    // columns of Q in groups of 8: all loads of a group go out before any use
-    constexpr int GRP = 8;
-    for (int i0 = 0; i0 <= J; i0 += GRP) {
+    // four columns of Q at a time: all their loads go out before any use
+    constexpr int GRP = 4;
+    const int step = gridDim.y;
+    for (int i0 = blockIdx.y; i0 <= J; i0 += GRP * step) {
       T qv[GRP][ITEMS];
 #pragma unroll
       for (int g = 0; g < GRP; ++g)
 #pragma unroll
         for (int k = 0; k < ITEMS; ++k) {
-          const bool ok = k < cnt && idx[k] >= 0 && i0 + g <= J;
-          qv[g][k] = ok ? Q[static_cast<int64_t>(i0 + g) * d + idx[k]] : static_cast<T>(0);
+          const bool ok = k < cnt && idx[k] >= 0 && i0 + g * step <= J;
+          qv[g][k] = ok ? Q[static_cast<int64_t>(i0 + g * step) * d + idx[k]] : static_cast<T>(0);
         }
 #pragma unroll
       for (int g = 0; g < GRP; ++g) {
-        if (i0 + g > J) break;
-        DotAcc<T> p, q;
+        const int i = i0 + g * step;
+        if (i > J) break;
+        double p = 0.0, q = 0.0;
 #pragma unroll
         for (int k = 0; k < ITEMS; ++k) {
-          p.add(sv[k], qv[g][k]);
-          q.add(qJ[k], qv[g][k]);
+          if (k >= cnt) break;   // (the entries past it are zero)
+          p = fma(sv[k], qv[g][k], p);
+          q = fma(qJ[k], qv[g][k], q);
         }
-        const double tp = p.warp_total(), tq = q.warp_total();
-        if (lane == 0) {
-          red[warp][i0 + g] = tp;
-          red[warp][J + 2 + i0 + g] = tq;
-        }
+        // both warp sums in one tree: the lower half-warp goes on with p, the upper with q
+        const bool up = (lane & 16) != 0;
+        double v = (up ? q : p) + __shfl_xor_sync(0xffffffffu, up ? p : q, 16);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if ((lane & 15) == 0) red[warp][up ? J + 2 + i : i] = v;
       }
     }
   }
   __syncthreads();
-  const int64_t row = blockIdx.x + gridDim.x * blockIdx.y;
+  const int64_t row = sizeof(T) == 4 ? blockIdx.x + gridDim.x * blockIdx.y : blockIdx.x;
   for (int i = threadIdx.x; i < ncols; i += blockDim.x) {
+    if constexpr (sizeof(T) == 8) {   // this block's columns
+      const int c = i <= J ? i : i - (J + 2);
+      if (c < 0 ? blockIdx.y != 0 : c % gridDim.y != blockIdx.y) continue;
+    }
     const int64_t at = static_cast<int64_t>(i) * w.part_rows + row;
     if constexpr (sizeof(T) == 4) reinterpret_cast<FF*>(w.part)[at] = ff_warps_total(rf, nw, i);
     else w.part[at] = warps_total(red, nw, i);
@@ -434,8 +467,9 @@ __device__ inline bool last_block_combine(const Work& w, int ncols, typename Sum
   using A = Sum<T>;
   using V = typename A::V;
   __syncthreads();
-  const unsigned nblk = gridDim.x * gridDim.y;
-  if (threadIdx.x == 0) *am_last = (ticket_acq_rel(w.counter, nblk - 1) == nblk - 1);
+  const unsigned all = gridDim.x * gridDim.y;
+  const unsigned nblk = sizeof(T) == 4 ? all : gridDim.x;   // entries of a column
+  if (threadIdx.x == 0) *am_last = (ticket_acq_rel(w.counter, all - 1) == all - 1);
   __syncthreads();
   if (!*am_last) return false;
   if constexpr (!std::is_same<Pre, void (*)()>::value) pre();   // e.g. start the Gram staging copies
@@ -544,8 +578,8 @@ __device__ inline void gs_finish_start(const Work& w, const StepOpts& o, const t
 
 // Starts the asynchronous copies of the stored Gram matrix rows and columns
 // 0..J-1 into the finish's shared staging area, so that they travel while
-// the last block combines the partial rows; the finish called with
-// staged = true waits for them.  Only where the finish stages G
+// the last block combines the partial sums; the finish waits for them.  Only
+// where the finish stages G
 // (J + 1 <= kGramSmemRows).  G is symmetric, so column k of G (contiguous
 // in global memory) is copied to row k of the staging area, in 16-byte
 // copies that bypass L1 (cp.async.cg): G's addresses are rewritten with
@@ -601,19 +635,11 @@ __device__ inline void gs_finish_gram(const Work& w, const StepOpts& o, int J, c
     double* Gs = red + 4;              // n x n
     double* pr = Gs + n * lg;          // [nw][n] partial products
     double* ab = pr + nw * n;          // [2][2] the two warps' sums of a and b
-    for (int e0 = 0; e0 < n * n; e0 += 8 * static_cast<int>(blockDim.x)) {   // eight loads in flight
-      double v[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int e = e0 + u * blockDim.x + threadIdx.x;
-        const int i = e % n, k = e / n;
-        v[u] = (e >= n * n) ? 0.0 : (i == J) ? grow[k] : (k == J ? grow[i] : __ldcg(G + i + static_cast<int64_t>(ldg) * k));
-      }
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int e = e0 + u * blockDim.x + threadIdx.x;
-        if (e < n * n) Gs[(e % n) * lg + e / n] = v[u];
-      }
+    // rows and columns < J arrived by gs_stage_gram_async; J from the new row
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      Gs[J * lg + i] = grow[i];
+      Gs[i * lg + J] = grow[i];
     }
     for (int i = threadIdx.x; i <= J; i += blockDim.x) {   // new row/column, for later steps
       G[i + static_cast<int64_t>(ldg) * J] = grow[i];
@@ -652,8 +678,7 @@ __device__ inline void gs_finish_gram(const Work& w, const StepOpts& o, int J, c
       const int i = threadIdx.x & 63, which = warp >> 1;
       double p = 0.0;
       if (i < n) p = which == 0 ? col[i] * h1[i] : col[i] * wsum(i);
-      const float hi = double_to_float_rn(p);
-      FF v{hi, double_to_float_rn(p - static_cast<double>(hi))};
+      FF v = double_split_rn(p);
       v = ff_warp_sum(v);
       if (lane == 0) ab[warp] = ff_to_double(v);
     }
@@ -739,8 +764,7 @@ __device__ inline void gs_finish_gram(const Work& w, const StepOpts& o, int J, c
 // 512 x 512 x 3 28.6 -> 24.2 us, 1024 x 1024 x 3 40.4 -> 33.8 us,
 // 256 x 256 x 3 x 64 (1728 blocks to combine) 149 -> 107 us; the error of
 // solves against 64 bits is the same to two digits, ill-conditioned ones too.
-__device__ inline void gs_finish_gram_ff(const Work& w, const StepOpts& o, int J, const FF* tot, double* sh,
-                                         bool staged = false) {
+__device__ inline void gs_finish_gram_ff(const Work& w, const StepOpts& o, int J, const FF* tot, double* sh) {
   Ctl* ctl = w.ctl;
   const int ld = w.m + 1, ldg = gram_ld(w.m);
   const double bd_tol = o.desc_bd_tol ? *o.desc_bd_tol : o.bd_tol;   // loaded early, used at the end
@@ -760,28 +784,11 @@ __device__ inline void gs_finish_gram_ff(const Work& w, const StepOpts& o, int J
     // G staged in shared memory (even row stride); each product G x runs
     // on every warp: warp w takes a slice of the columns, lane the rows
     // lane and lane + 32, and the warps' partial rows are summed in order
-    if (staged) {   // rows and columns < J arrived by gs_stage_gram_async; J from the new row
-      asm volatile("cp.async.wait_all;\n" ::: "memory");
-      for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        Gs[J * lg + i] = grow[i];
-        Gs[i * lg + J] = grow[i];
-      }
-    } else {
-      for (int e0 = 0; e0 < n * n; e0 += 8 * static_cast<int>(blockDim.x)) {   // eight loads in flight
-        FF v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int e = e0 + u * blockDim.x + threadIdx.x;
-          const int i = e % n, k = e / n;
-          v[u] = (e >= n * n) ? FF{0.f, 0.f}
-                              : (i == J) ? grow[k] : (k == J ? grow[i] : Sum<float>::ldcg(G + i + static_cast<int64_t>(ldg) * k));
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int e = e0 + u * blockDim.x + threadIdx.x;
-          if (e < n * n) Gs[(e % n) * lg + e / n] = v[u];
-        }
-      }
+    // rows and columns < J arrived by gs_stage_gram_async; J from the new row
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      Gs[J * lg + i] = grow[i];
+      Gs[i * lg + J] = grow[i];
     }
     for (int i = threadIdx.x; i <= J; i += blockDim.x) {   // new row/column, for later steps
       G[i + static_cast<int64_t>(ldg) * J] = grow[i];

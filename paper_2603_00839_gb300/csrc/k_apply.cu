@@ -372,6 +372,75 @@ k_apply_reg(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, FusedArgs a,
 #undef t1
 #undef t2
 
+// FP64 data on few tiles: the FP64 pipe retires 1.7 multiply-adds per SM and
+// cycle, so what counts is how many SMs take part.  Tile 32 x 4, 128 threads
+// (a warp per sub-partition), one output per thread and channel, the same
+// taps (zero-padded to RR) in the same order as k_apply_reg.  64 x 64 x 3,
+// radius 4: 14.0 us on 12 CTAs of 64 x 16, 5.9 us on 96 (cold caches).
+constexpr int STX64 = 32, STY64 = 4, ST64_THREADS = STX64 * STY64;
+
+template <int NC, int RR>
+__global__ void __launch_bounds__(ST64_THREADS)
+k_apply_small64(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, FusedArgs a, Batch bt) {
+  const BIdx bi = bidx(bt);
+  Xr = Xr.at(bi.off);
+  Yr = Yr.at(bi.off);
+  Zr = Zr.at(bi.off);
+  stop = bsh(stop, bi.off);
+  if (stop != nullptr && *stop) return;
+  const double* X = Xr.get<const double>();
+  double* __restrict__ Y = Yr.get<double>();
+  const double* Z = Zr.get<const double>();
+  constexpr int NT = 2 * RR + 1, Wd = STX64 + 2 * RR, Ht = STY64 + 2 * RR;
+  __shared__ double in_s[NC][Ht][Wd];
+  __shared__ double tmp[NC][STY64][Wd];
+  const int x0 = blockIdx.x * STX64, y0 = blockIdx.y * STY64;
+  const int I1 = static_cast<int>(a.I1), I2 = static_cast<int>(a.I2);
+  const int64_t plane = a.I1 * a.I2;
+  const int ox = threadIdx.x % STX64, oy = threadIdx.x / STX64;
+  for (int64_t slab = bi.z; slab < a.nslab; slab += bi.nz) {
+    const double* Xs = X + slab * NC * plane;
+    __syncthreads();
+#pragma unroll 4
+    for (int e = threadIdx.x; e < NC * Ht * Wd; e += ST64_THREADS) {
+      const int row = e / Wd, xx = e - row * Wd, c = row / Ht, yy = row - c * Ht;
+      const int gy = y0 - RR + yy, gx = x0 - RR + xx;
+      const bool v = gy >= 0 && gy < I2 && gx >= 0 && gx < I1;
+      in_s[c][yy][xx] = v ? __ldcg(Xs + c * plane + static_cast<int64_t>(gy) * I1 + gx) : 0.0;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < NC * STY64 * Wd; e += ST64_THREADS) {   // mode 2, every staged column
+      const int row = e / Wd, xx = e - row * Wd, c = row / STY64, y = row - c * STY64;
+      double s = 0.0;
+#pragma unroll
+      for (int t = 0; t < NT; ++t) s = fma(a.t2p[t], in_s[c][y + t][xx], s);
+      tmp[c][y][xx] = s;
+    }
+    __syncthreads();
+    double acc[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {   // mode 1
+      double s = 0.0;
+#pragma unroll
+      for (int t = 0; t < NT; ++t) s = fma(a.t1p[t], tmp[c][oy][ox + t], s);
+      acc[c] = s;
+    }
+    const int gx = x0 + ox, gy = y0 + oy;
+    if (gx < I1 && gy < I2) {
+#pragma unroll
+      for (int p = 0; p < NC; ++p) {
+        double v = 0.0;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) v += a.M[p + NC * c] * acc[c];
+        const int64_t o = (slab * NC + p) * plane + static_cast<int64_t>(gy) * I1 + gx;
+        double out = a.alpha * v;
+        if (Z != nullptr) out += a.beta * Z[o];
+        Y[o] = out;
+      }
+    }
+  }
+}
+
 // ---------------------------------------------------------------- spatio-temporal path
 // One HBM pass for the video operator (order 4: blur on modes 1-2, channel
 // mix on mode 3, banded temporal filter of radius <= 2 on mode 4) and for
@@ -839,6 +908,21 @@ static cudaError_t apply_t(const OpPlan& op, PtrRef X, PtrRef Y, double alpha, d
       dim3 grid(static_cast<unsigned>((a.I1 + RTX - 1) / RTX), static_cast<unsigned>((a.I2 + RTY - 1) / RTY),
                 batch_z(a.nslab, b));
       cudaError_t e = cudaSuccess;
+      // FP64 with fewer tiles than SMs: small tiles (radii the static tile holds)
+      if constexpr (sizeof(T) == 8) {
+        if (rr <= 9 && int64_t(grid.x) * grid.y * grid.z < 152) {
+          const dim3 g64(static_cast<unsigned>((a.I1 + STX64 - 1) / STX64),
+                         static_cast<unsigned>((a.I2 + STY64 - 1) / STY64), grid.z);
+#define RTG_SMALL64_CASE(NC, RR)                                                        \
+  if (a.nc == NC && rr == RR) {                                                         \
+    k_apply_small64<NC, RR><<<g64, ST64_THREADS, 0, s>>>(X, Y, Z, stop, a, b);          \
+    return cudaGetLastError();                                                          \
+  }
+          RTG_SMALL64_CASE(1, 3) RTG_SMALL64_CASE(1, 5) RTG_SMALL64_CASE(1, 7) RTG_SMALL64_CASE(1, 9)
+          RTG_SMALL64_CASE(3, 3) RTG_SMALL64_CASE(3, 5) RTG_SMALL64_CASE(3, 7) RTG_SMALL64_CASE(3, 9)
+#undef RTG_SMALL64_CASE
+        }
+      }
 #define RTG_REG_CASE(NC, RR)                                                                          \
   if (a.nc == NC && rr == RR) {                                                                       \
     using Gm = RegGeom<RR, T>;                                                                        \

@@ -39,8 +39,8 @@ int gs_grid(int64_t d) {
   return static_cast<int>(g < 1 ? 1 : g);
 }
 
-// pass 0: start of the process, beta = ||S|| with S summed from the
-// chain's partial sketches; pass 1: one Arnoldi step's Gram-Schmidt
+// pass 0: start of the process, beta = ||S|| with S copied from the chain's
+// sketch; pass 1: one Arnoldi step's Gram-Schmidt
 // reduction on S (s . Q_i, s . s and the new Gram row) and its finish.
 template <typename T>
 __global__ void __launch_bounds__(GS_THREADS) k_gs_pass(Work w0, int pass, StepOpts o0, const int* gate) {
@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(GS_THREADS) k_gs_pass(Work w0, int pass, StepO
   const int J = (pass == 0) ? -1 : ctl->j;
   const int d = w.d;
   T* S = static_cast<T*>(w.S);
-  __shared__ double red[GS_MAXW][kRedCols];
+  __shared__ __align__(16) double red[GS_MAXW][kRedCols];
   __shared__ typename Sum<T>::V tot[kRedCols];
   __shared__ int am_last;
   const int64_t chunk = (d + gridDim.x - 1) / gridDim.x;
@@ -65,21 +65,23 @@ __global__ void __launch_bounds__(GS_THREADS) k_gs_pass(Work w0, int pass, StepO
   int cnt = 0;
   const T* P = static_cast<const T*>(w.Spart);
 #pragma unroll
-  for (int k = 0; k < GS_ITEMS; ++k) {
+  for (int k = 0; k < GS_ITEMS; ++k) {   // all loads before the first store
     ix[k] = lo + threadIdx.x + static_cast<int64_t>(k) * GS_THREADS;
     sv[k] = 0;
     if (ix[k] < hi) {
       cnt = k + 1;
-      T v = 0;
-      for (int p = 0; p < w.nparts; ++p) v += P[static_cast<int64_t>(p) * d + ix[k]];
-      S[ix[k]] = v;
-      sv[k] = v;
+      sv[k] = P[ix[k]];
     } else {
       ix[k] = -1;
     }
   }
+  if (blockIdx.y == 0)
+#pragma unroll
+    for (int k = 0; k < GS_ITEMS; ++k)
+      if (ix[k] >= 0) S[ix[k]] = sv[k];
   block_partials<T, GS_ITEMS>(w, sv, ix, cnt, J, red);
-  if (!last_block_combine<T>(w, gs_ncols(J), tot, &am_last, &red[0][0])) return;
+  auto stage = [&]() { gs_stage_gram_async(w, J, &red[0][0]); };   // (J < 1: nothing)
+  if (!last_block_combine<T>(w, gs_ncols(J), tot, &am_last, &red[0][0], stage)) return;
   if (pass == 0) {
     if (threadIdx.x == 0) gs_finish_start<T>(w, o, tot);
   } else if constexpr (sizeof(T) == 4) {
@@ -651,8 +653,15 @@ cudaError_t launch_start(const Work& w, PtrRef src, const StepOpts& o, bool fuse
   return cudaGetLastError();
 }
 
+// FP64: up to sixteen blocks share the columns of one slice of the sketch, as
+// many as two waves of the GPU hold (64 x 64 x 3, 7 steps: the pass 23.7 us
+// with one, 14.3 us with the finish's staging and splitting as they are now).
 cudaError_t launch_pass1(const Work& w, const StepOpts& o, cudaStream_t s) {
-  const dim3 g(static_cast<unsigned>(gs_grid(w.d)), 1, static_cast<unsigned>(w.b.n));
+  const int slices = gs_grid(w.d);
+  int share = 304 / slices;
+  share = share < 1 ? 1 : (share > 16 ? 16 : share);
+  if (share > w.m) share = w.m;
+  const dim3 g(static_cast<unsigned>(slices), w.dtype == RTG_F64 ? share : 1, static_cast<unsigned>(w.b.n));
   if (w.dtype == RTG_F64) k_gs_pass<double><<<g, GS_THREADS, 0, s>>>(w, 1, o, nullptr);
   else k_gs_pass<float><<<g, GS_THREADS, 0, s>>>(w, 1, o, nullptr);
   return cudaGetLastError();

@@ -950,13 +950,22 @@ k_sk_inner_tc(PtrRef Xr, int in_blocked, float* __restrict__ out, int64_t L, int
   if (dots_pass == 0) {
     if (tid == 0) gs_finish_start<float>(w, o, tot);
   } else {
-    gs_finish_gram_ff(w, o, J, tot, fin_sh, true);
+    gs_finish_gram_ff(w, o, J, tot, fin_sh);
   }
 }
 
 // ------------------------------------------------------------------ CUDA-core chain (FP64)
 
-// Y(l, q, r) = scale * sum_i (-1)^bit(q, i) X(l, i, r)
+// Y(l, q, r) = scale * sum_i (-1)^bit(q, i) X(l, i, r), one thread per entry,
+// added in order.  The chain of additions is what it takes (an FP64 warp
+// instruction occupies its sub-partition for 64 cycles), so the values of 32
+// terms are loaded ahead of it, and blocks of one warp put the warps on as
+// many SMs as there are while they do not fill the GPU.  64 x 64 x 3 to 32 x
+// 32 x 3, both stages: 37 us with blocks of 256 and a load in front of every
+// addition, 15 us.
+__device__ __forceinline__ double flip_sign(double v, uint32_t bit) {   // on the integer pipe
+  return __hiloint2double(__double2hiint(v) ^ static_cast<int>(bit << 31), __double2loint(v));
+}
 template <typename T>
 __global__ void k_sketch_mode(PtrRef Xr, T* __restrict__ Y, int64_t L, int64_t I, int64_t R,
                               int64_t s, const uint32_t* bits, int wpr, T scale,
@@ -973,19 +982,39 @@ __global__ void k_sketch_mode(PtrRef Xr, T* __restrict__ Y, int64_t L, int64_t I
   const int64_t total = L * s * R;
   for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < total;
        o += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t l = o % L;
-    const int64_t q = (o / L) % s;
-    const int64_t r = o / (L * s);
+    int64_t l, q, r;
+    if (total < (int64_t(1) << 31)) {   // 32-bit divisions
+      const uint32_t o32 = static_cast<uint32_t>(o), L32 = static_cast<uint32_t>(L), s32 = static_cast<uint32_t>(s);
+      const uint32_t lq = o32 / L32, rr = lq / s32;
+      l = o32 - lq * L32;
+      q = lq - rr * s32;
+      r = rr;
+    } else {
+      l = o % L;
+      q = (o / L) % s;
+      r = o / (L * s);
+    }
     const T* xp = X + l + L * I * r;
     const uint32_t* brow = bits + q * wpr;
     T acc = 0;
     for (int w = 0; w < wpr; ++w) {
       const uint32_t b = __ldcg(brow + w);
       const int64_t i0 = static_cast<int64_t>(w) * 32;
-      const int cnt = (I - i0) < 32 ? static_cast<int>(I - i0) : 32;
-      for (int u = 0; u < cnt; ++u) {
-        const T x = xp[L * (i0 + u)];
-        acc += ((b >> u) & 1u) ? -x : x;
+      const T* xw = xp + L * i0;
+      if (I - i0 >= 32) {
+        T v[32];
+#pragma unroll
+        for (int u = 0; u < 32; ++u) v[u] = xw[L * u];
+#pragma unroll
+        for (int u = 0; u < 32; ++u) acc += flip_sign(v[u], b >> u);
+      } else {
+        const int cnt = static_cast<int>(I - i0);
+        T v[32];
+#pragma unroll
+        for (int u = 0; u < 32; ++u) v[u] = u < cnt ? xw[L * u] : static_cast<T>(0);
+#pragma unroll
+        for (int u = 0; u < 32; ++u)
+          if (u < cnt) acc += flip_sign(v[u], b >> u);
       }
     }
     Y[o] = acc * scale;
@@ -1023,7 +1052,11 @@ static cudaError_t sketch_f64(const SketchPlan& sp, const SketchScratch& sc, Ptr
     const bool last = (t == sp.nstage - 1);
     double* dst = last ? out : static_cast<double*>((t % 2 == 0) ? sc.tmp0 : sc.tmp1);
     const double scale = last ? sp.scale : 1.0;
-    k_sketch_mode<double><<<dim3(grid_for(sp.stage_out[t]), 1, b.n), 256, 0, s>>>(
+    // (2432 warps: sixteen per SM)
+    const int block = sp.stage_out[t] * b.n <= 2432 * 32 ? 32 : 256;
+    const int64_t want = (sp.stage_out[t] + block - 1) / block;
+    const unsigned grid = static_cast<unsigned>(want < 152 * 32 ? want : 152 * 32);
+    k_sketch_mode<double><<<dim3(grid, 1, b.n), block, 0, s>>>(
         src, dst, sp.stage_L[t], sp.stage_I[t], sp.stage_R[t], sp.stage_s[t],
         sc.bits + sp.word_off[k], sp.wpr[k], scale, stop, b);
     cudaError_t e = cudaGetLastError();

@@ -384,7 +384,6 @@ size_t carve_work(void* mem, int dtype, int64_t n, const SketchPlan& sp, int m, 
   w.U = nU > 0 ? c.take<char>(size_t(nU) * n * ev) : nullptr;
   w.S = c.take<char>(size_t(d) * e);
   w.Spart = c.take<char>(size_t(d) * e);
-  w.nparts = 1;
   void* skmem = c.take<char>(sketch_scratch_bytes(sp));
   *sk = carve_sketch_scratch(sp, skmem);
   w.tmp0 = sk->tmp0;

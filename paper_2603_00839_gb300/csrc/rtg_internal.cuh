@@ -181,8 +181,7 @@ struct Work {
   void* W;                     // n
   void* U;                     // Golub-Kahan: ring of 2 left-basis tensors (else null)
   void* S;                     // d   (sketch of W, then s after the first GS pass)
-  void* Spart;                 // nparts * d partial sketches written by the chain
-  int nparts;
+  void* Spart;                 // d (the sketch, where the chain's last stage does not run the dots)
   void* tmp0;                  // sketch chain intermediates
   void* tmp1;
   void* Q;                     // (m+1) * d sketched basis

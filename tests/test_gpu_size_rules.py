@@ -125,3 +125,41 @@ def test_convolution_gradients_of_unaligned_input(api):
     a = api.conv3x3(x, wt, None, dy=dy)
     b = api.conv3x3(x.clone(), wt, None, dy=dy)
     assert all(torch.equal(p, q) for p, q in zip(a, b))
+
+
+# ------------------------------------------------------------------------ FP64 paths
+
+@pytest.mark.parametrize("dims,radius,mix", [
+    ((1, 1, 3), 1, True),        # one pixel
+    ((31, 5, 3), 9, True),       # a tile and a bit, the largest radius of the small tiles
+    ((33, 4, 2), 4, False),      # two channels: each its own slab
+    ((640, 256, 1), 3, False),   # 160 tiles of 64 x 16: the large tiles
+    ((576, 256, 1), 3, False),   # 144: the small ones
+])
+def test_fp64_apply_tiles(api, h, dims, radius, mix):
+    rng = np.random.default_rng(radius)
+    X, t1, t2 = rng.standard_normal(dims), rng.standard_normal(2 * radius + 1), rng.standard_normal(2 * radius + 1)
+    fac, rfac = [(1, "banded", t1), (2, "banded", t2)], []
+    A, B = [api.banded(1, dims[0], t1), api.banded(2, dims[1], t2)], []
+    if mix:
+        M = rng.standard_normal((3, 3))
+        rfac, B = [(3, "dense", M)], [api.dense(3, M)]
+    ref = oracle.apply_operator(X, oracle.factor_matrices(dims, fac, rfac))
+    got = h.operator_apply(api.to_device(X), A, B)
+    torch.cuda.synchronize()
+    assert _rel(got.cpu().numpy(), ref) < 1e-13
+
+
+@pytest.mark.parametrize("m", [1, 3, 20])
+def test_fp64_gram_schmidt_shared_columns(api, h, m):
+    """Steps whose column count is below, at and above the blocks that share a slice of the sketch."""
+    import workloads as w
+    dims, sk = (70, 50, 3), (20, 20, 3)
+    t = w.gaussian_taps(1.0, 3)
+    fac = [(1, "banded", t), (2, "banded", t)]
+    C = np.random.default_rng(5).standard_normal(dims)
+    mats = oracle.factor_matrices(dims, fac)
+    ref = oracle.rtg_gmres(mats, C, m, oracle.sketch_matrices(dims, sk, 4), lam=1e-2)
+    X, info = h.gmres_solve(api.to_device(C), m, sk, 4, 1e-2, [api.banded(1, 70, t), api.banded(2, 50, t)])
+    assert info.iters == m and np.allclose(info.rho, ref["rho"], rtol=1e-9)
+    assert _rel(X.cpu().numpy(), ref["X"]) < 1e-9
