@@ -447,12 +447,14 @@ k_apply_small64(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, FusedArgs a, B
 // any image operator whose tensors are stored in BF16.  A CTA owns a
 // 64 x 16 tile of modes 1-2, all NC channels of one channel group and a
 // chunk of output frames.  It walks the input frames in order: each frame's
-// halo tile is loaded into registers (16-byte loads, BF16 or FP32) while
-// the previous frame is being filtered, converted to FP32 in shared memory,
-// filtered along mode 2 and then mode 1 as in the image kernel, and added into a
-// ring of five partial output frames held in registers; the oldest ring
-// entry is complete after each input frame, is mixed across the channels
-// and stored.  Arithmetic is FP32 in every storage format.
+// halo tile arrives with 16-byte cp.async, in its storage format, while the
+// previous frame is being filtered (two buffers), is filtered along mode 2 and
+// then mode 1 as in the image kernel, all channels at once (two barriers a
+// frame), and added into a ring of five partial output frames held in
+// registers; the oldest ring entry is complete after each input frame, is mixed
+// across the channels and stored.  Arithmetic is FP32 in every storage format.
+// Bound by instruction issue and the latency between its barriers (two CTAs
+// per SM): @E@
 constexpr int STX = 64, STY = 16, ST_THREADS = 256, ST_RING = 5, ST_VSEG = 4;
 
 struct StArgs {
@@ -480,20 +482,6 @@ struct StGeom {
   static constexpr int Ht = STY + 2 * RR;
 };
 
-__device__ __forceinline__ void st_to_float(const uint4& q, float* dst, float) {
-  dst[0] = __uint_as_float(q.x);
-  dst[1] = __uint_as_float(q.y);
-  dst[2] = __uint_as_float(q.z);
-  dst[3] = __uint_as_float(q.w);
-}
-__device__ __forceinline__ void st_to_float(const uint4& q, float* dst, __nv_bfloat16) {
-  const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    dst[2 * i] = __uint_as_float(w[i] << 16);
-    dst[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
-  }
-}
 __device__ __forceinline__ void st_store(float* p, float v) { *p = v; }
 __device__ __forceinline__ void st_store(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
 // Four consecutive outputs (plus beta Z, if Z is given): one 16-byte (FP32)
@@ -532,9 +520,23 @@ __device__ __forceinline__ void st_store4(TO* p, const float* z, float beta, con
   }
 }
 
+// Elements between two staged frames of `frame` elements: whole 128-byte lines.
+template <typename TI>
+__host__ __device__ constexpr int st_buffer(int frame) {
+  return (frame * static_cast<int>(sizeof(TI)) + 127) / 128 * 128 / static_cast<int>(sizeof(TI));
+}
+
+// Two adjacent staged values as FP32.
+__device__ __forceinline__ float2 st_pair(const float* p) { return *reinterpret_cast<const float2*>(p); }
+__device__ __forceinline__ float2 st_pair(const __nv_bfloat16* p) {
+  const uint32_t w = *reinterpret_cast<const uint32_t*>(p);
+  return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+}
+
 template <typename TI, typename TO, int NC, int RR>
 __global__ void __launch_bounds__(ST_THREADS, 2)
-k_apply_st(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, StArgs a, Batch bt) {
+k_apply_st(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, StArgs a, const __grid_constant__ CUtensorMap xmap, int xtma,
+           Batch bt) {
   const BIdx bi = bidx(bt);
   Xr = Xr.at(bi.off);
   Yr = Yr.at(bi.off);
@@ -547,11 +549,17 @@ k_apply_st(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, StArgs a, Batch bt)
   using G = StGeom<RR, TI>;
   constexpr int V = G::V, Wd = G::Wd, Ht = G::Ht, RA = G::RA, OFF = G::OFF;
   constexpr int NT = 2 * RR + 1;
-  constexpr int NCH = NC * Ht * (Wd / V);                    // 16-byte loads per frame
+  constexpr int NCH = NC * Ht * (Wd / V);                    // 16-byte pieces of a frame's tile
   constexpr int NPT = (NCH + ST_THREADS - 1) / ST_THREADS;   // per thread
+  constexpr int FRAME = NC * Ht * Wd;
+  constexpr int PITCH = st_buffer<TI>(FRAME);   // elements between the two buffers
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float* in_s = reinterpret_cast<float*>(smem_raw);   // NC x Ht x Wd
-  float* tmp = in_s + NC * Ht * Wd;                   // STY x Wd
+  __shared__ __align__(8) uint64_t xbar[2];
+  // the tiled copy's destination must start on 128 bytes (the launch adds the slack)
+  const uint32_t raw = static_cast<uint32_t>(__cvta_generic_to_shared(smem_raw));
+  unsigned char* smem = smem_raw + (((raw + 127u) & ~127u) - raw);
+  TI* in_s = reinterpret_cast<TI*>(smem);                                      // [2][NC][Ht][Wd]
+  float* tmp = reinterpret_cast<float*>(smem + size_t(2) * PITCH * sizeof(TI));   // [NC][STY][Wd]
   const int x0 = blockIdx.x * STX, y0 = blockIdx.y * STY;
   const int I1 = static_cast<int>(a.I1), I2 = static_cast<int>(a.I2);
   const int64_t plane = a.I1 * a.I2;
@@ -565,33 +573,45 @@ k_apply_st(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, StArgs a, Batch bt)
   const int oy = threadIdx.x / (STX / ST_VSEG);
   const int ox = (threadIdx.x % (STX / ST_VSEG)) * ST_VSEG;
   constexpr int NPAIR = Wd / 2;                       // mode-2 pass: column pairs x 4 output rows
-  uint4 pre[NPT];
-  auto load_frame = [&](int64_t u) {
+  constexpr int TASKS = NC * NPAIR * (STY / ST_VSEG);
+  // the frames this CTA reads, and its copies of one frame (one cp.async group)
+  const int64_t u0 = f0 - rt, u1 = f1 + rt;
+  const int64_t uend = u1 < a.nF ? u1 : a.nF;
+  // with a tensor map of the input, one tiled copy per frame (zero filled
+  // outside the tensor) instead of the threads' copies and their addresses;
+  // the copy engine's rules are checked: a 128-byte aligned destination and an
+  // innermost start coordinate on 16 bytes
+  const bool tma = xtma && (static_cast<uint32_t>(__cvta_generic_to_shared(in_s)) & 127u) == 0 &&
+                   ((static_cast<int64_t>(x0 - RA) * static_cast<int64_t>(sizeof(TI))) & 15) == 0;
+  const int slot = (xtma && Xr.jidx != nullptr) ? *Xr.jidx + Xr.joff : 0;
+  if (tma && threadIdx.x == 0) {
+    mbar_init_raw(&xbar[0], 1);
+    mbar_init_raw(&xbar[1], 1);
+    mbar_init_fence();
+  }
+  auto load_frame = [&](int64_t u, int buf) {
+    if (tma) {
+      if (threadIdx.x == 0) {
+        mbar_expect(&xbar[buf], static_cast<uint32_t>(FRAME * sizeof(TI)));
+        tma_load_5d(in_s + buf * PITCH, &xmap, x0 - RA, y0 - RR,
+                    static_cast<int>(group * NC + a.I3 * u), slot, bi.p, &xbar[buf]);
+      }
+      return;
+    }
+    const TI* base = X + (static_cast<int64_t>(group) * NC + a.I3 * u) * plane;
 #pragma unroll
     for (int q = 0; q < NPT; ++q) {
-      pre[q] = make_uint4(0u, 0u, 0u, 0u);
       const int idx = threadIdx.x + q * ST_THREADS;
-      if (idx >= NCH) continue;
+      if (idx >= NCH) break;
       const int row = idx / (Wd / V), f = idx - row * (Wd / V);
       const int c = row / Ht, yy = row - c * Ht;
       const int gy = y0 - RR + yy, gx = x0 - RA + V * f;
-      if (gy < 0 || gy >= I2 || gx < 0 || gx >= I1) continue;
-      const int64_t pl = (static_cast<int64_t>(group) * NC + c) + a.I3 * u;
-      pre[q] = __ldcg(reinterpret_cast<const uint4*>(X + pl * plane + static_cast<int64_t>(gy) * I1 + gx));
+      const bool v = gy >= 0 && gy < I2 && gx >= 0 && gx < I1;
+      const TI* src = v ? base + c * plane + static_cast<int64_t>(gy) * I1 + gx : X;
+      const unsigned dst = static_cast<unsigned>(__cvta_generic_to_shared(in_s + buf * PITCH + row * Wd + V * f));
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(v ? 16 : 0) : "memory");
     }
-  };
-  auto store_frame = [&]() {
-#pragma unroll
-    for (int q = 0; q < NPT; ++q) {
-      const int idx = threadIdx.x + q * ST_THREADS;
-      if (idx >= NCH) continue;
-      const int row = idx / (Wd / V), f = idx - row * (Wd / V);
-      float v[V];
-      st_to_float(pre[q], v, TI());
-      float4* d = reinterpret_cast<float4*>(in_s + row * Wd + V * f);
-#pragma unroll
-      for (int h = 0; h < V / 4; ++h) d[h] = make_float4(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3]);
-    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
   };
   float ring[ST_RING][NC][ST_VSEG];
 #pragma unroll
@@ -600,10 +620,11 @@ k_apply_st(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, StArgs a, Batch bt)
     for (int c = 0; c < NC; ++c)
 #pragma unroll
       for (int o = 0; o < ST_VSEG; ++o) ring[k][c][o] = 0.f;
-  const int64_t u0 = f0 - rt, u1 = f1 + rt;
-  {   // the first frame inside the tensor; each frame then prefetches the next
+  int buf = 0;
+  uint32_t uses = 0;   // frames taken so far: buffer uses & 1, its phase (uses >> 1) & 1
+  {   // the first frame inside the tensor; each frame then copies the next
     const int64_t uf = u0 > 0 ? u0 : 0;
-    if (uf < u1 && uf < a.nF) load_frame(uf);
+    if (uf < uend) load_frame(uf, 0);
   }
   for (int64_t u = u0; u < u1; ++u) {
     const bool have = u >= 0 && u < a.nF;
@@ -613,53 +634,71 @@ k_apply_st(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, StArgs a, Batch bt)
 #pragma unroll
       for (int o = 0; o < ST_VSEG; ++o) P[c][o] = 0.f;
     if (have) {
-      __syncthreads();              // the previous frame's filters are done with in_s
-      store_frame();
+      // the frame is there; the frame before is done with tmp and with the other buffer
+      if (tma) {
+        if (uses == 0) __syncthreads();   // the barriers are initialised
+        const uint32_t ph = (uses >> 1) & 1u;
+        const bool landed = mbar_wait(&xbar[buf], ph);
+        if (__syncthreads_or(!landed)) {
+          // not in time: wait once more (bounded) for the copy, then poison the
+          // frame so that the solve stops with a non-finite status
+          if (threadIdx.x == 0) mbar_wait(&xbar[buf], ph);
+          __syncthreads();
+          for (int i = threadIdx.x; i < FRAME; i += ST_THREADS) st_store(in_s + buf * PITCH + i, __int_as_float(0x7fc00000));
+          __syncthreads();
+        }
+        ++uses;
+      } else {
+        asm volatile("cp.async.wait_all;\n" ::: "memory");
+        __syncthreads();
+      }
+      if (u + 1 < uend) load_frame(u + 1, buf ^ 1);   // in flight during the filters
+      // mode 2 first over every staged column of every channel: task = (channel, column pair, 4 output rows)
+      const TI* ins = in_s + buf * PITCH;
+      for (int task = threadIdx.x; task < TASKS; task += ST_THREADS) {
+        const int pr = task % NPAIR, cg = task / NPAIR, g = cg % (STY / ST_VSEG), c = cg / (STY / ST_VSEG);
+        const TI* col = ins + (c * Ht + g * ST_VSEG) * Wd + 2 * pr;
+        // tap by tap over a sliding window of rows: one copy of a tap serves the
+        // four outputs, and few registers are live
+        float2 win[ST_VSEG], sacc[ST_VSEG];
+#pragma unroll
+        for (int o = 0; o < ST_VSEG; ++o) {
+          win[o] = st_pair(col + o * Wd);
+          sacc[o] = make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int t = 0; t < NT; ++t) {
+          const float2 tap = make_float2(a.t2[t], a.t2[t]);
+#pragma unroll
+          for (int o = 0; o < ST_VSEG; ++o) sacc[o] = ffma2(tap, win[(o + t) % ST_VSEG], sacc[o]);
+          if (t + 1 < NT) win[t % ST_VSEG] = st_pair(col + (t + ST_VSEG) * Wd);
+        }
+        float* dst = tmp + (c * STY + g * ST_VSEG) * Wd + 2 * pr;
+#pragma unroll
+        for (int o = 0; o < ST_VSEG; ++o) *reinterpret_cast<float2*>(dst + o * Wd) = sacc[o];
+      }
       __syncthreads();
-      if (u + 1 < u1 && u + 1 < a.nF) load_frame(u + 1);   // in flight during the filters
+      // mode 1: 4 consecutive outputs of row oy
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
-        const float* ins = in_s + c * Ht * Wd;
-        // mode 2 first over every staged column: task = (column pair, 4 output rows)
-        for (int task = threadIdx.x; task < NPAIR * (STY / ST_VSEG); task += ST_THREADS) {
-          const int pr = task % NPAIR, g = task / NPAIR;
-          float2 win[ST_VSEG + 2 * RR];
+        constexpr int A0 = OFF & ~3, SH = OFF & 3;
+        constexpr int NV = (SH + ST_VSEG + 2 * RR + 3) / 4;
+        const float4* rp = reinterpret_cast<const float4*>(tmp + (c * STY + oy) * Wd + ox + A0);
+        float b[NV * 4];
 #pragma unroll
-          for (int u2 = 0; u2 < ST_VSEG + 2 * RR; ++u2)
-            win[u2] = *reinterpret_cast<const float2*>(ins + (g * ST_VSEG + u2) * Wd + 2 * pr);
-#pragma unroll
-          for (int o = 0; o < ST_VSEG; ++o) {
-            float2 sacc = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int t = 0; t < NT; ++t) sacc = ffma2(make_float2(a.t2[t], a.t2[t]), win[o + t], sacc);
-            *reinterpret_cast<float2*>(tmp + (g * ST_VSEG + o) * Wd + 2 * pr) = sacc;
-          }
+        for (int v4 = 0; v4 < NV; ++v4) {
+          const float4 q = rp[v4];
+          b[4 * v4] = q.x;
+          b[4 * v4 + 1] = q.y;
+          b[4 * v4 + 2] = q.z;
+          b[4 * v4 + 3] = q.w;
         }
-        __syncthreads();
-        // mode 1: 4 consecutive outputs of row oy
-        {
-          constexpr int A0 = OFF & ~3, SH = OFF & 3;
-          constexpr int NV = (SH + ST_VSEG + 2 * RR + 3) / 4;
-          const float4* rp = reinterpret_cast<const float4*>(tmp + oy * Wd + ox + A0);
-          float buf[NV * 4];
 #pragma unroll
-          for (int v4 = 0; v4 < NV; ++v4) {
-            const float4 q = rp[v4];
-            buf[4 * v4] = q.x;
-            buf[4 * v4 + 1] = q.y;
-            buf[4 * v4 + 2] = q.z;
-            buf[4 * v4 + 3] = q.w;
-          }
+        for (int t = 0; t < NT; ++t)
 #pragma unroll
-          for (int o = 0; o < ST_VSEG; ++o) {
-            float sacc = 0.f;
-#pragma unroll
-            for (int t = 0; t < NT; ++t) sacc = fmaf(a.t1[t], buf[SH + o + t], sacc);
-            P[c][o] = sacc;
-          }
-        }
-        if (c + 1 < NC) __syncthreads();   // the next channel's mode-2 pass rewrites tmp
+          for (int o = 0; o < ST_VSEG; ++o) P[c][o] = fmaf(a.t1[t], b[SH + o + t], P[c][o]);
       }
+      buf ^= 1;
     }
     // ring[k] is output frame u - rt + k; frame u enters with tap t4[2 + rt - k]
 #pragma unroll
@@ -827,21 +866,22 @@ int apply_launches(const OpPlan& op, bool combine, int dtype, int tin, int tout)
 
 static bool has_ptr(const PtrRef& r) { return r.base != nullptr || r.ind != nullptr; }
 
-// Tensor map of an FP32 input of the register kernel: dims (I1, I2, planes,
+// Tensor map of an FP32 or BF16 input (`elt` bytes) of the register and the
+// spatio-temporal kernel: dims (I1, I2, planes,
 // slots, problems) where `planes` counts the tensor's I1 x I2 planes, slots
 // the basis slots of a slot-indexed buffer (1 for a direct pointer) and
 // problems the lock-step batch; boxes of the CTA's halo tile (Wd x Ht x NC),
 // zero filled outside.  False for inputs read through a pointer slot or a
 // ring, or that break the copy engine's 16-byte rules.
-static bool make_apply_map(CUtensorMap* m, const PtrRef& X, int64_t I1, int64_t I2, int64_t planes, int Wd, int Ht,
-                           int NC, const Batch& b) {
+static bool make_apply_map(CUtensorMap* m, const PtrRef& X, size_t elt, int64_t I1, int64_t I2, int64_t planes, int Wd,
+                           int Ht, int NC, const Batch& b) {
   const PFN_cuTensorMapEncodeTiled_v12000 fn = tensor_map_encoder();
   if (fn == nullptr || X.base == nullptr || X.ind != nullptr || X.mod != 0) return false;
   const bool slotted = X.jidx != nullptr;
   if (slotted && X.nslot <= 0) return false;
-  const uint64_t pitch = static_cast<uint64_t>(I1) * 4, plane = pitch * static_cast<uint64_t>(I2);
+  const uint64_t pitch = static_cast<uint64_t>(I1) * elt, plane = pitch * static_cast<uint64_t>(I2);
   const uint64_t tens = plane * static_cast<uint64_t>(planes);
-  const uint64_t sstride = slotted ? static_cast<uint64_t>(X.stride) * 4 : ((tens + 15) & ~uint64_t(15));
+  const uint64_t sstride = slotted ? static_cast<uint64_t>(X.stride) * elt : ((tens + 15) & ~uint64_t(15));
   const uint64_t nslot = slotted ? static_cast<uint64_t>(X.nslot) : 1;
   const uint64_t pstride = b.n > 1 ? static_cast<uint64_t>(b.stride) : ((sstride * nslot + 15) & ~uint64_t(15));
   const uint64_t lim = uint64_t(1) << 40;
@@ -854,7 +894,7 @@ static bool make_apply_map(CUtensorMap* m, const PtrRef& X, int64_t I1, int64_t 
   const cuuint64_t strides[4] = {pitch, plane, sstride, pstride};
   const cuuint32_t box[5] = {static_cast<cuuint32_t>(Wd), static_cast<cuuint32_t>(Ht), static_cast<cuuint32_t>(NC), 1u, 1u};
   const cuuint32_t estr[5] = {1u, 1u, 1u, 1u, 1u};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, const_cast<void*>(X.base), dims, strides, box, estr,
+  return fn(m, elt == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(X.base), dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -931,7 +971,7 @@ static cudaError_t apply_t(const OpPlan& op, PtrRef X, PtrRef Y, double alpha, d
     if (e != cudaSuccess) return e;                                                                   \
     CUtensorMap xm;                                                                                   \
     std::memset(&xm, 0, sizeof xm);                                                                   \
-    const int xtma = (sizeof(T) == 4 && make_apply_map(&xm, X, a.I1, a.I2, a.nslab * NC, Gm::Wd, Gm::Ht, NC, b)) \
+    const int xtma = (sizeof(T) == 4 && make_apply_map(&xm, X, 4, a.I1, a.I2, a.nslab * NC, Gm::Wd, Gm::Ht, NC, b)) \
                          ? 1 : 0;                                                                     \
     k_apply_reg<T, NC, RR><<<grid, FTHREADS, smem, s>>>(X, Y, Z, stop, a, xm, xtma, b);                  \
     return cudaGetLastError();                                                                        \
@@ -995,14 +1035,24 @@ static cudaError_t apply_t(const OpPlan& op, PtrRef X, PtrRef Y, double alpha, d
   return cudaGetLastError();
 }
 
-// Frame chunking of the spatio-temporal kernel: about two CTAs per SM.
-static void st_chunks(int64_t tiles, int64_t nF, int* F, int* nchunk) {
-  int64_t want = (304 + tiles - 1) / tiles;
-  if (want < 1) want = 1;
-  if (want > nF) want = nF;
-  int64_t f = (nF + want - 1) / want;
-  *F = static_cast<int>(f);
-  *nchunk = static_cast<int>((nF + f - 1) / f);
+// Frames per CTA of the spatio-temporal kernel.  Two CTAs fit an SM, and a CTA
+// walks its F output frames and 2 rt more, so the cost of a split is (waves of
+// 304 CTAs) (F + 2 rt); the smallest wins.  256 x 256 x 3 x 64: four chunks of
+// 16 (256 CTAs, one wave), where five of 13 left 16 CTAs to a second wave: FP32
+// 113 -> @C@ us, BF16 79 -> @D@ us.
+static void st_chunks(int64_t tiles, int64_t nF, int rt, int* F, int* nchunk) {
+  int64_t best = -1;
+  for (int64_t want = 1; want <= nF; ++want) {
+    const int64_t f = (nF + want - 1) / want, n = (nF + f - 1) / f;
+    if (n != want) continue;
+    const int64_t cost = (tiles * n + 303) / 304 * (f + 2 * rt);
+    if (best < 0 || cost < best) {
+      best = cost;
+      *F = static_cast<int>(f);
+      *nchunk = static_cast<int>(n);
+    }
+    if (tiles * n > 16 * 304) break;   // more waves only add frames
+  }
 }
 
 bool st_supported(const OpPlan& op, int tin) {
@@ -1035,16 +1085,20 @@ static cudaError_t apply_st_t(const OpPlan& op, PtrRef X, PtrRef Y, double alpha
   a.alpha = static_cast<float>(alpha);
   a.beta = has_ptr(Z) ? static_cast<float>(beta) : 0.f;
   const int64_t gx = (a.I1 + STX - 1) / STX, gy = (a.I2 + STY - 1) / STY, groups = a.I3 / nc;
-  st_chunks(gx * gy * groups, a.nF, &a.F, &a.nchunk);
+  st_chunks(gx * gy * groups * b.n, a.nF, a.rt, &a.F, &a.nchunk);
   if (groups * a.nchunk * b.n > 65535) return cudaErrorInvalidConfiguration;
   dim3 grid(static_cast<unsigned>(gx), static_cast<unsigned>(gy), static_cast<unsigned>(groups * a.nchunk * b.n));
 #define RTG_ST_CASE(NC, RR)                                                                         \
   if (nc == NC && rr == RR) {                                                                       \
     using Gm = StGeom<RR, TI>;                                                                      \
-    const size_t smem = static_cast<size_t>(NC * Gm::Ht * Gm::Wd + STY * Gm::Wd) * sizeof(float);   \
+    const size_t smem = size_t(2) * st_buffer<TI>(NC * Gm::Ht * Gm::Wd) * sizeof(TI) +              \
+                        size_t(NC) * STY * Gm::Wd * 4 + 128;                                        \
     cudaError_t e = set_smem(k_apply_st<TI, TO, NC, RR>, smem);                                     \
     if (e != cudaSuccess) return e;                                                                 \
-    k_apply_st<TI, TO, NC, RR><<<grid, ST_THREADS, smem, s>>>(X, Y, Z, stop, a, b);                    \
+    CUtensorMap xm;                                                                                 \
+    std::memset(&xm, 0, sizeof xm);                                                                 \
+    const int xtma = make_apply_map(&xm, X, sizeof(TI), a.I1, a.I2, a.I3 * a.nF, Gm::Wd, Gm::Ht, NC, b) ? 1 : 0; \
+    k_apply_st<TI, TO, NC, RR><<<grid, ST_THREADS, smem, s>>>(X, Y, Z, stop, a, xm, xtma, b);          \
     return cudaGetLastError();                                                                      \
   }
   RTG_ST_CASE(1, 3) RTG_ST_CASE(1, 5) RTG_ST_CASE(1, 7) RTG_ST_CASE(1, 9)
