@@ -128,14 +128,16 @@ k_apply_fused(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, FusedArgs a, Bat
 // to 2*RR+1) and NC jointly mixed channels.  Tile 64 x 16 of modes 1-2,
 // 256 threads.  All NC halo tiles are staged in shared memory at once with
 // cp.async (zero fill outside the tensor: the zero boundary of Eq. 57), so
-// the CTA waits on global memory once.  Per channel the mode-2 filter runs
-// first, over the 16 output rows and every staged column (a task: two
-// adjacent columns x 4 rows, paired FP32 FMAs), then the mode-1 filter over
-// the 16 x 64 outputs (a thread: 4 consecutive outputs of one row from a
+// the CTA waits on global memory once.  The mode-2 filter runs
+// first, over the 16 output rows and every staged column of all channels (a
+// task: two adjacent columns x 4 rows, paired FP32 FMAs), then the mode-1 filter
+// over the 16 x 64 outputs (a thread: 4 consecutive outputs of one row from a
 // register window of 4+2RR values): filtering the halo rows along mode 2
 // first costs 16 (64 + 2RR) + 16 x 64 products per tap instead of
 // (16 + 2RR) 64 + 16 x 64, and the thread's 4 outputs leave in one 16-byte
-// store after the channel mix.
+// store after the channel mix.  Bound by the latency of its few phases:
+// 1024 x 1024 x 3, radius 7, 12.7 us with both filters channel by channel (six
+// barriers), 12.1 us (cold caches).
 constexpr int RTX = 64;
 constexpr int RTY = 16;
 
@@ -201,7 +203,7 @@ k_apply_reg(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, FusedArgs a,
   constexpr int NPAIR = Wd / 2;                 // mode-2 pass: column pairs
   constexpr int V2 = 4;                          // mode-2 pass: output rows per task
   constexpr int M1 = 4;                          // mode-1 pass: outputs per thread
-  static_assert(Wd % 2 == 0 && NPAIR * (RTY / V2) <= 2 * FTHREADS, "mode-2 tasks");
+  static_assert(Wd % 2 == 0, "mode-2 tasks");
   static_assert(RTY * (RTX / M1) == FTHREADS, "mode-1 tasks: one per thread");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t xbar;
@@ -209,7 +211,7 @@ k_apply_reg(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, FusedArgs a,
   // there explicitly (the launch adds 128 bytes of slack)
   const uint32_t raw = static_cast<uint32_t>(__cvta_generic_to_shared(smem_raw));
   T* in_s = reinterpret_cast<T*>(smem_raw + (((raw + 127u) & ~127u) - raw));   // NC x Ht x Wd
-  T* tmp = in_s + NC * Ht * Wd;                  // RTY x Wd
+  T* tmp = in_s + NC * Ht * Wd;                  // NC x RTY x Wd
   const int x0 = blockIdx.x * RTX;
   const int y0 = blockIdx.y * RTY;
   const int I1 = static_cast<int>(a.I1), I2 = static_cast<int>(a.I2);
@@ -269,67 +271,68 @@ k_apply_reg(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, FusedArgs a,
     }
     asm volatile("cp.async.wait_all;\n" ::: "memory");
     __syncthreads();
+    // mode 2 first (along y, all Wd staged columns of all channels): task =
+    // (channel, column pair, 4 output rows), paired FMAs over the two columns, tap
+    // by tap over a sliding window of rows: one copy of a tap serves the four outputs
+    for (int task = threadIdx.x; task < NC * NPAIR * (RTY / V2); task += FTHREADS) {
+      const int pr = task % NPAIR, cg = task / NPAIR, g = cg % (RTY / V2), c = cg / (RTY / V2);
+      const T* col = in_s + (c * Ht + g * V2) * Wd + 2 * pr;
+      Pair<T> win[V2], s[V2];
+#pragma unroll
+      for (int o = 0; o < V2; ++o) {
+        win[o] = load_pair(col + o * Wd);
+        s[o] = {static_cast<T>(0), static_cast<T>(0)};
+      }
+#pragma unroll
+      for (int t = 0; t < NT; ++t) {
+#pragma unroll
+        for (int o = 0; o < V2; ++o) s[o] = pfma(t2(t), win[(o + t) % V2], s[o]);
+        if (t + 1 < NT) win[t % V2] = load_pair(col + (t + V2) * Wd);
+      }
+      T* q = tmp + (c * RTY + g * V2) * Wd + 2 * pr;
+#pragma unroll
+      for (int o = 0; o < V2; ++o) {
+        if constexpr (sizeof(T) == 4) {
+          *reinterpret_cast<float2*>(q + o * Wd) = make_float2(s[o].x, s[o].y);
+        } else {
+          q[o * Wd] = s[o].x;
+          q[o * Wd + 1] = s[o].y;
+        }
+      }
+    }
+    __syncthreads();
+    // mode 1 (along x): 4 consecutive outputs of one row per thread and channel
     T acc[NC][M1];
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-      const T* ins = in_s + c * Ht * Wd;
-      // mode 2 first (along y, all Wd staged columns): task = (column pair,
-      // 4 output rows), paired FMAs over the two columns
-      for (int task = threadIdx.x; task < NPAIR * (RTY / V2); task += FTHREADS) {
-        const int pr = task % NPAIR, g = task / NPAIR;
-        Pair<T> win[V2 + 2 * RR];
 #pragma unroll
-        for (int u = 0; u < V2 + 2 * RR; ++u) {
-          win[u] = load_pair(ins + (g * V2 + u) * Wd + 2 * pr);
+      for (int o = 0; o < M1; ++o) acc[c][o] = 0;
+      T win[M1 + 2 * RR];
+      if (sizeof(T) == 4) {
+        // aligned 16-byte loads covering the window, which starts OFF & 3 floats in
+        constexpr int A0 = OFF & ~3, SH = OFF & 3;
+        constexpr int NV = (SH + M1 + 2 * RR + 3) / 4;
+        const float4* rp = reinterpret_cast<const float4*>(tmp + (c * RTY + oy) * Wd + ox + A0);
+        float buf[NV * 4];
+#pragma unroll
+        for (int v4 = 0; v4 < NV; ++v4) {
+          const float4 q = rp[v4];
+          buf[4 * v4] = q.x;
+          buf[4 * v4 + 1] = q.y;
+          buf[4 * v4 + 2] = q.z;
+          buf[4 * v4 + 3] = q.w;
         }
 #pragma unroll
-        for (int o = 0; o < V2; ++o) {
-          Pair<T> s{static_cast<T>(0), static_cast<T>(0)};
+        for (int u = 0; u < M1 + 2 * RR; ++u) win[u] = static_cast<T>(buf[SH + u]);
+      } else {
+        const T* row = tmp + (c * RTY + oy) * Wd + ox + OFF;
 #pragma unroll
-          for (int t = 0; t < NT; ++t) s = pfma(t2(t), win[o + t], s);
-          T* q = tmp + (g * V2 + o) * Wd + 2 * pr;
-          if constexpr (sizeof(T) == 4) {
-            *reinterpret_cast<float2*>(q) = make_float2(s.x, s.y);
-          } else {
-            q[0] = s.x;
-            q[1] = s.y;
-          }
-        }
+        for (int u = 0; u < M1 + 2 * RR; ++u) win[u] = row[u];
       }
-      __syncthreads();
-      // mode 1 (along x): 4 consecutive outputs of one row per thread
-      {
-        T win[M1 + 2 * RR];
-        if (sizeof(T) == 4) {
-          // aligned 16-byte loads covering the window, which starts OFF & 3 floats in
-          constexpr int A0 = OFF & ~3, SH = OFF & 3;
-          constexpr int NV = (SH + M1 + 2 * RR + 3) / 4;
-          const float4* rp = reinterpret_cast<const float4*>(tmp + oy * Wd + ox + A0);
-          float buf[NV * 4];
 #pragma unroll
-          for (int v4 = 0; v4 < NV; ++v4) {
-            const float4 q = rp[v4];
-            buf[4 * v4] = q.x;
-            buf[4 * v4 + 1] = q.y;
-            buf[4 * v4 + 2] = q.z;
-            buf[4 * v4 + 3] = q.w;
-          }
+      for (int t = 0; t < NT; ++t)
 #pragma unroll
-          for (int u = 0; u < M1 + 2 * RR; ++u) win[u] = static_cast<T>(buf[SH + u]);
-        } else {
-          const T* row = tmp + oy * Wd + ox + OFF;
-#pragma unroll
-          for (int u = 0; u < M1 + 2 * RR; ++u) win[u] = row[u];
-        }
-#pragma unroll
-        for (int o = 0; o < M1; ++o) {
-          T sacc = 0;
-#pragma unroll
-          for (int t = 0; t < NT; ++t) sacc += t1(t) * win[o + t];
-          acc[c][o] = sacc;
-        }
-      }
-      __syncthreads();
+        for (int o = 0; o < M1; ++o) acc[c][o] += t1(t) * win[o + t];
     }
     const int gy = y0 + oy;
     if (gy < I2) {
@@ -454,7 +457,11 @@ k_apply_small64(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, FusedArgs a, B
 // registers; the oldest ring entry is complete after each input frame, is mixed
 // across the channels and stored.  Arithmetic is FP32 in every storage format.
 // Bound by instruction issue and the latency between its barriers (two CTAs
-// per SM): @E@
+// per SM).  256 x 256 x 3 x 64, radius 6, four chunks (cold caches), FP32 / BF16:
+// frames through registers and eight barriers a frame 89 / 65 us; cp.async, two
+// barriers 86 / 67; filters tap by tap (a tap's copies were a third of the
+// instructions) 62 / 56; one tiled TMA copy per frame where the input has a
+// tensor map (the copies' addresses were another quarter) 50 / 50.
 constexpr int STX = 64, STY = 16, ST_THREADS = 256, ST_RING = 5, ST_VSEG = 4;
 
 struct StArgs {
@@ -966,7 +973,7 @@ static cudaError_t apply_t(const OpPlan& op, PtrRef X, PtrRef Y, double alpha, d
 #define RTG_REG_CASE(NC, RR)                                                                          \
   if (a.nc == NC && rr == RR) {                                                                       \
     using Gm = RegGeom<RR, T>;                                                                        \
-    const size_t smem = static_cast<size_t>(NC * Gm::Ht * Gm::Wd + RTY * Gm::Wd) * sizeof(T) + 128;   \
+    const size_t smem = static_cast<size_t>(NC) * (Gm::Ht + RTY) * Gm::Wd * sizeof(T) + 128;             \
     e = set_smem(k_apply_reg<T, NC, RR>, smem);                                                       \
     if (e != cudaSuccess) return e;                                                                   \
     CUtensorMap xm;                                                                                   \
@@ -1039,7 +1046,7 @@ static cudaError_t apply_t(const OpPlan& op, PtrRef X, PtrRef Y, double alpha, d
 // walks its F output frames and 2 rt more, so the cost of a split is (waves of
 // 304 CTAs) (F + 2 rt); the smallest wins.  256 x 256 x 3 x 64: four chunks of
 // 16 (256 CTAs, one wave), where five of 13 left 16 CTAs to a second wave: FP32
-// 113 -> @C@ us, BF16 79 -> @D@ us.
+// 113 -> 89 us, BF16 79 -> 65 us.
 static void st_chunks(int64_t tiles, int64_t nF, int rt, int* F, int* nchunk) {
   int64_t best = -1;
   for (int64_t want = 1; want <= nF; ++want) {
