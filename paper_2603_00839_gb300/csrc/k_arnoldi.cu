@@ -170,8 +170,9 @@ __global__ void k_update(Work w0, StepOpts o0) {
     return;
   }
   if (ctl->skip_update || ctl->j == 0) return;
-  // lock-step batch: a problem that stopped in an earlier body has nothing to update
-  if (o.group_left != nullptr && ctl->stop && !ctl->givens) return;
+  // a problem that stopped in an earlier step (lock-step batch, two steps a
+  // loop body) has nothing to update
+  if (o.solve_mode && ctl->stop && !ctl->givens) return;
   const int jj = ctl->j;
   if (jj > w.m) {   // V holds m+1 tensors: never write past V_m
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -410,7 +411,7 @@ __global__ void k_update_bf16(Work w0, StepOpts o0) {
     return;
   }
   if (ctl->skip_update || ctl->j == 0) return;
-  if (o.group_left != nullptr && ctl->stop && !ctl->givens) return;
+  if (o.solve_mode && ctl->stop && !ctl->givens) return;
   const int jj = ctl->j;
   if (jj > w.m) {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -523,7 +524,7 @@ __global__ void __launch_bounds__(UP_THREADS) k_update_ring(Work w0, StepOpts o0
     return;
   }
   if (ctl->skip_update || ctl->j == 0) return;
-  if (o.group_left != nullptr && ctl->stop && !ctl->givens) return;
+  if (o.solve_mode && ctl->stop && !ctl->givens) return;
   const int jj = ctl->j;
   if (jj > w.m) {   // V holds m+1 tensors: never write past V_m
     if (blockIdx.x == 0 && threadIdx.x == 0) {

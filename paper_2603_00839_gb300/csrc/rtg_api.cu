@@ -940,9 +940,10 @@ rtg_status add_conditional(cudaStream_t cs, cudaGraphConditionalHandle hnd, cuda
 
 // Captures P's solve (prologue, a WHILE node over one Arnoldi step, epilogue)
 // on `cs`, which is capturing into graph g; cs2 captures the loop's body.
-// The loop's condition handle goes to *loop when loop is not null.
+// The loop's condition handle goes to *loop when loop is not null.  The body
+// holds `steps` Arnoldi steps; kernels of a step after the stop return at once.
 rtg_status capture_solve(SolvePlan& P, cudaGraph_t g, cudaStream_t cs, cudaStream_t cs2,
-                         cudaGraphConditionalHandle* loop = nullptr) {
+                         cudaGraphConditionalHandle* loop = nullptr, int steps = 1) {
   cudaGraphConditionalHandle hnd;
   CK(cudaGraphConditionalHandleCreate(&hnd, g, 1, cudaGraphCondAssignDefault));
   if (loop) *loop = hnd;
@@ -959,8 +960,10 @@ rtg_status capture_solve(SolvePlan& P, cudaGraph_t g, cudaStream_t cs, cudaStrea
     so.rs_cond = static_cast<unsigned long long>(rh);
   }
   CK(cudaStreamBeginCaptureToGraph(cs2, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-  rtg_status st = P.method == 1 ? enqueue_gk_step(P, so, cs2)
-                                : enqueue_step(P.op, P.sp, P.w, P.dtype, P.tA, P.tB, P.sk, so, cs2);
+  rtg_status st = RTG_OK;
+  for (int q = 0; q < steps && st == RTG_OK; ++q)
+    st = P.method == 1 ? enqueue_gk_step(P, so, cs2)
+                       : enqueue_step(P.op, P.sp, P.w, P.dtype, P.tA, P.tB, P.sk, so, cs2);
   if (st == RTG_OK && P.w.cycles > 1) st = capture_restart_if(P, so, cs2);
   cudaGraph_t bodyout = nullptr;
   const cudaError_t e = cudaStreamEndCapture(cs2, &bodyout);
@@ -1020,11 +1023,11 @@ rtg_status branch_tail(cudaStream_t cs, const ChainLink& ch, rtg_status st) {
 }
 
 // Captures P's solve into g as a branch (after ch.after, if given).
-rtg_status build_branch(SolvePlan& P, cudaGraph_t g, const ChainLink& ch = ChainLink{}) {
+rtg_status build_branch(SolvePlan& P, cudaGraph_t g, const ChainLink& ch = ChainLink{}, int steps = 1) {
   CaptureStreams cs;
   RK(cs.create());
   RK(begin_branch(cs.s[0], g, ch));
-  return end_capture(cs.s[0], branch_tail(cs.s[0], ch, capture_solve(P, g, cs.s[0], cs.s[1])));
+  return end_capture(cs.s[0], branch_tail(cs.s[0], ch, capture_solve(P, g, cs.s[0], cs.s[1], nullptr, steps)));
 }
 
 // A branch of a work-queue batch: it takes a problem of its class, then
@@ -1063,7 +1066,14 @@ rtg_status build_queue_branch(SolvePlan& P, cudaGraph_t g, QueueArgs q, const Ch
 rtg_status build_graph(SolvePlan& P) {
   cudaGraph_t g = nullptr;
   CK(cudaGraphCreate(&g, 0));
-  const rtg_status st = build_branch(P, g);
+  // Two steps a body where a solve may take many: starting a WHILE body again
+  // costs 4 to 5 us, the idle kernels of a half-used last body about 15, so
+  // from 8 steps on (odd stops included) the pair wins.  1024 x 1024, 12 steps:
+  // 902 -> 875 us; 333 x 517, 20 steps: 1013 -> 977; at 5 to 7 steps no
+  // difference.  Batches keep one step (their branches fill each other's
+  // gaps: 48 problems took 3769 us both ways), and so do restarted solves,
+  // whose restart stands at the end of each body.
+  const rtg_status st = build_branch(P, g, ChainLink{}, P.w.cycles == 1 && P.w.m >= 8 ? 2 : 1);
   if (st != RTG_OK) {
     cudaGraphDestroy(g);
     return st;

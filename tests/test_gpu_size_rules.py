@@ -163,3 +163,29 @@ def test_fp64_gram_schmidt_shared_columns(api, h, m):
     X, info = h.gmres_solve(api.to_device(C), m, sk, 4, 1e-2, [api.banded(1, 70, t), api.banded(2, 50, t)])
     assert info.iters == m and np.allclose(info.rho, ref["rho"], rtol=1e-9)
     assert _rel(X.cpu().numpy(), ref["X"]) < 1e-9
+
+
+# ------------------------------------------------------------------------ steps per loop body
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("m,stop_at", [(7, 0), (8, 0), (9, 0), (12, 5), (12, 6), (13, 1)])
+def test_two_steps_a_loop_body_equal_direct_launches(api, h, dtype, m, stop_at):
+    """A stop (tolerance or m) in the first or the second step of a body gives
+    the solve that launches step by step: the same bits."""
+    rng = np.random.default_rng(m)
+    dims = (40, 36)
+    t = np.array([0.2, 1.0, 0.3])
+    A, B = [api.banded(1, 40, t), api.banded(2, 36, t)], [api.banded(2, 36, np.array([0.1, 1.0, 0.2]))]
+    Cd = api.to_device(np.asfortranarray(rng.standard_normal(dims).astype(dtype)))
+    for solve in (h.gmres_solve, h.gk_solve):
+        kw = dict(A_factors=A, B_factors=B)
+        X, r = solve(Cd, m, (20, 18), 3, 0.0, use_graph=False, **kw)
+        tol = 0.0
+        if stop_at:
+            assert r.iters == m
+            tol = float(r.rho[stop_at - 1]) * (1 + 1e-9)
+            X, r = solve(Cd, m, (20, 18), 3, 0.0, use_graph=False, tol=tol, **kw)
+            assert r.iters == stop_at
+        Xg, g = solve(Cd, m, (20, 18), 3, 0.0, tol=tol, **kw)
+        assert (g.iters, g.converged, g.breakdown) == (r.iters, r.converged, r.breakdown)
+        assert torch.equal(Xg, X) and np.array_equal(g.rho, r.rho)
