@@ -10,11 +10,25 @@ from __future__ import annotations
 
 import ctypes as C
 import dataclasses
+import struct
 from typing import List, Optional, Sequence, Tuple
 
 import numpy as np
 
 from . import _lib as L
+
+# The ABI's records as one struct format each (native sizes and alignment).  A
+# record filled field by field through ctypes costs 0.2 to 1.5 us a field on a
+# Grace core, packed whole about 0.5: 48 problems of 512 x 512 spent 1.1 ms of
+# 3.7 in marshalling beside 2.4 on the device, and 0.4 ms so.
+_FACTOR = struct.Struct("iiiiPP")
+_OPTS = struct.Struct("dPiidiiii")
+_PROBLEM = struct.Struct("PiPi4xi4qPPPii4qQdd")
+_INFO = struct.Struct(f"4i3dPP2d3i{L.PHASE_COUNT}d{L.PHASE_COUNT}id")
+_INFO_PTRS = struct.Struct("PP")   # rho_hist, gcv
+assert (_FACTOR.size, _OPTS.size, _PROBLEM.size, _INFO.size) == (
+    C.sizeof(L.Factor), C.sizeof(L.Opts), C.sizeof(L.Problem), C.sizeof(L.Info))
+assert L.Info.gcv.offset == L.Info.rho_hist.offset + C.sizeof(C.c_void_p)
 
 __all__ = ["Handle", "Factor", "banded", "dense", "identity", "empty", "to_device",
            "colmajor_strides", "SolveResult", "Krylov"]
@@ -37,8 +51,8 @@ def empty(dims: Sequence[int], dtype=None, device="cuda"):
     """Uninitialised column-major tensor of shape ``dims`` on ``device``."""
     torch = _torch()
     dtype = dtype or torch.float32
-    rev = tuple(int(d) for d in reversed(dims))
-    return torch.empty(rev, dtype=dtype, device=device).permute(*reversed(range(len(dims))))
+    dims = tuple(int(d) for d in dims)
+    return torch.empty_strided(dims, colmajor_strides([max(d, 1) for d in dims]), dtype=dtype, device=device)
 
 
 def to_device(a: np.ndarray, dtype=None, device="cuda"):
@@ -107,24 +121,83 @@ def identity(mode: int, n: int) -> Factor:
     return Factor(mode, L.FACTOR_IDENTITY, n)
 
 
-def _factor_array(fs: Sequence[Factor]):
-    arr = (L.Factor * max(len(fs), 1))()
-    keep = []
-    for i, f in enumerate(fs):
-        arr[i].mode, arr[i].kind, arr[i].n, arr[i].radius = f.mode, f.kind, f.n, f.radius
-        if f.taps is not None:
-            arr[i].taps = f.taps.ctypes.data_as(C.POINTER(C.c_double))
-            keep.append(f.taps)
-        if f.matrix is not None:
-            m = np.ascontiguousarray(f.matrix.ravel(order="F"))
-            keep.append(m)
-            arr[i].dense = m.ctypes.data_as(C.POINTER(C.c_double))
-    return (arr if fs else None), len(fs), keep
+_ZEROS = (0,) * L.MAX_ORDER
+
+
+def _address(a: np.ndarray) -> int:
+    return a.ctypes.data
+
+
+# Values of a dense factor up to this many are copied beside the taps; above, the
+# factor's own memory is passed (the copy of a 64 x 64 matrix costs as much as
+# asking numpy for its address).
+_COPY_VALUES = 4096
+
+
+def _factor_arrays(*lists: Sequence[Factor]):
+    """ABI records of several factor lists: ([array or None per list], what
+    they point to).  Taps and small matrices are copied into one buffer: one
+    address to ask for instead of one a factor."""
+    vals, keep, recs, off = [], [], [], 0
+    for fs in lists:
+        for f in fs:
+            taps, mat, t, d, r = f.taps, f.matrix, 0, 0, 0
+            if taps is not None:
+                vals.append(taps)
+                r = (len(taps) - 1) // 2
+                t = off + 1
+                off += len(taps)
+            if mat is not None:
+                v = mat.ravel(order="F")
+                if v.size <= _COPY_VALUES:
+                    vals.append(v)
+                    d = off + 1
+                    off += v.size
+                else:
+                    v = np.ascontiguousarray(v, dtype=np.float64)
+                    keep.append(v)
+                    d = -_address(v)
+            recs.append((f.mode, f.kind, f.n, r, t, d))
+    base = 0
+    if vals:
+        buf = np.concatenate(vals, dtype=np.float64) if off else np.zeros(1)
+        keep.append(buf)
+        base = _address(buf) - 8
+    arrays, k = [], 0
+    for fs in lists:
+        n = len(fs)
+        arr = (L.Factor * n)() if n else None
+        for i in range(n):
+            mode, kind, fn, r, t, d = recs[k + i]
+            _FACTOR.pack_into(arr, i * _FACTOR.size, mode, kind, fn, r, base + 8 * t if t else 0,
+                              base + 8 * d if d > 0 else -d)
+        k += n
+        arrays.append(arr)
+    return arrays, keep
+
+
+def _solve_opts(tol, mu_grid, max_restarts, breakdown_tol, flags, slot=0, group_max=0, queue_slots=0):
+    """rtg_opts and the mu grid it points to (None: none)."""
+    opts = L.Opts()
+    grid = None if mu_grid is None else np.ascontiguousarray(mu_grid, dtype=np.float64)
+    _OPTS.pack_into(opts, 0, float(tol), 0 if grid is None else _address(grid), 0 if grid is None else len(grid),
+                    int(max_restarts), float(breakdown_tol), flags, int(slot), int(group_max), int(queue_slots))
+    return opts, grid
+
+
+def _solve_info(m: int, cycles: int):
+    """rtg_info with room for its histories: (info, rho, gcv)."""
+    info = L.Info()
+    rho = np.zeros(m * cycles + 1 + L.MAX_MU)
+    at = _address(rho)
+    _INFO_PTRS.pack_into(info, L.Info.rho_hist.offset, at, at + 8 * (m * cycles + 1))
+    return info, rho[:m * cycles + 1], rho[m * cycles + 1:]
 
 
 def _stream(stream) -> Optional[int]:
     if stream is None:
-        return _torch().cuda.current_stream().cuda_stream
+        torch = _torch()   # the handle of current_stream(), without the Stream object (3 us)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return getattr(stream, "cuda_stream", stream)
 
 
@@ -196,9 +269,8 @@ class Handle:
         if Y is None:
             Y = empty(dims, X.dtype, X.device)
         _check_tensor(Y, dims, "Y")
-        a, na, ka = _factor_array(A_factors)
-        b, nb, kb = _factor_array(B_factors)
-        L.check(self.lib.rtg_operator_apply(self._h, a, na, b, nb, _shape(dims), _dtype_code(X),
+        (a, b), keep = _factor_arrays(A_factors, B_factors)
+        L.check(self.lib.rtg_operator_apply(self._h, a, len(A_factors), b, len(B_factors), _shape(dims), _dtype_code(X),
                                             X.data_ptr(), Y.data_ptr(), _stream(stream)))
         return Y
 
@@ -247,33 +319,16 @@ class Handle:
         _check_tensor(C_obs, dims, "C")
         if X is None:
             X = empty(dims, C_obs.dtype, C_obs.device)
-        a, na, ka = _factor_array(A_factors)
-        b, nb, kb = _factor_array(B_factors)
+        (a, b), keep = _factor_arrays(A_factors, B_factors)
         sk = (C.c_int64 * len(dims))(*[int(s) for s in sketch_dims])
-        opts = L.Opts()
-        opts.tol = float(tol)
-        grid = None
-        if mu_grid is not None:
-            grid = np.ascontiguousarray(mu_grid, dtype=np.float64)
-            opts.mu_grid = grid.ctypes.data_as(C.POINTER(C.c_double))
-            opts.n_mu = len(grid)
-        opts.breakdown_tol = float(breakdown_tol)
-        opts.flags = ((0 if use_graph else L.FLAG_NO_GRAPH) | (L.FLAG_PHASE_TIMES if phase_times else 0)
-                      | (L.FLAG_TRUE_RESIDUAL if true_residual else 0))
-        opts.slot = int(slot)
-        info = L.Info()
-        rho = np.zeros(m + 1)
-        info.rho_hist = rho.ctypes.data_as(C.POINTER(C.c_double))
-        gcv = np.zeros(L.MAX_MU)
-        info.gcv = gcv.ctypes.data_as(C.POINTER(C.c_double))
-        L.check(self.lib.rtg_gk_solve(self._h, a, na, b, nb, _shape(dims), _dtype_code(C_obs), _ptr(C_obs),
+        flags = ((0 if use_graph else L.FLAG_NO_GRAPH) | (L.FLAG_PHASE_TIMES if phase_times else 0)
+                 | (L.FLAG_TRUE_RESIDUAL if true_residual else 0))
+        opts, grid = _solve_opts(tol, mu_grid, 0, breakdown_tol, flags, slot)
+        info, rho, gcv = _solve_info(m, 1)
+        L.check(self.lib.rtg_gk_solve(self._h, a, len(A_factors), b, len(B_factors), _shape(dims), _dtype_code(C_obs), _ptr(C_obs),
                                       int(m), sk, C.c_uint64(seed), float(lam), _ptr(X0), _ptr(X),
                                       C.byref(opts), C.byref(info), _stream(stream)))
-        res = _solve_result(info, rho, gcv, grid, lam)
-        if phase_times:
-            res.phase_ms = {k: info.phase_ms[i] for i, k in enumerate(L.PHASES)}
-            res.phase_launches = {k: info.phase_launches[i] for i, k in enumerate(L.PHASES)}
-        return X, res
+        return X, _solve_result(_INFO.unpack(info), rho, gcv, grid, lam, phase_times)
 
     def gmres_submit(self, C_obs, m: int, sketch_dims: Sequence[int], seed: int, lam: float,
                      A_factors: Sequence[Factor] = (), B_factors: Sequence[Factor] = (),
@@ -297,28 +352,18 @@ class Handle:
             dt = _dtype_code(C_obs)
             if X is None:
                 X = empty(dims, C_obs.dtype, C_obs.device)
-        a, na, ka = _factor_array(A_factors)
-        b, nb, kb = _factor_array(B_factors)
+        (a, b), keep = _factor_arrays(A_factors, B_factors)
         sk = (C.c_int64 * len(dims))(*[int(s) for s in sketch_dims])
-        opts = L.Opts()
-        opts.tol = float(tol)
-        grid = None
-        if mu_grid is not None:
-            grid = np.ascontiguousarray(mu_grid, dtype=np.float64)
-            opts.mu_grid = grid.ctypes.data_as(C.POINTER(C.c_double))
-            opts.n_mu = len(grid)
-        opts.max_restarts = int(max_restarts)
-        opts.breakdown_tol = float(breakdown_tol)
-        opts.flags = ((0 if use_graph else L.FLAG_NO_GRAPH) | (L.FLAG_PHASE_TIMES if phase_times else 0)
-                      | (L.FLAG_BF16_BASIS if bf16_basis else 0)
-                      | (L.FLAG_TRUE_RESIDUAL if true_residual else 0))
-        opts.slot = int(slot)
-        L.check(self.lib.rtg_gmres_submit(self._h, a, na, b, nb, _shape(dims), dt, _ptr(C_obs), int(m),
+        flags = ((0 if use_graph else L.FLAG_NO_GRAPH) | (L.FLAG_PHASE_TIMES if phase_times else 0)
+                 | (L.FLAG_BF16_BASIS if bf16_basis else 0)
+                 | (L.FLAG_TRUE_RESIDUAL if true_residual else 0))
+        opts, grid = _solve_opts(tol, mu_grid, max_restarts, breakdown_tol, flags, slot)
+        L.check(self.lib.rtg_gmres_submit(self._h, a, len(A_factors), b, len(B_factors), _shape(dims), dt, _ptr(C_obs), int(m),
                                           sk, C.c_uint64(seed), float(lam), _ptr(X0), _ptr(X),
                                           C.byref(opts), _stream(stream)))
         # the host arrays (C, X0, X) and factor arrays stay referenced until the wait
         return PendingSolve(int(slot), X, m, max_restarts, grid, lam, phase_times,
-                            (C_obs, X0, a, b, ka, kb, sk))
+                            (C_obs, X0, a, b, keep, sk))
 
     def gmres_solve_batched(self, problems: Sequence[dict], mu_grid=None, breakdown_tol: float = 0.0,
                             bf16_basis: bool = False, use_graph: bool = True, phase_times: bool = False,
@@ -338,85 +383,74 @@ class Handle:
         Returns ([X], [SolveResult])."""
         if not problems:
             raise ValueError("no problems")
-        arr = (L.Problem * len(problems))()
-        keep = []
-        Xs = []
-        dt = _dtype_code(problems[0]["C"])
+        n = len(problems)
+        cycles = int(max_restarts) + 1
+        arr = (L.Problem * n)()
+        infos = (L.Info * n)()
+        Xs, rows, room = [], [], 0
+        dt, dtype = _dtype_code(problems[0]["C"]), problems[0]["C"].dtype
+        lists = [q.get(k, ()) for q in problems for k in ("A", "B")]
+        factors, keep = _factor_arrays(*lists)
         for i, q in enumerate(problems):
             Cq = q["C"]
             dims = tuple(Cq.shape)
             _check_tensor(Cq, dims, "C")
-            if _dtype_code(Cq) != dt:
+            if Cq.dtype != dtype:
+                _dtype_code(Cq)
                 raise ValueError("all problems of a batch share one dtype")
             X = q.get("X")
             if X is None:
                 X = empty(dims, Cq.dtype, Cq.device)
             _check_tensor(X, dims, "X")
-            a, na, ka = _factor_array(q.get("A", ()))
-            b, nb, kb = _factor_array(q.get("B", ()))
-            keep.append((a, b, ka, kb, q.get("X0")))
-            pr = arr[i]
-            pr.A_factors, pr.nA, pr.B_factors, pr.nB = a, na, b, nb
-            pr.shape = _shape(dims)
-            pr.C, pr.X0, pr.X = _ptr(Cq), _ptr(q.get("X0")), _ptr(X)
-            pr.m = int(q["m"])
-            for k, sdim in enumerate(q["sketch_dims"]):
-                pr.sketch_dims[k] = int(sdim)
-            pr.seed = int(q["seed"])
-            pr.lam = float(q["lam"])
-            pr.tol = float(q.get("tol", 0.0))
+            order = len(dims)
+            if not 1 <= order <= L.MAX_ORDER:
+                raise ValueError("order must be 1..4")
+            sd = [int(sdim) for sdim in q["sketch_dims"]]
+            if len(sd) > L.MAX_ORDER:
+                raise IndexError("sketch_dims: more than 4 modes")
+            a, b = factors[2 * i], factors[2 * i + 1]
+            m = int(q["m"])
+            lam = float(q["lam"])
+            _PROBLEM.pack_into(arr, i * _PROBLEM.size, C.addressof(a) if a else 0, len(lists[2 * i]),
+                               C.addressof(b) if b else 0, len(lists[2 * i + 1]),
+                               order, *dims, *_ZEROS[order:], Cq.data_ptr(), _ptr(q.get("X0")) or 0, X.data_ptr(), m, 0,
+                               *sd, *_ZEROS[len(sd):], int(q["seed"]) & 0xFFFFFFFFFFFFFFFF, lam,
+                               float(q.get("tol", 0.0)))
+            if m * cycles + 1 < 0:
+                raise ValueError("negative dimensions are not allowed")
+            rows.append((room, m * cycles + 1, lam))
+            room += m * cycles + 1 + L.MAX_MU
             Xs.append(X)
-        opts = L.Opts()
-        grid = None
-        if mu_grid is not None:
-            grid = np.ascontiguousarray(mu_grid, dtype=np.float64)
-            opts.mu_grid = grid.ctypes.data_as(C.POINTER(C.c_double))
-            opts.n_mu = len(grid)
-        opts.breakdown_tol = float(breakdown_tol)
-        opts.group_max = int(group_max)
-        opts.queue_slots = int(queue_slots)
-        opts.max_restarts = int(max_restarts)
-        opts.flags = ((L.FLAG_BF16_BASIS if bf16_basis else 0) | (0 if use_graph else L.FLAG_NO_GRAPH) |
-                      (L.FLAG_PHASE_TIMES if phase_times else 0) | (L.FLAG_TRUE_RESIDUAL if true_residual else 0))
-        infos = (L.Info * len(problems))()
-        bufs = []
-        for i, q in enumerate(problems):
-            rho = np.zeros(int(q["m"]) * (int(max_restarts) + 1) + 1)
-            gcv = np.zeros(L.MAX_MU)
-            infos[i].rho_hist = rho.ctypes.data_as(C.POINTER(C.c_double))
-            infos[i].gcv = gcv.ctypes.data_as(C.POINTER(C.c_double))
-            bufs.append((rho, gcv))
-        L.check(self.lib.rtg_gmres_solve_batched(self._h, len(problems), arr, dt, C.byref(opts), infos,
-                                                 _stream(stream)))
-        res = [_solve_result(infos[i], bufs[i][0], bufs[i][1], grid, float(q["lam"]))
-               for i, q in enumerate(problems)]
-        if phase_times:
-            for i, r in enumerate(res):
-                r.phase_ms = {k: infos[i].phase_ms[j] for j, k in enumerate(L.PHASES)}
-                r.phase_launches = {k: infos[i].phase_launches[j] for j, k in enumerate(L.PHASES)}
+        flags = ((L.FLAG_BF16_BASIS if bf16_basis else 0) | (0 if use_graph else L.FLAG_NO_GRAPH) |
+                 (L.FLAG_PHASE_TIMES if phase_times else 0) | (L.FLAG_TRUE_RESIDUAL if true_residual else 0))
+        opts, grid = _solve_opts(0.0, mu_grid, max_restarts, breakdown_tol, flags, 0, group_max, queue_slots)
+        hist = np.zeros(room)   # rho and gcv of every problem
+        at = _address(hist)
+        for i, (o, k, _) in enumerate(rows):
+            _INFO_PTRS.pack_into(infos, i * _INFO.size + L.Info.rho_hist.offset, at + 8 * o, at + 8 * (o + k))
+        L.check(self.lib.rtg_gmres_solve_batched(self._h, n, arr, dt, C.byref(opts), infos, _stream(stream)))
+        res = [_solve_result(f, hist[o:o + k], hist[o + k:o + k + L.MAX_MU], grid, lam, phase_times)
+               for f, (o, k, lam) in zip(_INFO.iter_unpack(infos), rows)]
         return Xs, res
 
     def gmres_wait(self, pend: "PendingSolve"):
         """Wait for a submitted solve (rtg_gmres_wait); returns (X, SolveResult)."""
-        info = L.Info()
-        rho = np.zeros(pend.m * (pend.max_restarts + 1) + 1)
-        info.rho_hist = rho.ctypes.data_as(C.POINTER(C.c_double))
-        gcv = np.zeros(L.MAX_MU)
-        info.gcv = gcv.ctypes.data_as(C.POINTER(C.c_double))
+        info, rho, gcv = _solve_info(pend.m, pend.max_restarts + 1)
         L.check(self.lib.rtg_gmres_wait(self._h, pend.slot, C.byref(info)))
-        res = _solve_result(info, rho, gcv, pend.grid, pend.lam)
-        if pend.phase_times:
-            res.phase_ms = {k: info.phase_ms[i] for i, k in enumerate(L.PHASES)}
-            res.phase_launches = {k: info.phase_launches[i] for i, k in enumerate(L.PHASES)}
-        return pend.X, res
+        return pend.X, _solve_result(_INFO.unpack(info), rho, gcv, pend.grid, pend.lam, pend.phase_times)
 
 
-def _solve_result(info, rho, gcv, grid, lam):
-    return SolveResult(info.iters, info.restarts, bool(info.breakdown), bool(info.converged),
-                       info.beta, info.mu, info.rho_final, rho[:info.iters].copy(),
-                       gcv[:len(grid)].copy() if (grid is not None and lam < 0) else None,
-                       info.elapsed_ms, info.device_status, info.launches, tile_config=info.tile_config,
-                       true_rel_resid=info.true_rel_resid, true_rel_resid_theta=info.true_rel_resid_theta)
+def _solve_result(f, rho, gcv, grid, lam, phase_times=False):
+    """SolveResult of an unpacked rtg_info record."""
+    (iters, restarts, breakdown, converged, beta, mu, rho_final, _, _, resid, elapsed, status, launches, tile,
+     *phases, resid_theta) = f
+    res = SolveResult(iters, restarts, bool(breakdown), bool(converged), beta, mu, rho_final, rho[:iters].copy(),
+                      gcv[:len(grid)].copy() if (grid is not None and lam < 0) else None, elapsed, status, launches,
+                      tile_config=tile, true_rel_resid=resid, true_rel_resid_theta=resid_theta)
+    if phase_times:
+        res.phase_ms = dict(zip(L.PHASES, phases))
+        res.phase_launches = dict(zip(L.PHASES, phases[L.PHASE_COUNT:]))
+    return res
 
 
 @dataclasses.dataclass
@@ -444,11 +478,10 @@ class Krylov:
         self.dtype = dtype
         self.m = m
         code = L.F64 if dtype == torch.float64 else L.F32
-        a, na, ka = _factor_array(A_factors)
-        b, nb, kb = _factor_array(B_factors)
+        (a, b), keep = _factor_arrays(A_factors, B_factors)
         sk = (C.c_int64 * len(dims))(*[int(s) for s in sketch_dims])
         k = C.c_void_p()
-        L.check(handle.lib.rtg_krylov_create(handle._h, a, na, b, nb, _shape(dims), code, int(m), sk,
+        L.check(handle.lib.rtg_krylov_create(handle._h, a, len(A_factors), b, len(B_factors), _shape(dims), code, int(m), sk,
                                              C.c_uint64(seed), C.c_uint64(problem_id), C.byref(k)))
         self._k = k
         self.sdims = tuple(int(min(s, d)) for s, d in zip(sketch_dims, dims))
@@ -569,27 +602,16 @@ class WarmStart:
         _check_tensor(C_obs, dims, "C")
         if X is None:
             X = empty(dims, C_obs.dtype, C_obs.device)
-        a, na, ka = _factor_array(A_factors)
-        b, nb, kb = _factor_array(B_factors)
+        (a, b), keep = _factor_arrays(A_factors, B_factors)
         sk = (C.c_int64 * len(dims))(*[int(s) for s in sketch_dims])
-        opts = L.Opts()
-        opts.tol = float(tol)
-        grid = np.ascontiguousarray(mu_grid, dtype=np.float64)
-        opts.mu_grid = grid.ctypes.data_as(C.POINTER(C.c_double))
-        opts.n_mu = len(grid)
-        opts.max_restarts = int(max_restarts)
-        opts.flags = L.FLAG_TRUE_RESIDUAL if true_residual else 0
-        opts.slot = int(slot)
-        info = L.Info()
-        rho = np.zeros(m * (max_restarts + 1) + 1)
-        info.rho_hist = rho.ctypes.data_as(C.POINTER(C.c_double))
-        gcv = np.zeros(L.MAX_MU)
-        info.gcv = gcv.ctypes.data_as(C.POINTER(C.c_double))
+        opts, grid = _solve_opts(tol, np.ascontiguousarray(mu_grid, dtype=np.float64), max_restarts, 0.0,
+                                 L.FLAG_TRUE_RESIDUAL if true_residual else 0, slot)
+        info, rho, gcv = _solve_info(m, max_restarts + 1)
         dec = L.WsResult()
-        L.check(self.lib.rtg_ws_solve(self._h, handle._h, a, na, b, nb, _shape(dims), C_obs.data_ptr(), int(m), sk,
+        L.check(self.lib.rtg_ws_solve(self._h, handle._h, a, len(A_factors), b, len(B_factors), _shape(dims), C_obs.data_ptr(), int(m), sk,
                                       C.c_uint64(seed), X.data_ptr(), C.byref(opts), C.byref(info), C.byref(dec),
                                       _stream(stream)))
-        res = _solve_result(info, rho, gcv, grid, -1.0 if dec.fell_back else 1.0)
+        res = _solve_result(_INFO.unpack(info), rho, gcv, grid, -1.0 if dec.fell_back else 1.0)
         return X, res, {"fell_back": bool(dec.fell_back), "lam": dec.lam, "tol": dec.tol,
                         "sketch_norm_C": dec.sketch_norm_C, "sketch_norm_R0": dec.sketch_norm_R0}
 
