@@ -992,4 +992,44 @@ __device__ inline void givens_step(const Work& w, const StepOpts& o) {
   set_cond(o, !ctl->stop, ctl);
 }
 
+// new_cycle = 0: start of a solve; 1: start of a restarted cycle (gated by
+// rs_skip inside the step body: it keeps the body count, the lock-step
+// count of running problems and the restart flag, which the restart
+// sequence clears last).
+__device__ inline void reset_ctl(const Work& w0, int new_cycle, unsigned* group_left, const int* gate) {
+  const BIdx bi = bidx(w0.b);
+  Ctl* ctl = bsh(w0.ctl, bi.off);
+  gate = bsh(gate, bi.off);
+  if (gate != nullptr && *gate) return;
+  unsigned* counter = bsh(w0.counter, bi.off);
+  // last-block counters wrap to zero by themselves; clearing them here also
+  // recovers from a solve that ended inside a kernel
+  for (int i = 0; i < 8; ++i) counter[i] = 0u;
+  ctl->j = 0;
+  ctl->stop = 0;
+  ctl->breakdown = 0;
+  ctl->converged = 0;
+  ctl->skip_update = 0;
+  ctl->pre2 = 0.0;
+  ctl->hnext = 0.0;
+  ctl->givens = 0;
+  if (new_cycle) {
+    ctl->cycle += 1;
+  } else {
+    if (group_left != nullptr && bi.p == 0) *group_left = static_cast<unsigned>(w0.b.n);
+    ctl->counted = 0;
+    ctl->loops = 0;
+    ctl->rs_skip = 1;
+    ctl->status = 0;
+    ctl->iters_total = 0;
+    ctl->cycle = 0;
+    ctl->beta0 = 0.0;
+    ctl->beta = 0.0;
+    ctl->rho = 1.0;
+    ctl->mu = 0.0;
+    ctl->true_rr = -1.0;
+    ctl->true_th = -1.0;
+  }
+}
+
 }  // namespace rtg

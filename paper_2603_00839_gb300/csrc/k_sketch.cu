@@ -31,6 +31,7 @@
 #include <cuda_bf16.h>
 
 #include "gs_common.cuh"
+#include "philox.cuh"
 #include "tma_common.cuh"
 #include "umma_common.cuh"
 
@@ -169,133 +170,151 @@ SketchScratch carve_sketch_scratch(const SketchPlan& sp, void* base) {
 
 // ------------------------------------------------------------------ Theta fragments
 
-__device__ __forceinline__ uint32_t pm1_pair(uint32_t b0, uint32_t b1, bool v0, bool v1) {
-  // packed bf16x2: +1 = 0x3F80, -1 = 0xBF80, padding = 0
-  const uint32_t lo = v0 ? (0x3F80u | (b0 << 15)) : 0u;
-  const uint32_t hi = v1 ? (0x3F80u | (b1 << 15)) : 0u;
-  return lo | (hi << 16);
-}
+enum ThetaKind { kThetaBits, kThetaImage, kThetaFrags };
 
-__device__ __forceinline__ uint32_t theta_bit(const uint32_t* rowbits, int64_t i) {
-  return (rowbits[i >> 5] >> (i & 31)) & 1u;
-}
-
-struct FragArgs {
-  int nstage;
-  int64_t s[kMaxOrder], I[kMaxOrder], word_off[kMaxOrder], frag_off[kMaxOrder];
-  int wpr[kMaxOrder], kt[kMaxOrder], ntile[kMaxOrder];
-  int64_t total_lanes;
-  int64_t lane_off[kMaxOrder + 1];
+struct ThetaMode {
+  int kind, wpr, kt, kblocks;
+  uint32_t words;               // words a row, padding included
+  int64_t s, I, bit_off, word_off, frag_off;
 };
 
-// One thread per (tile, k-tile, lane) of every later stage (L > 1): the
-// fragment registers of mma.m16n8k16 for Theta^T (the B operand).
-__global__ void k_theta_frags(FragArgs a, const uint32_t* bits0, uint32_t* frags0, Batch bt) {
-  const int64_t bo = bidx(bt).off;
-  const uint32_t* bits = bsh(bits0, bo);
-  uint32_t* frags = bsh(frags0, bo);
-  const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (g >= a.total_lanes) return;
-  int t = 0;
-  while (t + 1 < a.nstage && g >= a.lane_off[t + 1]) ++t;
-  const int64_t local = g - a.lane_off[t];
-  const int lane = static_cast<int>(local & 31);
-  // blocked layout: ((block * kt + kk) * N_NT + tile_in_block) * 32 + lane
-  constexpr int per = N_NT;
-  const int64_t idx = local >> 5;
-  const int tin = static_cast<int>(idx % per);
-  const int kk = static_cast<int>((idx / per) % a.kt[t]);
-  const int64_t blk = idx / (static_cast<int64_t>(per) * a.kt[t]);
-  const int64_t tile = blk * per + tin;
-  const int64_t tile_k = idx;
-  const int gid = lane >> 2, tig = lane & 3;
-  const uint32_t* rows = bits + a.word_off[t];
-  const int64_t k0 = static_cast<int64_t>(kk) * 16 + tig * 2;
-  // B (16 x 8, "col"): reg0 (k0..k0+1, n), reg1 (k0+8.., n); B(k = i, n = q) = Theta(q, i)
-  const int64_t q = tile * 8 + gid;
-  const bool rv = q < a.s[t];
-  const uint32_t* rb = rows + (rv ? q : 0) * a.wpr[t];
-  uint32_t reg[2];
-  for (int h = 0; h < 2; ++h) {
-    const int64_t i = k0 + (h ? 8 : 0);
-    const bool v0 = rv && i < a.I[t], v1 = rv && (i + 1) < a.I[t];
-    reg[h] = pm1_pair(v0 ? theta_bit(rb, i) : 0u, v1 ? theta_bit(rb, i + 1) : 0u, v0, v1);
-  }
-  uint2* out = reinterpret_cast<uint2*>(frags + a.frag_off[t]);
-  out[tile_k * 32 + lane] = make_uint2(reg[0], reg[1]);
-}
+struct ThetaArgs {
+  int nmodes;                   // sketched modes
+  ThetaMode md[kMaxOrder];
+  int64_t off[kMaxOrder + 1];   // first unit of each mode
+  uint64_t seed, pid;
+  const uint64_t* key;          // if set: (seed, pid) read from device memory at run time
+};
 
-// One thread per 16-byte chunk of the first stage's tcgen05 operand: Theta
-// rows q of M tile mt and K block kb as a 128-row x 64-value BF16 tile in
-// the 128-byte swizzled K-major layout (umma_common.cuh), one 16 KB image
-// per (mt, kb), rows q >= s and values i >= I zero.
-__global__ void k_theta_image(const uint32_t* bits0, uint32_t* frags0, int64_t word_off, int wpr, int64_t s,
-                              int64_t I, int kblocks, int64_t frag_off, int64_t nchunks, Batch bt) {
-  const int64_t bo = bidx(bt).off;
-  const uint32_t* bits = bsh(bits0, bo);
-  uint32_t* frags = bsh(frags0, bo);
-  const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (g >= nchunks) return;
-  const uint32_t j = static_cast<uint32_t>(g & 7);
-  const uint32_t r = static_cast<uint32_t>((g >> 3) & 127);
-  const int64_t tile = g >> 10;                       // mt * kblocks + kb
-  const int64_t kb = tile % kblocks, mt = tile / kblocks;
-  const int64_t q = mt * 128 + r, i0 = kb * 64 + 8 * j;
-  const bool rv = q < s;
-  const uint32_t* rb = bits + word_off + (rv ? q : 0) * wpr;
-  uint32_t w[4];
-#pragma unroll
-  for (int h = 0; h < 4; ++h) {
-    const int64_t i = i0 + 2 * h;
-    const bool v0 = rv && i < I, v1 = rv && (i + 1) < I;
-    w[h] = pm1_pair(v0 ? theta_bit(rb, i) : 0u, v1 ? theta_bit(rb, i + 1) : 0u, v0, v1);
+// All of Theta and the solve's control words in one launch.  One thread per 32
+// signs (row q, word wi) of a mode: bit b of the packed word holds the sign of
+// Theta(q, 32 wi + b), padding past I is 0 (+1), and the same thread expands
+// them into what the mode's contraction reads:
+//  * tcgen05 stage: four 16-byte chunks of the 128-row x 64-value BF16 tile of
+//    M tile q / 128 and K block wi / 2 (128-byte swizzled K-major layout,
+//    umma_common.cuh; one 16 KB image per tile), rows q >= s and values i >= I
+//    zero: the rows are padded to M tiles, the words to K blocks;
+//  * mma.sync stage: eight lanes' registers of mma.m16n8k16's B operand
+//    (Theta^T), blocked ((block kt + kk) N_NT + tile) 32 + lane;
+//  * FP64 chain: the packed words alone.
+// The work is a few hundred instructions a thread (one Philox block yields 256
+// signs, two when the word straddles a block) and latency is all of its time:
+// CTAs of 64 spread it over the chip.  Block gridDim.x - 1 resets the control
+// words when asked to.  Bits, image, fragments and reset as kernels of their
+// own took 15.5 us and three launch gaps: a 512 x 512 solve went from 280 to
+// 265 us with this one, an FP64 64 x 64 solve from 324 to 291.
+__global__ void __launch_bounds__(64) k_theta(ThetaArgs a, uint32_t* bits0, uint32_t* frags0, Batch bt, int reset,
+                                              Work w0, unsigned* group_left) {
+  if (reset && blockIdx.x == gridDim.x - 1) {
+    if (threadIdx.x == 0) reset_ctl(w0, 0, group_left, nullptr);
+    return;
   }
-  unsigned char* img = reinterpret_cast<unsigned char*>(frags + frag_off) + tile * 16384;
-  *reinterpret_cast<uint4*>(img + sw128_off(r, j)) = make_uint4(w[0], w[1], w[2], w[3]);
+  const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (g >= a.off[a.nmodes]) return;
+  const int64_t bo = bidx(bt).off;
+  uint32_t* bits = bsh(bits0, bo);
+  uint32_t* frags = bsh(frags0, bo);
+  const uint64_t* key = bsh(a.key, bo);
+  const uint64_t seed = key ? key[0] : a.seed, pid = key ? key[1] : a.pid;
+  int t = 0;
+  while (t + 1 < a.nmodes && g >= a.off[t + 1]) ++t;
+  const ThetaMode& md = a.md[t];
+  const int64_t local = g - a.off[t];
+  int64_t q;
+  if (local >> 32) q = local / md.words;
+  else q = static_cast<uint32_t>(local) / md.words;
+  const uint32_t wi = static_cast<uint32_t>(local - q * md.words);
+  const int64_t i0 = static_cast<int64_t>(wi) * 32;
+  const int valid = (q < md.s && i0 < md.I) ? static_cast<int>(md.I - i0 < 32 ? md.I - i0 : 32) : 0;
+  uint32_t out = 0;
+  if (valid > 0) {
+    const int64_t e0 = md.bit_off + q * md.I + i0;
+    const int64_t b0 = e0 >> 6;
+    const int sh = static_cast<int>(e0 & 63), l = static_cast<int>(b0 & 3);
+    uint64_t r[4];
+    philox4x64_10(static_cast<uint64_t>(b0 >> 2) + 1, 0, 0, 0, seed, pid, r);
+    uint64_t v = (l == 0 ? r[0] : l == 1 ? r[1] : l == 2 ? r[2] : r[3]) >> sh;
+    if (sh > 32) {   // the signs go on in the next 64-bit word
+      uint64_t next = l == 0 ? r[1] : l == 1 ? r[2] : r[3];
+      if (l == 3) {
+        philox4x64_10(static_cast<uint64_t>(b0 >> 2) + 2, 0, 0, 0, seed, pid, r);
+        next = r[0];
+      }
+      v |= next << (64 - sh);
+    }
+    out = static_cast<uint32_t>(v);
+    if (valid < 32) out &= (1u << valid) - 1u;
+    bits[md.word_off + q * md.wpr + wi] = out;
+  }
+  // bf16x2 of the signs at positions p, p + 1: +1 = 0x3F80, -1 = 0xBF80, padding = 0
+  auto pair = [&](int p) {
+    const uint32_t x = out >> p;
+    const uint32_t lo = p < valid ? 0x3F80u | ((x & 1u) << 15) : 0u;
+    const uint32_t hi = p + 1 < valid ? 0x3F80u | ((x & 2u) << 14) : 0u;
+    return lo | (hi << 16);
+  };
+  if (md.kind == kThetaImage) {
+    const uint32_t row = static_cast<uint32_t>(q & 127);
+    unsigned char* img = reinterpret_cast<unsigned char*>(frags + md.frag_off) +
+                         ((q >> 7) * md.kblocks + (wi >> 1)) * 16384;
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      *reinterpret_cast<uint4*>(img + sw128_off(row, (wi & 1) * 4 + c)) =
+          make_uint4(pair(8 * c), pair(8 * c + 2), pair(8 * c + 4), pair(8 * c + 6));
+  } else if (md.kind == kThetaFrags) {
+    const int64_t tile = q >> 3;
+    uint2* o = reinterpret_cast<uint2*>(frags + md.frag_off);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int kk = static_cast<int>(2 * wi) + h;
+      if (kk >= md.kt) break;
+      const int64_t at = (((tile / N_NT) * md.kt + kk) * N_NT + tile % N_NT) * 32 + (q & 7) * 4;
+#pragma unroll
+      for (int tig = 0; tig < 4; ++tig)
+        o[at + tig] = make_uint2(pair(16 * h + 2 * tig), pair(16 * h + 2 * tig + 8));
+    }
+  }
 }
 
 cudaError_t launch_theta(const SketchPlan& sp, uint32_t* bits, uint32_t* frags, cudaStream_t s,
-                         const uint64_t* key_dev, Batch b) {
-  cudaError_t e = launch_theta_bits(sp, bits, s, key_dev, b);
-  if (e != cudaSuccess || sp.dtype != RTG_F32 || sp.nstage == 0) return e;
-  bool frag_stages = false;
-  for (int t = 0; t < sp.nstage; ++t) {
-    if (!sp.stage_umma[t]) {
-      frag_stages = true;
-      continue;
+                         const uint64_t* key_dev, Batch b, const Work* reset, unsigned* group_left) {
+  ThetaArgs a{};
+  a.key = key_dev;
+  a.seed = sp.seed;
+  a.pid = sp.pid;
+  for (int k = 0; k < sp.order; ++k) {
+    if (!sp.sketched[k]) continue;
+    ThetaMode& md = a.md[a.nmodes];
+    md.s = sp.sdims[k];
+    md.I = sp.dims[k];
+    md.bit_off = sp.bit_off[k];
+    md.word_off = sp.word_off[k];
+    md.wpr = sp.wpr[k];
+    md.kind = kThetaBits;
+    md.words = static_cast<uint32_t>(sp.wpr[k]);
+    int64_t rows = md.s;
+    for (int t = 0; sp.dtype == RTG_F32 && t < sp.nstage; ++t) {
+      if (sp.stage_mode[t] != k) continue;
+      md.frag_off = sp.frag_off[t];
+      if (sp.stage_umma[t]) {
+        md.kind = kThetaImage;
+        md.kblocks = sp.stage_kb[t];
+        md.words = 2u * static_cast<uint32_t>(sp.stage_kb[t]);
+        rows = int64_t(sp.stage_ntile[t]) * 128;
+      } else {
+        md.kind = kThetaFrags;
+        md.kt = sp.stage_kt[t];
+        md.words = (static_cast<uint32_t>(sp.stage_kt[t]) + 1) / 2;
+        rows = int64_t((sp.stage_ntile[t] + N_NT - 1) / N_NT) * N_NT * 8;
+      }
     }
-    const int k = sp.stage_mode[t];
-    const int64_t nchunks = int64_t(sp.stage_ntile[t]) * sp.stage_kb[t] * 1024;
-    k_theta_image<<<dim3(static_cast<unsigned>((nchunks + 255) / 256), 1, b.n), 256, 0, s>>>(
-        bits, frags, sp.word_off[k], sp.wpr[k], sp.stage_s[t], sp.stage_I[t], sp.stage_kb[t], sp.frag_off[t],
-        nchunks, b);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    a.off[a.nmodes + 1] = a.off[a.nmodes] + rows * md.words;
+    ++a.nmodes;
   }
-  if (!frag_stages) return cudaSuccess;
-  FragArgs a{};
-  a.nstage = sp.nstage;
-  int64_t lanes = 0;
-  for (int t = 0; t < sp.nstage; ++t) {
-    if (sp.stage_umma[t]) {   // no fragments for this stage: zero lanes
-      a.lane_off[t] = lanes;
-      a.kt[t] = 1;
-      continue;
-    }
-    const int k = sp.stage_mode[t];
-    a.s[t] = sp.stage_s[t];
-    a.I[t] = sp.stage_I[t];
-    a.word_off[t] = sp.word_off[k];
-    a.frag_off[t] = sp.frag_off[t];
-    a.wpr[t] = sp.wpr[k];
-    a.kt[t] = sp.stage_kt[t];
-    a.ntile[t] = sp.stage_ntile[t];
-    a.lane_off[t] = lanes;
-    lanes += ((sp.stage_ntile[t] + N_NT - 1) / N_NT) * N_NT * int64_t(sp.stage_kt[t]) * 32;
-  }
-  a.lane_off[sp.nstage] = lanes;
-  a.total_lanes = lanes;
-  k_theta_frags<<<dim3(static_cast<unsigned>((lanes + 255) / 256), 1, b.n), 256, 0, s>>>(a, bits, frags, b);
+  if (a.off[a.nmodes] == 0) return reset ? launch_reset(*reset, 0, s, group_left) : cudaSuccess;
+  const int64_t blocks = (a.off[a.nmodes] + 63) / 64 + (reset ? 1 : 0);
+  k_theta<<<dim3(static_cast<unsigned>(blocks), 1, b.n), 64, 0, s>>>(a, bits, frags, b, reset ? 1 : 0,
+                                                                     reset ? *reset : Work{}, group_left);
   return cudaGetLastError();
 }
 

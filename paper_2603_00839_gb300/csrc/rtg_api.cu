@@ -462,7 +462,7 @@ struct SolvePlan {
   int dtype = RTG_F32;
   int vdtype = RTG_F32;                                           // storage of V and W
   int launches_pro = 0, launches_step = 0, launches_epi = 0;   // kernels per phase
-  int launches_setup = 0;                                         // reset + Theta, part of the prologue
+  int launches_setup = 0;                                         // reset and Theta, part of the prologue
   int launches_restart = 0;   // one restart sequence (graph: per restart; direct: every step)
   int direct_steps = 0;                                           // steps launched by the last direct solve
   int* stop_host = nullptr;                                       // pinned: ctl->stop read back per direct step
@@ -702,8 +702,7 @@ rtg_status enqueue_prologue(SolvePlan& P, const StepOpts& so, cudaStream_t s,
   Work& w = P.w;
   {
     PhaseScope ps(pt, RTG_PHASE_SETUP, -1, P.launches_setup);
-    CK(launch_reset(w, 0, s, P.group_left));
-    CK(launch_theta(P.sp, P.sk.bits, P.sk.frags, s, P.desc_dev->key, w.b));
+    CK(launch_theta(P.sp, P.sk.bits, P.sk.frags, s, P.desc_dev->key, w.b, &w, P.group_left));
   }
   PhaseScope ps(pt, RTG_PHASE_INIT, -1, P.launches_pro - P.launches_setup);
   PtrRef C = desc_ref(reinterpret_cast<const void* const*>(&P.desc_dev->C));
@@ -820,8 +819,7 @@ rtg_status enqueue_gk_prologue(SolvePlan& P, const StepOpts& so, cudaStream_t s,
   Work& w = P.w;
   {
     PhaseScope ps(pt, RTG_PHASE_SETUP, -1, P.launches_setup);
-    CK(launch_reset(w, 0, s));
-    CK(launch_theta(P.sp, P.sk.bits, P.sk.frags, s, P.desc_dev->key));
+    CK(launch_theta(P.sp, P.sk.bits, P.sk.frags, s, P.desc_dev->key, Batch{}, &w));
   }
   PhaseScope ps(pt, RTG_PHASE_INIT, -1, P.launches_pro - P.launches_setup);
   PtrRef C = desc_ref(reinterpret_cast<const void* const*>(&P.desc_dev->C));
@@ -1323,10 +1321,8 @@ rtg_status make_plan(const PlanSpec& ps, SolveDesc* ddev, InfoDev* idev, SolveDe
   CK(cudaEventCreate(&P->ev0));
   CK(cudaEventCreate(&P->ev1));
   {
-    int nsk = 0;
-    for (int k = 0; k < sp.order; ++k) nsk += sp.sketched[k];
     const int gs = sp.fused_dots ? 0 : 1;
-    P->launches_setup = 1 + (nsk > 0 ? (dtype == RTG_F32 ? 2 : 1) : 0);
+    P->launches_setup = 1;
     P->launches_pro = P->launches_setup +
                       (has_x0 ? apply_launches(P->op.op, true, dtype, dtype, vdtype) : 0) +
                       sketch_launches(sp) + gs + 1;

@@ -345,13 +345,13 @@ void record_error(const char* msg);
 // k_philox.cu
 cudaError_t launch_philox_words(uint64_t seed, uint64_t pid, int64_t n_words, uint64_t* out,
                                 cudaStream_t s);
+// Signs and, for the FP32 chain, the Theta images and fragments of every stage.
 // key_dev (optional): device array {seed, problem_id} read when the kernel runs,
 // so one captured graph serves every seed; otherwise sp.seed / sp.pid.
-cudaError_t launch_theta_bits(const SketchPlan& sp, uint32_t* bits, cudaStream_t s,
-                              const uint64_t* key_dev = nullptr, Batch b = Batch{});
-// signs, then (FP32 chain) the Theta images and fragments of every stage
+// reset: launch_reset(*reset, 0, s, group_left) in the same kernel.
 cudaError_t launch_theta(const SketchPlan& sp, uint32_t* bits, uint32_t* frags, cudaStream_t s,
-                         const uint64_t* key_dev = nullptr, Batch b = Batch{});
+                         const uint64_t* key_dev = nullptr, Batch b = Batch{}, const Work* reset = nullptr,
+                         unsigned* group_left = nullptr);
 
 // k_apply.cu: Y = alpha * Phi(X) + beta * Z (Z may be null when beta == 0).
 // tmp: scratch of n elements for the unfused path (may be null if unused).

@@ -189,3 +189,20 @@ def test_two_steps_a_loop_body_equal_direct_launches(api, h, dtype, m, stop_at):
         Xg, g = solve(Cd, m, (20, 18), 3, 0.0, tol=tol, **kw)
         assert (g.iters, g.converged, g.breakdown) == (r.iters, r.converged, r.breakdown)
         assert torch.equal(Xg, X) and np.array_equal(g.rho, r.rho)
+
+
+# ------------------------------------------------------------------------ Theta
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("dims,sk", [
+    ((31, 33), (1, 32)), ((32, 65), (31, 1)), ((63, 257), (62, 129)), ((64, 17), (9, 16)), ((130, 255), (129, 8)),
+    ((5, 300), (5, 97)), ((257, 3), (256, 3)),   # one mode sketched only
+])
+def test_theta_words(api, h, dtype, dims, sk):
+    """Rows whose signs start anywhere in the stream's 64-bit words and blocks of
+    four, last words of every length, padded rows and K tiles."""
+    X = np.random.default_rng(dims[0]).standard_normal(dims).astype(dtype)
+    ref = oracle.sketch(X.astype(np.float64), oracle.sketch_matrices(dims, sk, 2 ** 64 - 3, problem_id=7))
+    got = h.sketch(api.to_device(np.asfortranarray(X)), sk, 2 ** 64 - 3, problem_id=7).cpu().double().numpy()
+    # one wrong sign changes the result by over 1e-3; the chains have at most 257 terms
+    assert _rel(got, ref) < (1e-13 if dtype == np.float64 else 5e-6)
