@@ -20,33 +20,74 @@ namespace rtg {
 // Four warps per candidate mu.  An FP64 warp instruction occupies its SM
 // sub-partition's FP64 unit for about 64 cycles on this GPU, so the cost of
 // this kernel is the number of FP64 warp instructions each sub-partition
-// issues: the work of every step is spread over all 128 lanes (rows and
-// columns at once), and the scalars of a reflection are computed by every
-// warp at the same time instead of being broadcast.
+// issues one after another: the columns of a reflection are dealt over the
+// warps and its rows over the lanes, every warp takes the pivot column's norm
+// itself (no exchange before the update), and the square root and the
+// quotients are Newton-Raphson refinements of FP32 seeds (8 FP64 instructions
+// a reflection; sqrt() and two divisions take over 30).  Back substitution
+// and residual (warp 0) run beside the trace's inverse (warps 1 to 3).
+// With this form a 512 x 512 solve (8 candidates) went from 279 to 275 us, a
+// 1024 x 1024 one of 12 steps from 881 to 873, an FP64 64 x 64 one from 358 to 354.
 constexpr int TK_THREADS = 128;
 constexpr int TK_WARPS = TK_THREADS / 32;
 
-__device__ __forceinline__ double tk_block_sum(double v, double* wsum) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = v;
-  __syncthreads();
-  const double t = (wsum[0] + wsum[1]) + (wsum[2] + wsum[3]);
-  __syncthreads();
-  return t;
+// 2^-e x by the exponent field (x and the result normal).
+__device__ __forceinline__ double tk_scale(double x, int e) {
+  return __hiloint2double(__double2hiint(x) - (e << 20), __double2loint(x));
 }
 
-// Back substitution y = U^{-1} b for an upper-triangular k x k U (leading
-// dimension ldu) with precomputed reciprocal pivots rinv (0 for a zero
-// pivot: y_i = 0, the smallest-norm least-squares choice on that
-// direction), run by one warp; b is overwritten.
-__device__ void back_subst(const double* U, int ldu, const double* rinv, double* b, double* y,
-                           int k) {
+// Double value of a normal positive float, and the float of a double in [1, 4)
+// with its low bits cut, in the integer pipes (a conversion between the two
+// types takes about as long as a dozen FP64 instructions).
+__device__ __forceinline__ double tk_widen(float f) {
+  const uint32_t b = __float_as_uint(f);
+  return __hiloint2double(static_cast<int>((b >> 3) + ((1023u - 127u) << 20)), static_cast<int>(b << 29));
+}
+__device__ __forceinline__ float tk_narrow(double x) {
+  const uint32_t h = static_cast<uint32_t>(__double2hiint(x));
+  return __uint_as_float(((h - ((1023u - 127u) << 20)) << 3) | (static_cast<uint32_t>(__double2loint(x)) >> 29));
+}
+
+// 1 / sqrt(q), q > 0: an FP32 seed (relative error below 2^-21) and one step of
+// third order, y (1 + e / 2 + 3 e^2 / 8) with e = 1 - q y^2: its remainder,
+// 5 e^3 / 16, is below 2^-61, so rounding alone is left.
+__device__ __forceinline__ double tk_rsqrt(double q) {
+  const int hi = __double2hiint(q);
+  if (hi < 0x00200000 || hi >= 0x7fe00000) return 1.0 / sqrt(q);   // subnormal, infinite, NaN
+  const int e = ((hi >> 20) - 1023) & ~1;
+  const double a = tk_scale(q, e);   // [1, 4)
+  const double y = tk_widen(rsqrtf(tk_narrow(a)));
+  const double r = fma(-(a * y), y, 1.0);
+  return tk_scale(fma(y, r * fma(0.375, r, 0.5), y), e / 2);
+}
+
+// 1 / h for h in [1, 4): r (1 + e + e^2), e = 1 - h r, remainder e^3 < 2^-63.
+__device__ __forceinline__ double tk_recip(double h) {
+  const double r = tk_widen(__frcp_rn(tk_narrow(h)));
+  const double e = fma(-h, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
+// Back substitution with the unit upper-triangular U D^{-1} (U's columns
+// already multiplied by rinv; leading dimension ldu) by one warp: b becomes
+// D y.  rinv is 0 for a zero pivot: y_i = 0, the smallest-norm least-squares
+// choice on that direction.
+__device__ void back_subst(const double* U, int ldu, double* b, int k) {
   const int lane = threadIdx.x & 31;
-  for (int i = k - 1; i >= 0; --i) {
+  if (k <= 32) {   // b in the lanes' registers
+    double v = lane < k ? b[lane] : 0.0;
+    for (int i = k - 1; i > 0; --i) {
+      const double bi = __shfl_sync(0xffffffffu, v, i);
+      if (lane < i) v = fma(-U[lane + static_cast<int64_t>(ldu) * i], bi, v);
+    }
+    if (lane < k) b[lane] = v;
     __syncwarp();
-    const double yi = b[i] * rinv[i];
-    if (lane == 0) y[i] = yi;
-    for (int t = lane; t < i; t += 32) b[t] -= U[t + static_cast<int64_t>(ldu) * i] * yi;
+    return;
+  }
+  for (int i = k - 1; i > 0; --i) {
+    __syncwarp();
+    const double bi = b[i];
+    for (int t = lane; t < i; t += 32) b[t] = fma(-U[t + static_cast<int64_t>(ldu) * i], bi, b[t]);
   }
   __syncwarp();
 }
@@ -75,8 +116,6 @@ k_tikhonov(Work w0, const SolveDesc* desc0, int mode, double* scratch0, int in_s
   }
   const int k = ctl->j;
   const int m = w.m, ld = m + 1;
-  __shared__ double red[TK_WARPS][kMaxK + 1];   // per-warp partial dot products of a step
-  __shared__ double sp[TK_WARPS];               // per-warp partial squares of the next column
   __shared__ double wsum[TK_WARPS];
   __shared__ int am_last;
   extern __shared__ __align__(16) double tk_smem[];
@@ -97,133 +136,164 @@ k_tikhonov(Work w0, const SolveDesc* desc0, int mode, double* scratch0, int in_s
     T[i + lm * col] = (col == k) ? w.g[i] : (i <= col ? w.R[i + static_cast<int64_t>(ld) * col] : 0.0);
     Bm[i + lm * col] = (i == col) ? smu : 0.0;
   }
-  if (tid < TK_WARPS) sp[tid] = 0.0;
   __syncthreads();
   if (mode != 0) {
     // Householder on column j: rows {j of T} U {0..j of B}; row j of B is
     // still sqrt(mu), rows 0..j-1 were filled by the earlier reflections.
+    // Slot 0 of every warp is the pivot column, slot c > 0 its column
+    // j + 1 + warp + 4 (c - 1) (column k: the right-hand side); a warp covers
+    // cw slots at a time and 32 / cw stripes of rows.
     for (int j = 0; j < k; ++j) {
-      const int nc = k - j;   // columns j+1 .. k (k: the right-hand side)
-      // a warp covers cw column slots and 32/cw row stripes
-      const int cw = nc >= 32 ? 32 : 1 << (32 - __clz(nc - 1));
-      const int nst = TK_WARPS * (32 / cw);
-      const int st = warp * (32 / cw) + lane / cw;
-      const int cs = lane % cw;
-      const double sigma = ((sp[0] + sp[1]) + (sp[2] + sp[3])) + smu * smu;
-      const double alpha = T[j + lm * j];
-      const double nrm = sqrt(alpha * alpha + sigma);
-      const bool refl = nrm != 0.0 && sigma != 0.0;
-      const double sgn = (alpha >= 0.0) ? 1.0 : -1.0;
-      const double v0 = alpha + sgn * nrm;
-      const double tau = refl ? 2.0 / (v0 * v0 + sigma) : 0.0;
-      if (refl) {   // v . column, per stripe, then over the warp's stripes
-        for (int c0 = 0; c0 < nc; c0 += cw) {
-          const int c = c0 + cs, col = j + 1 + c;
-          double a = 0.0;
-          if (c < nc) {
-            if (st == 0) a = v0 * T[j + lm * col];
-            for (int i = st; i <= j; i += nst) a = fma(Bm[i + lm * j], Bm[i + lm * col], a);
-          }
-          for (int o = cw; o < 32; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-          if (lane < cw && c < nc) red[warp][c] = a;
-        }
-      }
-      __syncthreads();
-      double s2 = 0.0;   // squares of the updated column j+1 (slot 0) over this thread's rows
-      for (int c0 = 0; c0 < nc; c0 += cw) {
-        const int c = c0 + cs, col = j + 1 + c;
-        if (c >= nc) continue;
-        double wv = 0.0;
-        if (refl) {
-          wv = tau * ((red[0][c] + red[1][c]) + (red[2][c] + red[3][c]));
-          if (st == 0) T[j + lm * col] -= wv * v0;
-        }
-        for (int i = st; i <= j; i += nst) {
-          double bv = Bm[i + lm * col];
+      const int slots = 1 + ((k - j + TK_WARPS - 1) >> 2);
+      const int cw = slots >= 32 ? 32 : 1 << (32 - __clz(slots - 1));
+      const int nst = 32 / cw, st = lane / cw, cs = lane % cw;
+      const double* Bj = Bm + lm * j;
+      const double alpha = T[j + lm * j];   // row j of T is this step's alone
+      double v0 = 0.0, tau = 0.0;
+      bool refl = false;
+      for (int c0 = 0; c0 < slots; c0 += cw) {
+        const int c = c0 + cs;
+        const int own = j + 1 + warp + TK_WARPS * (c - 1);
+        const bool in = c > 0 && c < slots && own <= k;
+        const int col = in ? own : j;
+        double* Bc = Bm + lm * col;
+        const double tj = T[j + lm * col];
+        double a = 0.0;
+        for (int i = st; i <= j; i += nst) a = fma(Bj[i], Bc[i], a);
+        for (int o = cw; o < 32; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (c0 == 0) {
+          // nrm = sqrt(alpha^2 + sigma); v0 = alpha + sgn nrm = sgn nrm h with
+          // h = 1 + |alpha| / nrm in [1, 2]; tau = 2 / v.v = 1 / (nrm^2 h);
+          // the new pivot is -sgn nrm
+          const double sigma = __shfl_sync(0xffffffffu, a, 0);
+          const double q = fma(alpha, alpha, sigma);
+          double pinv = 0.0;
+          refl = q != 0.0 && sigma != 0.0;
           if (refl) {
-            bv = fma(-wv, Bm[i + lm * j], bv);
-            Bm[i + lm * col] = bv;
+            const double yq = tk_rsqrt(q);
+            const double h = fma(fabs(alpha), yq, 1.0);
+            v0 = q * yq * h;
+            tau = yq * yq * (h < 4.0 ? tk_recip(h) : 1.0 / h);   // (NaN takes the division)
+            pinv = -yq;
+            if (!(alpha >= 0.0)) {
+              v0 = -v0;
+              pinv = yq;
+            }
+          } else if (alpha != 0.0) {
+            pinv = 1.0 / alpha;
           }
-          if (c == 0) s2 = fma(bv, bv, s2);
+          if (tid == 0) rinv[j] = pinv;
+        }
+        __syncwarp();   // every lane has read row j of its column
+        if (refl && in) {
+          const double wv = tau * fma(v0, tj, a);
+          if (st == 0) T[j + lm * col] = fma(-wv, v0, tj);
+          for (int i = st; i <= j; i += nst) Bc[i] = fma(-wv, Bj[i], Bc[i]);
         }
       }
-      for (int o = cw; o < 32; o <<= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-      if (lane == 0) sp[warp] = s2;
-      if (tid == 0 && refl) T[j + lm * j] = -sgn * nrm;
       __syncthreads();
     }
-  }
-  for (int i = tid; i < k; i += TK_THREADS) {
-    const double piv = T[i + lm * i];
-    rinv[i] = (piv != 0.0) ? 1.0 / piv : 0.0;
-  }
-  __syncthreads();
-  if (warp == 0) back_subst(T, lm, rinv, T + lm * k, y, k);
-  __syncthreads();
-  // residual ||g_{0:k} - R y||^2 + g_k^2 with the unregularised R
-  double part = 0.0;
-  for (int i = tid; i < k; i += TK_THREADS) {
-    double r0 = w.g[i], r1 = 0.0;
-    int jj = i;
-    for (; jj + 1 < k; jj += 2) {
-      r0 -= w.R[i + static_cast<int64_t>(ld) * jj] * y[jj];
-      r1 -= w.R[i + static_cast<int64_t>(ld) * (jj + 1)] * y[jj + 1];
-    }
-    if (jj < k) r0 -= w.R[i + static_cast<int64_t>(ld) * jj] * y[jj];
-    const double r = r0 + r1;
-    part += r * r;
-  }
-  const double res2 = tk_block_sum(part, wsum) + w.g[k] * w.g[k];
-  if (mode == 2) {
-    // ||Z||_F^2 with Z = R_mu^{-1}: right-looking substitution on W = I
-    // (stored in B), rows of Z from the last up.  Row l of Z is
-    // W[l, l:] / R_mu[l,l]; with the columns of R_mu above the diagonal
-    // pre-scaled by the pivot's reciprocal, each update of W is one FMA.
-    for (int idx = tid; idx < k * k; idx += TK_THREADS) {
-      const int col = idx / k, i = idx - col * k;
-      Bm[i + lm * col] = (i == col) ? 1.0 : 0.0;
-      if (i < col) T[i + lm * col] *= rinv[col];
+  } else {
+    for (int i = tid; i < k; i += TK_THREADS) {
+      const double piv = T[i + lm * i];
+      rinv[i] = (piv != 0.0) ? 1.0 / piv : 0.0;
     }
     __syncthreads();
-    double inv2 = 0.0;
-    for (int l = k - 1; l >= 0; --l) {
-      const int nc = k - l;
-      const double rl = rinv[l];
-      for (int idx = tid; idx < (l + 1) * nc; idx += TK_THREADS) {
-        const int i = idx / nc, col = l + (idx - i * nc);
-        const double wl = Bm[l + lm * col];
-        if (i == l) {
-          const double z = wl * rl;
-          inv2 = fma(z, z, inv2);
-        } else {
-          Bm[i + lm * col] = fma(-T[i + lm * l], wl, Bm[i + lm * col]);
+  }
+  // U D^{-1} in place of U above the diagonal, and I in B
+  for (int idx = tid; idx < k * k; idx += TK_THREADS) {
+    const int col = idx / k, i = idx - col * k;
+    if (mode == 2) Bm[i + lm * col] = (i == col) ? 1.0 : 0.0;
+    if (i < col) T[i + lm * col] *= rinv[col];
+  }
+  __syncthreads();
+  if (warp == 0) {
+    double* b = T + lm * k;
+    back_subst(T, lm, b, k);
+    for (int i = lane; i < k; i += 32) y[i] = b[i] * rinv[i];
+    __syncwarp();
+    if (mode == 2) {   // residual ||g_{0:k} - R y||^2 + g_k^2 with the unregularised R
+      double part = 0.0;
+      for (int i = lane; i < k; i += 32) {
+        double r0 = w.g[i], r1 = 0.0;
+        int jj = i;
+        for (; jj + 1 < k; jj += 2) {
+          r0 -= w.R[i + static_cast<int64_t>(ld) * jj] * y[jj];
+          r1 -= w.R[i + static_cast<int64_t>(ld) * (jj + 1)] * y[jj + 1];
         }
+        if (jj < k) r0 -= w.R[i + static_cast<int64_t>(ld) * jj] * y[jj];
+        const double r = r0 + r1;
+        part = fma(r, r, part);
       }
-      __syncthreads();
+      for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+      if (lane == 0) wsum[0] = fma(w.g[k], w.g[k], part);
     }
-    const double trace = 1.0 + mu * tk_block_sum(inv2, wsum);
-    const double gcv = res2 / (trace * trace);
-    if (tid == 0) w.gcv[blockIdx.x] = gcv;
+  } else if (mode == 2) {
+    // ||Z||_F^2 with Z = R_mu^{-1}: right-looking substitution on W = I
+    // (stored in B), rows of Z from the last up; row l of Z is
+    // W[l, l:] / R_mu[l,l].
+    constexpr int NT = TK_THREADS - 32;
+    const int id = tid - 32;
+    for (int l = k - 1; l > 0; --l) {
+      const int nc = k - l;
+      for (int idx = id; idx < l * nc; idx += NT) {
+        const int i = idx / nc, col = l + (idx - i * nc);
+        Bm[i + lm * col] = fma(-T[i + lm * l], Bm[l + lm * col], Bm[i + lm * col]);
+      }
+      asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
+    }
+    double inv2 = 0.0;
+    for (int idx = id; idx < k * k; idx += NT) {
+      const int col = idx / k, i = idx - col * k;
+      if (i <= col) {
+        const double z = Bm[i + lm * col] * rinv[i];
+        inv2 = fma(z, z, inv2);
+      }
+    }
+    for (int o = 16; o > 0; o >>= 1) inv2 += __shfl_xor_sync(0xffffffffu, inv2, o);
+    if (lane == 0) wsum[warp] = inv2;
+  }
+  __syncthreads();
+  if (mode == 2) {
+    if (tid == 0) {
+      const double trace = fma(mu, wsum[1] + wsum[2] + wsum[3], 1.0);
+      w.gcv[blockIdx.x] = wsum[0] / (trace * trace);
+    }
     for (int i = tid; i < k; i += TK_THREADS) w.ysel[static_cast<int64_t>(blockIdx.x) * m + i] = y[i];
     __syncthreads();
     if (tid == 0) am_last = (ticket_acq_rel(w.counter, gridDim.x - 1) == gridDim.x - 1);
     __syncthreads();
     if (!am_last) return;
     __shared__ int best;
-    if (tid == 0) {
-      int bi = 0;
-      double bv = __ldcg(w.gcv), bm = desc->mu_grid[0];
-      for (unsigned u = 1; u < gridDim.x; ++u) {
-        const double v = __ldcg(w.gcv + u), mm = desc->mu_grid[u];
-        if (v < bv || (v == bv && mm > bm)) {
-          bv = v;
-          bm = mm;
-          bi = static_cast<int>(u);
+    // the smallest value, of equal ones the larger mu, of equal ones the first;
+    // the values are not negative, so their bits order them, and a NaN
+    // (anywhere but in front) never wins
+    if (warp == 0) {
+      unsigned long long bv = ~0ull, bm = 0ull;
+      int bi = lane;
+      if (lane < static_cast<int>(gridDim.x)) {
+        bv = static_cast<unsigned long long>(__double_as_longlong(__ldcg(w.gcv + lane)));
+        bm = static_cast<unsigned long long>(__double_as_longlong(desc->mu_grid[lane]));
+        bm = (bm >> 63) ? ~bm : (bm | (1ull << 63));
+        if (lane == 0 && (bv << 1) > (0x7ffull << 53)) {
+          bv = 0ull;
+          bm = ~0ull;
         }
       }
-      best = bi;
-      ctl->mu = bm;
-      ctl->gcv_best = bv;
+      for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long ov = __shfl_xor_sync(0xffffffffu, bv, o), om = __shfl_xor_sync(0xffffffffu, bm, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (ov < bv || (ov == bv && (om > bm || (om == bm && oi < bi)))) {
+          bv = ov;
+          bm = om;
+          bi = oi;
+        }
+      }
+      if (lane == 0) {
+        best = bi;
+        ctl->mu = desc->mu_grid[bi];
+        ctl->gcv_best = __ldcg(w.gcv + bi);
+      }
     }
     __syncthreads();
     for (int i = tid; i < k; i += TK_THREADS) w.y[i] = __ldcg(w.ysel + static_cast<int64_t>(best) * m + i);

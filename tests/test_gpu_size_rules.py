@@ -206,3 +206,33 @@ def test_theta_words(api, h, dtype, dims, sk):
     got = h.sketch(api.to_device(np.asfortranarray(X)), sk, 2 ** 64 - 3, problem_id=7).cpu().double().numpy()
     # one wrong sign changes the result by over 1e-3; the chains have at most 257 terms
     assert _rel(got, ref) < (1e-13 if dtype == np.float64 else 5e-6)
+
+
+# ------------------------------------------------------------------------ projected Tikhonov
+
+# columns are dealt over four warps: up to 32 slots a warp (k <= 124) in one pass; 32 rows a warp
+@pytest.mark.parametrize("m", [1, 2, 4, 5, 31, 32, 33, 124, 125, 130])
+def test_gcv_values(api, h, m):
+    """GCV over the grid from the Hessenberg matrix of the same Arnoldi run, by NumPy's SVD."""
+    dims, sk = (24, 20), (24, 20)
+    t = np.exp(-0.5 * (np.arange(-4, 5) / 1.7) ** 2)
+    t /= t.sum()
+    A = [api.banded(1, 24, t), api.banded(2, 20, t)]
+    Cd = api.to_device(np.asfortranarray(np.random.default_rng(m).standard_normal(dims)))
+    grid = [1e-2, 3e-2, 1e-1, 0.3, 1.0]
+    _, r = h.gmres_solve(Cd, m, sk, 3, -1.0, A_factors=A, mu_grid=grid)
+    assert r.iters == m
+    kr = api.Krylov(h, dims, torch.float64, m, sk, 3, A_factors=A)
+    kr.start(Cd)
+    for _ in range(m):
+        kr.step()
+    view, H = kr.query()
+    U, s, _ = np.linalg.svd(H, full_matrices=True)
+    c = view.beta * U[0]   # U^T beta e1
+    for mu, got in zip(grid, r.gcv):
+        f = s * s / (s * s + mu)
+        res2 = np.sum(((1 - f) * c[:m]) ** 2) + c[m] ** 2
+        # residual and trace are sums of over 1e-4 of their terms: m rounding errors each, far below 1e-9
+        assert got == pytest.approx(res2 / (m + 1 - f.sum()) ** 2, rel=1e-9)
+    assert r.mu == grid[int(np.argmin(r.gcv))]
+    kr.close()
