@@ -58,6 +58,7 @@ k_apply_fused(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, FusedArgs a, Bat
   Zr = Zr.at(bi.off);
   stop = bsh(stop, bi.off);
   if (stop != nullptr && *stop) return;
+  pdl_trigger();
   const T* X = Xr.get<const T>();
   T* __restrict__ Y = Yr.get<T>();
   const T* Z = Zr.get<const T>();
@@ -194,6 +195,7 @@ k_apply_reg(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, FusedArgs a,
   Zr = Zr.at(bi.off);
   stop = bsh(stop, bi.off);
   if (stop != nullptr && *stop) return;
+  pdl_trigger();
   const T* X = Xr.get<const T>();
   T* __restrict__ Y = Yr.get<T>();
   const T* Z = Zr.get<const T>();
@@ -391,6 +393,7 @@ k_apply_small64(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, FusedArgs a, B
   Zr = Zr.at(bi.off);
   stop = bsh(stop, bi.off);
   if (stop != nullptr && *stop) return;
+  pdl_trigger();
   const double* X = Xr.get<const double>();
   double* __restrict__ Y = Yr.get<double>();
   const double* Z = Zr.get<const double>();
@@ -550,6 +553,7 @@ k_apply_st(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, StArgs a, const __g
   Zr = Zr.at(bi.off);
   stop = bsh(stop, bi.off);
   if (stop != nullptr && *stop) return;
+  pdl_trigger();
   const TI* X = Xr.get<const TI>();
   TO* __restrict__ Y = Yr.get<TO>();
   const float* Z = Zr.get<const float>();
@@ -778,6 +782,7 @@ __global__ void k_pass_band(PtrRef Xr, PtrRef Yr, int64_t L, int64_t I, int64_t 
   Yr = Yr.at(bo);
   stop = bsh(stop, bo);
   if (stop != nullptr && *stop) return;
+  pdl_trigger();
   const T* X = Xr.get<const T>();
   T* __restrict__ Y = Yr.get<T>();
   const int64_t total = L * I * R;
@@ -804,6 +809,7 @@ __global__ void k_pass_dense(PtrRef Xr, PtrRef Yr, int64_t L, int64_t I, int64_t
   Yr = Yr.at(bo);
   stop = bsh(stop, bo);
   if (stop != nullptr && *stop) return;
+  pdl_trigger();
   const T* X = Xr.get<const T>();
   T* __restrict__ Y = Yr.get<T>();
   const int64_t total = L * I * R;
@@ -828,6 +834,7 @@ __global__ void k_axpby(PtrRef Ar, PtrRef Yr, PtrRef Zr, double alpha, double be
   Zr = Zr.at(bo);
   stop = bsh(stop, bo);
   if (stop != nullptr && *stop) return;
+  pdl_trigger();
   const T* A = Ar.get<const T>();
   T* Y = Yr.get<T>();
   const T* Z = Zr.get<const T>();

@@ -49,6 +49,8 @@ __global__ void __launch_bounds__(GS_THREADS) k_gs_pass(Work w0, int pass, StepO
   const StepOpts o = o0.at(bo);
   Ctl* ctl = w.ctl;
   gate = bsh(gate, bo);
+  pdl_trigger();
+  pdl_wait();
   if (gate != nullptr && *gate) return;
   if (ctl->stop) return;
   const int J = (pass == 0) ? -1 : ctl->j;
@@ -165,6 +167,7 @@ __global__ void k_update(Work w0, StepOpts o0) {
   const Work w = w0.at(bo);
   const StepOpts o = o0.at(bo);
   Ctl* ctl = w.ctl;
+  pdl_wait();
   if (blockIdx.x == gridDim.x - 1) {
     givens_step(w, o);
     return;
@@ -370,6 +373,7 @@ __global__ void k_update_bf16(Work w0, StepOpts o0) {
   const Work w = w0.at(bo);
   const StepOpts o = o0.at(bo);
   Ctl* ctl = w.ctl;
+  pdl_wait();
   if (blockIdx.x == gridDim.x - 1) {
     givens_step(w, o);
     return;
@@ -483,6 +487,7 @@ __global__ void __launch_bounds__(UP_THREADS) k_update_ring(Work w0, StepOpts o0
   const Work w = w0.at(bo);
   const StepOpts o = o0.at(bo);
   Ctl* ctl = w.ctl;
+  pdl_wait();
   if (blockIdx.x == gridDim.x - 1) {
     givens_step(w, o);
     return;
@@ -627,9 +632,8 @@ cudaError_t launch_pass1(const Work& w, const StepOpts& o, cudaStream_t s) {
   share = share < 1 ? 1 : (share > 16 ? 16 : share);
   if (share > w.m) share = w.m;
   const dim3 g(static_cast<unsigned>(slices), w.dtype == RTG_F64 ? share : 1, static_cast<unsigned>(w.b.n));
-  if (w.dtype == RTG_F64) k_gs_pass<double><<<g, GS_THREADS, 0, s>>>(w, 1, o, nullptr);
-  else k_gs_pass<float><<<g, GS_THREADS, 0, s>>>(w, 1, o, nullptr);
-  return cudaGetLastError();
+  return launch_pdl(w.dtype == RTG_F64 ? k_gs_pass<double> : k_gs_pass<float>, g, dim3(GS_THREADS), 0, s, o.pdl, w, 1, o,
+                    nullptr);
 }
 
 
@@ -643,8 +647,7 @@ static cudaError_t launch_update_ring_cfg(const Work& w, const StepOpts& o, cuda
   const int nchunks = static_cast<int>((w.n + CE - 1) / CE);
   const int qblocks = static_cast<int>((w.d + UP_THREADS - 1) / UP_THREADS);
   const dim3 grid(static_cast<unsigned>(nchunks + qblocks + 1), 1, static_cast<unsigned>(w.b.n));
-  k_update_ring<TV, SLOT, STAGES><<<grid, UP_THREADS, sm, s>>>(w, o, nchunks);
-  return cudaGetLastError();
+  return launch_pdl(k_update_ring<TV, SLOT, STAGES>, grid, dim3(UP_THREADS), sm, s, o.pdl, w, o, nchunks);
 }
 
 template <typename TV>
@@ -668,10 +671,9 @@ cudaError_t launch_update(const Work& w, const StepOpts& o, cudaStream_t s) {
     return w.vdtype == RTG_BF16 ? launch_update_ring<__nv_bfloat16>(w, o, s) : launch_update_ring<float>(w, o, s);
   // one block more than the update needs: it runs the Givens step
   const unsigned nb = static_cast<unsigned>(w.b.n);
-  if (w.vdtype == RTG_BF16) k_update_bf16<<<dim3(ew_grid(w.n / 8 + 1) + 1, 1, nb), 256, 0, s>>>(w, o);
-  else if (w.dtype == RTG_F64) k_update<double><<<dim3(ew_grid(w.n) + 1, 1, nb), 256, 0, s>>>(w, o);
-  else k_update<float><<<dim3(ew_grid(w.n / 4 + 1) + 1, 1, nb), 256, 0, s>>>(w, o);
-  return cudaGetLastError();
+  const int64_t items = w.vdtype == RTG_BF16 ? w.n / 8 + 1 : (w.dtype == RTG_F64 ? w.n : w.n / 4 + 1);
+  auto kernel = w.vdtype == RTG_BF16 ? k_update_bf16 : (w.dtype == RTG_F64 ? k_update<double> : k_update<float>);
+  return launch_pdl(kernel, dim3(ew_grid(items) + 1, 1, nb), dim3(256), 0, s, o.pdl, w, o);
 }
 
 }  // namespace rtg

@@ -39,6 +39,8 @@ __device__ __forceinline__ double gk_coef(const Work& w, int phase) {
 template <typename T>
 __global__ void __launch_bounds__(GK_THREADS) k_gk_norm(Work w, int phase, StepOpts o) {
   Ctl* ctl = w.ctl;
+  pdl_trigger();
+  pdl_wait();
   if (ctl->stop) return;
   __shared__ double red[GS_MAXW][kRedCols];
   __shared__ double tot[4];
@@ -133,6 +135,7 @@ __global__ void __launch_bounds__(GK_THREADS) k_gk_norm(Work w, int phase, StepO
 template <typename T>
 __global__ void k_gk_update(Work w, int phase, PtrRef srcr, StepOpts o) {
   Ctl* ctl = w.ctl;
+  pdl_wait();
   if (phase == 2 && blockIdx.x == gridDim.x - 1) {   // Givens of column j - 1 beside the update
     givens_step(w, o);
     return;
@@ -212,19 +215,15 @@ static unsigned gk_ew_grid(int64_t n) {
 }
 
 cudaError_t launch_gk_norm(const Work& w, int phase, const StepOpts& o, cudaStream_t s) {
-  const int g = gk_grid(w.d);
-  if (w.dtype == RTG_F64) k_gk_norm<double><<<g, GK_THREADS, 0, s>>>(w, phase, o);
-  else k_gk_norm<float><<<g, GK_THREADS, 0, s>>>(w, phase, o);
-  return cudaGetLastError();
+  return launch_pdl(w.dtype == RTG_F64 ? k_gk_norm<double> : k_gk_norm<float>, dim3(gk_grid(w.d)), dim3(GK_THREADS), 0, s,
+                    o.pdl, w, phase, o);
 }
 
 cudaError_t launch_gk_update(const Work& w, int phase, PtrRef src, const StepOpts& o, cudaStream_t s) {
   const unsigned extra = (phase == 2) ? 1u : 0u;   // the Givens block
-  if (w.dtype == RTG_F64)
-    k_gk_update<double><<<gk_ew_grid(w.n) + extra, 256, 0, s>>>(w, phase, src, o);
-  else
-    k_gk_update<float><<<gk_ew_grid(w.n / 4 + 1) + extra, 256, 0, s>>>(w, phase, src, o);
-  return cudaGetLastError();
+  const bool f64 = w.dtype == RTG_F64;
+  return launch_pdl(f64 ? k_gk_update<double> : k_gk_update<float>, dim3(gk_ew_grid(f64 ? w.n : w.n / 4 + 1) + extra),
+                    dim3(256), 0, s, o.pdl, w, phase, src, o);
 }
 
 }  // namespace rtg

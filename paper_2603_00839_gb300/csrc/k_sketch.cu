@@ -514,7 +514,11 @@ k_sk_first_umma(PtrRef Xr, float* __restrict__ out, int64_t I, int64_t R, int64_
     mbar_init_fence();
     s_bad = 0;
   }
-  if (stopped) return;   // (the same in every thread)
+  if (stopped) {   // (the same in every thread)
+    pdl_wait();
+    return;
+  }
+  pdl_trigger();
   __syncthreads();
   auto rows_of = [&](int kb) {
     const int64_t i0 = static_cast<int64_t>(kb) * 64;
@@ -557,6 +561,7 @@ k_sk_first_umma(PtrRef Xr, float* __restrict__ out, int64_t I, int64_t R, int64_
       }
       asm volatile("cp.async.commit_group;\n" ::: "memory");
     };
+    pdl_wait();   // X, and the buffers this kernel writes
     for (int it = set; it < U_XSTAGES; it += U_LBUF) fill_x(it);
     unsigned char* Ls = smem + LOFF + set * LB;
     for (int it = set; it < steps; it += U_LBUF) {
@@ -676,6 +681,7 @@ k_sk_first_umma(PtrRef Xr, float* __restrict__ out, int64_t I, int64_t R, int64_
       mbar_wait(&full[kb % U_TSTAGES], static_cast<uint32_t>((kb / U_TSTAGES) & 1));
   } else if (xtma) {
     // ---------------------------------------------------------------- X ring (tensor map)
+    pdl_wait();
     int issued = 0;
     for (int it = 0; it < steps; ++it) {
       const int st = it % U_XSTAGES;
@@ -837,7 +843,11 @@ k_sk_inner_tc(PtrRef Xr, int in_blocked, float* __restrict__ out, int64_t L, int
     status = bsh(status, bo);
     stop = bsh(stop, bo);
   }
-  if (stop != nullptr && *stop) return;
+  if (stop != nullptr && *stop) {
+    pdl_wait();
+    return;
+  }
+  pdl_trigger();
   const float* X = Xr.get<const float>();
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t bar;
@@ -869,8 +879,10 @@ k_sk_inner_tc(PtrRef Xr, int in_blocked, float* __restrict__ out, int64_t L, int
       const uint32_t xbytes = bulk_in ? static_cast<uint32_t>(rows) * XA * 4 : 0u;
       mbar_expect(&bar, fbytes + xbytes);
       bulk_g2s(fB, fragB + (static_cast<int64_t>(nb) * kt_total + kc0) * N_NT * 32, fbytes, &bar);
+      if (kc0 == 0) pdl_wait();   // the input; Theta is older
       if (bulk_in) bulk_g2s(xa, X + ((r * ltiles + lt) * I + i0) * XA, static_cast<uint32_t>(rows) * XA * 4, &bar);
     }
+    if (kc0 == 0 && tid != 0) pdl_wait();
     // rows past I are zero; without bulk input, load the natural layout
     if (!bulk_in || rows < nk * 16)
     for (int idx = tid; idx < nk * 16 * 16; idx += TC_THREADS) {
@@ -996,6 +1008,8 @@ __global__ void k_sketch_mode(PtrRef Xr, T* __restrict__ Y, int64_t L, int64_t I
     bits = bsh(bits, bo);
     stop = bsh(stop, bo);
   }
+  pdl_trigger();
+  pdl_wait();
   if (stop != nullptr && *stop) return;
   const T* X = Xr.get<const T>();
   const int64_t total = L * s * R;
@@ -1064,7 +1078,7 @@ static unsigned grid_for(int64_t n) {
 int sketch_launches(const SketchPlan& sp) { return sp.nstage == 0 ? 1 : sp.nstage; }
 
 static cudaError_t sketch_f64(const SketchPlan& sp, const SketchScratch& sc, PtrRef X, double* out,
-                              const int* stop, cudaStream_t s, Batch b) {
+                              const int* stop, cudaStream_t s, Batch b, int pdl) {
   PtrRef src = X;
   for (int t = 0; t < sp.nstage; ++t) {
     const int k = sp.stage_mode[t];
@@ -1075,10 +1089,9 @@ static cudaError_t sketch_f64(const SketchPlan& sp, const SketchScratch& sc, Ptr
     const int block = sp.stage_out[t] * b.n <= 2432 * 32 ? 32 : 256;
     const int64_t want = (sp.stage_out[t] + block - 1) / block;
     const unsigned grid = static_cast<unsigned>(want < 152 * 32 ? want : 152 * 32);
-    k_sketch_mode<double><<<dim3(grid, 1, b.n), block, 0, s>>>(
-        src, dst, sp.stage_L[t], sp.stage_I[t], sp.stage_R[t], sp.stage_s[t],
-        sc.bits + sp.word_off[k], sp.wpr[k], scale, stop, b);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_pdl(k_sketch_mode<double>, dim3(grid, 1, b.n), dim3(block), 0, s, pdl, src, dst, sp.stage_L[t],
+                               sp.stage_I[t], sp.stage_R[t], sp.stage_s[t], sc.bits + sp.word_off[k], sp.wpr[k], scale,
+                               stop, b);
     if (e != cudaSuccess) return e;
     src = ref(dst);
   }
@@ -1125,7 +1138,7 @@ static bool make_xmap(CUtensorMap* m, const void* base, size_t elt, int64_t I, i
 template <typename TI, int NH>
 static cudaError_t launch_first_umma_nh(PtrRef src, float* dst, const SketchPlan& sp, int t, const uint32_t* fr,
                                         float scale, OutMap om, int* status, int poison, const int* stop,
-                                        cudaStream_t s, Batch b) {
+                                        cudaStream_t s, Batch b, int pdl) {
   constexpr size_t sm = u_smem<TI>();
   cudaError_t e = set_smem(k_sk_first_umma<TI, NH>, sm);
   if (e != cudaSuccess) return e;
@@ -1137,10 +1150,9 @@ static cudaError_t launch_first_umma_nh(PtrRef src, float* dst, const SketchPlan
                     make_xmap(&xm, src.base, sizeof(TI), sp.stage_I[t], sp.stage_R[t], b)) ? 1 : 0;
   const dim3 grid(static_cast<unsigned>((sp.stage_R[t] + NH * U_BN - 1) / (NH * U_BN)),
                   static_cast<unsigned>(sp.stage_ntile[t]), static_cast<unsigned>(b.n));
-  k_sk_first_umma<TI, NH><<<grid, U_THREADS, sm, s>>>(src, dst, sp.stage_I[t], sp.stage_R[t], sp.stage_s[t],
-                                                      sp.stage_kb[t], reinterpret_cast<const unsigned char*>(fr),
-                                                      scale, om, status, poison, stop, xm, xtma, b);
-  return cudaGetLastError();
+  return launch_pdl(k_sk_first_umma<TI, NH>, grid, dim3(U_THREADS), sm, s, pdl, src, dst, sp.stage_I[t], sp.stage_R[t],
+                    sp.stage_s[t], sp.stage_kb[t], reinterpret_cast<const unsigned char*>(fr), scale, om, status,
+                    poison, stop, xm, xtma, b);
 }
 
 // Groups of 32 columns per CTA: one while the groups fit two CTAs per SM at
@@ -1149,14 +1161,14 @@ static cudaError_t launch_first_umma_nh(PtrRef src, float* dst, const SketchPlan
 template <typename TI>
 static cudaError_t launch_first_umma(PtrRef src, float* dst, const SketchPlan& sp, int t, const uint32_t* fr,
                                      float scale, OutMap om, int* status, int poison, const int* stop,
-                                     cudaStream_t s, Batch b) {
+                                     cudaStream_t s, Batch b, int pdl) {
   const int64_t groups = ((sp.stage_R[t] + U_BN - 1) / U_BN) * sp.stage_ntile[t] * b.n;
-  return groups <= 2 * 152 ? launch_first_umma_nh<TI, 1>(src, dst, sp, t, fr, scale, om, status, poison, stop, s, b)
-                           : launch_first_umma_nh<TI, 2>(src, dst, sp, t, fr, scale, om, status, poison, stop, s, b);
+  return groups <= 2 * 152 ? launch_first_umma_nh<TI, 1>(src, dst, sp, t, fr, scale, om, status, poison, stop, s, b, pdl)
+                           : launch_first_umma_nh<TI, 2>(src, dst, sp, t, fr, scale, om, status, poison, stop, s, b, pdl);
 }
 
 static cudaError_t sketch_f32(const SketchPlan& sp, const SketchScratch& sc, PtrRef X, float* out,
-                              const SketchDots* dots, const int* stop, cudaStream_t s, int xdtype, Batch b) {
+                              const SketchDots* dots, const int* stop, cudaStream_t s, int xdtype, Batch b, int pdl) {
   PtrRef src = X;
   for (int t = 0; t < sp.nstage; ++t) {
     const bool last = (t == sp.nstage - 1);
@@ -1173,8 +1185,8 @@ static cudaError_t sketch_f32(const SketchPlan& sp, const SketchScratch& sc, Ptr
     cudaError_t e = cudaSuccess;
     if (sp.stage_umma[t]) {
       e = (t == 0 && xdtype == RTG_BF16)
-              ? launch_first_umma<__nv_bfloat16>(src, dst, sp, t, fr, scale, om, status, poison, stop, s, b)
-              : launch_first_umma<float>(src, dst, sp, t, fr, scale, om, status, poison, stop, s, b);
+              ? launch_first_umma<__nv_bfloat16>(src, dst, sp, t, fr, scale, om, status, poison, stop, s, b, pdl)
+              : launch_first_umma<float>(src, dst, sp, t, fr, scale, om, status, poison, stop, s, b, pdl);
     } else {
       const int64_t ltiles = (sp.stage_L[t] + 15) / 16;
       dim3 grid(static_cast<unsigned>(ltiles * sp.stage_R[t]),
@@ -1187,21 +1199,18 @@ static cudaError_t sketch_f32(const SketchPlan& sp, const SketchScratch& sc, Ptr
         constexpr size_t sm = inner_smem<32>();
         e = set_smem(k_sk_inner_tc<32>, sm);
         if (e != cudaSuccess) return e;
-        k_sk_inner_tc<32><<<grid, TC_THREADS, sm, s>>>(src, inb, dst, sp.stage_L[t], sp.stage_I[t],
-                                                       sp.stage_R[t], sp.stage_s[t], kt,
-                                                       reinterpret_cast<const uint2*>(fr), sp.stage_ntile[t],
-                                                       scale, om, dpass, wk, so, status, poison, stop, b);
+        e = launch_pdl(k_sk_inner_tc<32>, grid, dim3(TC_THREADS), sm, s, pdl, src, inb, dst, sp.stage_L[t], sp.stage_I[t],
+                       sp.stage_R[t], sp.stage_s[t], kt, reinterpret_cast<const uint2*>(fr), sp.stage_ntile[t], scale,
+                       om, dpass, wk, so, status, poison, stop, b);
       } else {
         constexpr size_t sm = inner_smem<16>();
         e = set_smem(k_sk_inner_tc<16>, sm);
         if (e != cudaSuccess) return e;
-        k_sk_inner_tc<16><<<grid, TC_THREADS, sm, s>>>(src, inb, dst, sp.stage_L[t], sp.stage_I[t],
-                                                       sp.stage_R[t], sp.stage_s[t], kt,
-                                                       reinterpret_cast<const uint2*>(fr), sp.stage_ntile[t],
-                                                       scale, om, dpass, wk, so, status, poison, stop, b);
+        e = launch_pdl(k_sk_inner_tc<16>, grid, dim3(TC_THREADS), sm, s, pdl, src, inb, dst, sp.stage_L[t], sp.stage_I[t],
+                       sp.stage_R[t], sp.stage_s[t], kt, reinterpret_cast<const uint2*>(fr), sp.stage_ntile[t], scale,
+                       om, dpass, wk, so, status, poison, stop, b);
       }
     }
-    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     src = ref(dst);
   }
@@ -1209,7 +1218,7 @@ static cudaError_t sketch_f32(const SketchPlan& sp, const SketchScratch& sc, Ptr
 }
 
 cudaError_t launch_sketch(const SketchPlan& sp, const SketchScratch& sc, PtrRef X, void* out,
-                          const SketchDots* dots, const int* stop, cudaStream_t s, int xdtype, Batch b) {
+                          const SketchDots* dots, const int* stop, cudaStream_t s, int xdtype, Batch b, int pdl) {
   if (xdtype < 0) xdtype = sp.dtype;
   // BF16 input is read only by a first stage on mode 1 (FP32 plans)
   if (xdtype == RTG_BF16 && (sp.dtype != RTG_F32 || sp.nstage == 0 || !sp.stage_first[0]))
@@ -1222,8 +1231,8 @@ cudaError_t launch_sketch(const SketchPlan& sp, const SketchScratch& sc, PtrRef 
     else k_copy<float><<<g, 256, 0, s>>>(X, static_cast<float*>(out), n, stop, b);
     return cudaGetLastError();
   }
-  if (sp.dtype == RTG_F64) return sketch_f64(sp, sc, X, static_cast<double*>(out), stop, s, b);
-  return sketch_f32(sp, sc, X, static_cast<float*>(out), sp.fused_dots ? dots : nullptr, stop, s, xdtype, b);
+  if (sp.dtype == RTG_F64) return sketch_f64(sp, sc, X, static_cast<double*>(out), stop, s, b, pdl);
+  return sketch_f32(sp, sc, X, static_cast<float*>(out), sp.fused_dots ? dots : nullptr, stop, s, xdtype, b, pdl);
 }
 
 }  // namespace rtg

@@ -738,7 +738,7 @@ rtg_status enqueue_step(const OpHolder& op, const SketchPlan& sp, const Work& w,
   {
     PhaseScope ps(pt, RTG_PHASE_SKETCH, step, sketch_launches(sp));
     SketchDots dots{&w, 1, so};
-    CK(launch_sketch(sp, sk, ref(w.W), fused ? w.S : w.Spart, fused ? &dots : nullptr, stop, s, w.vdtype, w.b));
+    CK(launch_sketch(sp, sk, ref(w.W), fused ? w.S : w.Spart, fused ? &dots : nullptr, stop, s, w.vdtype, w.b, so.pdl));
   }
   if (!fused) {
     PhaseScope ps(pt, RTG_PHASE_GS, step, 1);
@@ -861,7 +861,7 @@ rtg_status enqueue_gk_step(SolvePlan& P, const StepOpts& so, cudaStream_t s, Pha
   }
   {
     PhaseScope ps(pt, RTG_PHASE_SKETCH, step, sketch_launches(P.sp));
-    CK(launch_sketch(P.sp, P.sk, ref(w.W), w.S, nullptr, stop, s));
+    CK(launch_sketch(P.sp, P.sk, ref(w.W), w.S, nullptr, stop, s, -1, Batch{}, so.pdl));
   }
   {
     PhaseScope ps(pt, RTG_PHASE_GS, step, 1);
@@ -877,7 +877,7 @@ rtg_status enqueue_gk_step(SolvePlan& P, const StepOpts& so, cudaStream_t s, Pha
   }
   {
     PhaseScope ps(pt, RTG_PHASE_SKETCH, step, sketch_launches(P.sp));
-    CK(launch_sketch(P.sp, P.sk, ref(w.W), w.S, nullptr, stop, s));
+    CK(launch_sketch(P.sp, P.sk, ref(w.W), w.S, nullptr, stop, s, -1, Batch{}, so.pdl));
   }
   {
     PhaseScope ps(pt, RTG_PHASE_GS, step, 1);
@@ -941,7 +941,7 @@ rtg_status add_conditional(cudaStream_t cs, cudaGraphConditionalHandle hnd, cuda
 // The loop's condition handle goes to *loop when loop is not null.  The body
 // holds `steps` Arnoldi steps; kernels of a step after the stop return at once.
 rtg_status capture_solve(SolvePlan& P, cudaGraph_t g, cudaStream_t cs, cudaStream_t cs2,
-                         cudaGraphConditionalHandle* loop = nullptr, int steps = 1) {
+                         cudaGraphConditionalHandle* loop = nullptr, int steps = 1, int pdl = 0) {
   cudaGraphConditionalHandle hnd;
   CK(cudaGraphConditionalHandleCreate(&hnd, g, 1, cudaGraphCondAssignDefault));
   if (loop) *loop = hnd;
@@ -958,10 +958,12 @@ rtg_status capture_solve(SolvePlan& P, cudaGraph_t g, cudaStream_t cs, cudaStrea
     so.rs_cond = static_cast<unsigned long long>(rh);
   }
   CK(cudaStreamBeginCaptureToGraph(cs2, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
+  so.pdl = pdl;
   rtg_status st = RTG_OK;
   for (int q = 0; q < steps && st == RTG_OK; ++q)
     st = P.method == 1 ? enqueue_gk_step(P, so, cs2)
                        : enqueue_step(P.op, P.sp, P.w, P.dtype, P.tA, P.tB, P.sk, so, cs2);
+  so.pdl = 0;
   if (st == RTG_OK && P.w.cycles > 1) st = capture_restart_if(P, so, cs2);
   cudaGraph_t bodyout = nullptr;
   const cudaError_t e = cudaStreamEndCapture(cs2, &bodyout);
@@ -1021,11 +1023,11 @@ rtg_status branch_tail(cudaStream_t cs, const ChainLink& ch, rtg_status st) {
 }
 
 // Captures P's solve into g as a branch (after ch.after, if given).
-rtg_status build_branch(SolvePlan& P, cudaGraph_t g, const ChainLink& ch = ChainLink{}, int steps = 1) {
+rtg_status build_branch(SolvePlan& P, cudaGraph_t g, const ChainLink& ch = ChainLink{}, int steps = 1, int pdl = 0) {
   CaptureStreams cs;
   RK(cs.create());
   RK(begin_branch(cs.s[0], g, ch));
-  return end_capture(cs.s[0], branch_tail(cs.s[0], ch, capture_solve(P, g, cs.s[0], cs.s[1], nullptr, steps)));
+  return end_capture(cs.s[0], branch_tail(cs.s[0], ch, capture_solve(P, g, cs.s[0], cs.s[1], nullptr, steps, pdl)));
 }
 
 // A branch of a work-queue batch: it takes a problem of its class, then
@@ -1071,7 +1073,12 @@ rtg_status build_graph(SolvePlan& P) {
   // difference.  Batches keep one step (their branches fill each other's
   // gaps: 48 problems took 3769 us both ways), and so do restarted solves,
   // whose restart stands at the end of each body.
-  const rtg_status st = build_branch(P, g, ChainLink{}, P.w.cycles == 1 && P.w.m >= 8 ? 2 : 1);
+  // Programmatic dependents within a step: a launch gap of a kernel that waits
+  // for its predecessor's end costs 1 to 2 us, three to four a step (512 x 512:
+  // 267 -> 255 us; Golub-Kahan 512 x 512: 752 -> 718; FP64 64 x 64: 326 -> 316;
+  // 256 x 256 x 3 x 32 video: 2539 -> 2495).  Not in batches: a waiting kernel
+  // would hold SMs that the other branches could use.
+  const rtg_status st = build_branch(P, g, ChainLink{}, P.w.cycles == 1 && P.w.m >= 8 ? 2 : 1, 1);
   if (st != RTG_OK) {
     cudaGraphDestroy(g);
     return st;

@@ -341,6 +341,35 @@ inline cudaError_t set_smem(K* kernel, size_t bytes) {
 // Sets the thread-local message rtg_last_error() returns (rtg_api.cu).
 void record_error(const char* msg);
 
+// Programmatic dependent launch, for the kernels of an Arnoldi or Golub-Kahan
+// step of a plan that runs alone: the sketch, norm and update kernels start
+// while their predecessor still runs (it has called pdl_trigger, or its last
+// CTAs have ended), set up their barriers, and pdl_wait for it to complete
+// before they touch anything a kernel of this step writes.  Every CTA of a
+// kernel launched so waits before it ends, also where it returns at once, so a
+// kernel's end still means that all before it have ended.  The step's operator
+// kernel is launched plainly: what earlier steps and the setup wrote (the stop
+// flag, Theta) needs no wait.  Both calls do nothing in a plain launch.
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, int pdl, A&&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+#endif
+
 // ---------------------------------------------------------------- launchers
 // k_philox.cu
 cudaError_t launch_philox_words(uint64_t seed, uint64_t pid, int64_t n_words, uint64_t* out,
@@ -380,7 +409,7 @@ struct SketchDots;
 // first stage contracts mode 1.
 cudaError_t launch_sketch(const SketchPlan& sp, const SketchScratch& sc, PtrRef X, void* out,
                           const SketchDots* dots, const int* stop, cudaStream_t s, int xdtype = -1,
-                          Batch b = Batch{});
+                          Batch b = Batch{}, int pdl = 0);
 int sketch_launches(const SketchPlan& sp);
 
 // k_arnoldi.cu: the sketched Arnoldi process on a Work.
@@ -401,6 +430,8 @@ struct StepOpts {
   // sequence's last kernel)
   int use_rs_cond;
   unsigned long long rs_cond;
+  // 1: the step's kernels are launched as programmatic dependents (PDL)
+  int pdl;
   // lock-step batch: problems still running (the loop ends when it reaches 0);
   // shared by the batch, not moved with a problem's memory
   unsigned* group_left;
