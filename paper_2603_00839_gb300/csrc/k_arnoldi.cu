@@ -157,6 +157,18 @@ __device__ __forceinline__ float sketch_column_entry(float sv, const float* q, i
   return __fadd_rn(p.hi, lo);
 }
 
+// Whether a block of the update has nothing to do, the same for all its threads
+// (every thread of the block calls it): a breakdown, or a problem that stopped
+// in an earlier step (lock-step batch, two steps a loop body).  The Givens block
+// of the same launch writes stop and givens, so threads that each read them for
+// themselves could part: some would leave and the others wait on copies and
+// barriers that nobody set up.  A block that sees this launch's own stop may
+// leave or go on: V_{j+1} of a stopped solve is not read.
+__device__ __forceinline__ bool update_idle(const Ctl* ctl, const StepOpts& o) {
+  const volatile Ctl* c = ctl;
+  return __syncthreads_or(c->skip_update || c->j == 0 || (o.solve_mode && c->stop && !c->givens)) != 0;
+}
+
 // V_{j} = (W - sum_{i<j} h_i V_i) / h_{j,j-1};  Q_{j} = (S - sum_{i<j} h2_i Q_i) / h_{j,j-1}
 // FP32 tensors move as float4; four basis vectors are in flight per iteration.
 // The last block of the grid runs givens_step (Eq. 11S, rho_j, the stop
@@ -172,10 +184,7 @@ __global__ void k_update(Work w0, StepOpts o0) {
     givens_step(w, o);
     return;
   }
-  if (ctl->skip_update || ctl->j == 0) return;
-  // a problem that stopped in an earlier step (lock-step batch, two steps a
-  // loop body) has nothing to update
-  if (o.solve_mode && ctl->stop && !ctl->givens) return;
+  if (update_idle(ctl, o)) return;
   const int jj = ctl->j;
   if (jj > w.m) {   // V holds m+1 tensors: never write past V_m
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -378,8 +387,7 @@ __global__ void k_update_bf16(Work w0, StepOpts o0) {
     givens_step(w, o);
     return;
   }
-  if (ctl->skip_update || ctl->j == 0) return;
-  if (o.solve_mode && ctl->stop && !ctl->givens) return;
+  if (update_idle(ctl, o)) return;
   const int jj = ctl->j;
   if (jj > w.m) {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -492,8 +500,7 @@ __global__ void __launch_bounds__(UP_THREADS) k_update_ring(Work w0, StepOpts o0
     givens_step(w, o);
     return;
   }
-  if (ctl->skip_update || ctl->j == 0) return;
-  if (o.solve_mode && ctl->stop && !ctl->givens) return;
+  if (update_idle(ctl, o)) return;
   const int jj = ctl->j;
   if (jj > w.m) {   // V holds m+1 tensors: never write past V_m
     if (blockIdx.x == 0 && threadIdx.x == 0) {
