@@ -157,16 +157,18 @@ __device__ __forceinline__ float sketch_column_entry(float sv, const float* q, i
   return __fadd_rn(p.hi, lo);
 }
 
-// Whether a block of the update has nothing to do, the same for all its threads
-// (every thread of the block calls it): a breakdown, or a problem that stopped
-// in an earlier step (lock-step batch, two steps a loop body).  The Givens block
-// of the same launch writes stop and givens, so threads that each read them for
-// themselves could part: some would leave and the others wait on copies and
-// barriers that nobody set up.  A block that sees this launch's own stop may
-// leave or go on: V_{j+1} of a stopped solve is not read.
-__device__ __forceinline__ bool update_idle(const Ctl* ctl, const StepOpts& o) {
-  const volatile Ctl* c = ctl;
-  return __syncthreads_or(c->skip_update || c->j == 0 || (o.solve_mode && c->stop && !c->givens)) != 0;
+// The step index j of a block of the update, 0 if it has nothing to do, the same
+// for all its threads (every thread of the block calls it): a breakdown, or a
+// problem that stopped in an earlier step (lock-step batch, two steps a loop
+// body).  The Givens block of the same launch writes stop and givens, so threads
+// that each decided for themselves could part: some would leave and the others
+// wait on copies and barriers that nobody set up.  A block that sees this launch's
+// own stop may leave or go on: V_{j+1} of a stopped solve is not read.  The four
+// words are loaded together: one after another they cost 4 % of a solve.
+__device__ __forceinline__ int update_index(const Ctl* ctl, const StepOpts& o) {
+  const int skip = ctl->skip_update, j = ctl->j, stop = ctl->stop, givens = ctl->givens;
+  const int idle = (skip != 0) | (j == 0) | ((o.solve_mode != 0) & (stop != 0) & (givens == 0));
+  return __syncthreads_or(idle) ? 0 : j;
 }
 
 // V_{j} = (W - sum_{i<j} h_i V_i) / h_{j,j-1};  Q_{j} = (S - sum_{i<j} h2_i Q_i) / h_{j,j-1}
@@ -184,8 +186,8 @@ __global__ void k_update(Work w0, StepOpts o0) {
     givens_step(w, o);
     return;
   }
-  if (update_idle(ctl, o)) return;
-  const int jj = ctl->j;
+  const int jj = update_index(ctl, o);
+  if (jj == 0) return;
   if (jj > w.m) {   // V holds m+1 tensors: never write past V_m
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       ctl->status = RTG_ERR_INVALID_ARG;
@@ -387,8 +389,8 @@ __global__ void k_update_bf16(Work w0, StepOpts o0) {
     givens_step(w, o);
     return;
   }
-  if (update_idle(ctl, o)) return;
-  const int jj = ctl->j;
+  const int jj = update_index(ctl, o);
+  if (jj == 0) return;
   if (jj > w.m) {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       ctl->status = RTG_ERR_INVALID_ARG;
@@ -500,8 +502,8 @@ __global__ void __launch_bounds__(UP_THREADS) k_update_ring(Work w0, StepOpts o0
     givens_step(w, o);
     return;
   }
-  if (update_idle(ctl, o)) return;
-  const int jj = ctl->j;
+  const int jj = update_index(ctl, o);
+  if (jj == 0) return;
   if (jj > w.m) {   // V holds m+1 tensors: never write past V_m
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       ctl->status = RTG_ERR_INVALID_ARG;
