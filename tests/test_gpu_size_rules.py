@@ -236,3 +236,49 @@ def test_gcv_values(api, h, m):
         assert got == pytest.approx(res2 / (m + 1 - f.sum()) ** 2, rel=1e-9)
     assert r.mu == grid[int(np.argmin(r.gcv))]
     kr.close()
+
+
+# ------------------------------------------------------------------------ FP32 step finish, video apply
+
+# the finish keeps up to 56 rows of the Gram matrix in shared memory (J + 1 <= 56)
+@pytest.mark.parametrize("m,dims,sk", [(54, (64, 60), (32, 30)), (55, (64, 60), (32, 30)), (56, (64, 60), (32, 30)),
+                                       (58, (64, 60), (32, 30)), (57, (300, 290), (128, 128)), (57, (90, 17), (20, 17))])
+def test_fp32_finish_rows(api, h, m, dims, sk):
+    """The sketched basis is orthonormal and the Hessenberg columns are its sketches' coefficients."""
+    t = np.exp(-0.5 * (np.arange(-4, 5) / 1.1) ** 2)
+    A = [api.banded(1, dims[0], t / t.sum()), api.banded(2, dims[1], t / t.sum())]
+    Cd = api.to_device(np.random.default_rng(m).standard_normal(dims).astype(np.float32))
+    kr = api.Krylov(h, dims, torch.float32, m, sk, 3, A_factors=A)
+    kr.start(Cd)
+    for _ in range(m):
+        kr.step()
+    view, H = kr.query()
+    V, Q = kr.basis()
+    q = torch.stack([x.permute(1, 0).reshape(-1) for x in Q]).double().cpu().numpy()
+    assert view.j == m and not view.breakdown and q.shape[0] == m + 1
+    # each entry of Q is rounded once (2^-24) after its subtraction
+    assert np.abs(q @ q.T - np.eye(m + 1)).max() < 1e-6
+    for j in (0, m // 2, m - 1):
+        s = h.sketch(h.operator_apply(V[j], A), sk, 3).permute(1, 0).reshape(-1).double().cpu().numpy()
+        # S(Phi V_j) = sum_i h_ij Q_i: roundings of Q and S at 2^-24 of ||S||, FP32 sketch chains below 5e-6
+        assert np.linalg.norm(s - H[:j + 2, j] @ q[:j + 2]) < 1e-5 * np.linalg.norm(s)
+    kr.close()
+
+
+@pytest.mark.parametrize("dims", [(64, 16, 3, 37), (8, 5, 3, 2), (136, 33, 3, 11), (256, 256, 3, 10), (60, 17, 1, 40)])
+@pytest.mark.parametrize("bf16", [False, True])
+def test_video_apply_chunks(api, h, dims, bf16):
+    """Frames cut into chunks of every length, tiles at the tensor's edges, one and three channels."""
+    rng = np.random.default_rng(dims[3])
+    if bf16 and dims[0] % 8:
+        pytest.skip("BF16 rows are whole 16-byte pieces")
+    t1, t2, t4 = rng.standard_normal(9), rng.standard_normal(13), rng.standard_normal(5)
+    A = [api.banded(1, dims[0], t1), api.banded(2, dims[1], t2), api.banded(4, dims[3], t4)]
+    X = api.to_device(rng.standard_normal(dims).astype(np.float32))
+    if bf16:
+        X = api.to_device(X.cpu().numpy(), torch.bfloat16)
+    ref = oracle.apply_operator(X.float().cpu().double().numpy(),
+                                oracle.factor_matrices(dims, [(1, "banded", t1), (2, "banded", t2), (4, "banded", t4)], []))
+    got = h.operator_apply(X, A).float().cpu().double().numpy()
+    # at most 9 + 13 + 5 FP32 roundings along a chain (6e-8 each); BF16: one rounding of the result (2^-9)
+    assert _rel(got, ref) < (3e-3 if bf16 else 1e-6)
