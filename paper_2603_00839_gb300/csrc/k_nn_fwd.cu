@@ -233,7 +233,7 @@ k_conv_in3(const float* __restrict__ x, const __nv_bfloat16* __restrict__ wt, Fw
     tile[pix * 3 + c] = __float2bfloat16(v);
   }
   __syncthreads();
-  // offsets of this thread's patch entries: k = 16 s + 2 tig + {0, 1, 8, 9}, s = 0, 1 (k >= 27 meets zero weights)
+  // offsets of this thread's patch entries: k = 16 s + 2 tig + {0, 1, 8, 9}, s = 0, 1
   int off[8];
 #pragma unroll
   for (int u = 0; u < 8; ++u) {
@@ -247,6 +247,9 @@ k_conv_in3(const float* __restrict__ x, const __nv_bfloat16* __restrict__ wt, Fw
   for (int b = 0; b < BN / 8; ++b)
 #pragma unroll
     for (int c = 0; c < 4; ++c) acc[b][c] = 0.f;
+  // entries past the 27: zeros, as in the general kernel (a real value there would
+  // meet a zero weight, and an infinite one would make a NaN of it)
+  const uint32_t tail = tig == 0 ? 0xffffffffu : (tig == 1 ? 0xffffu : 0u);   // k = 24 + 2 tig, + 1
   const unsigned short* p0 = tl + (a * stride * hc + gid * stride) * 3;
   const unsigned short* p1 = p0 + 8 * stride * 3;
 #pragma unroll
@@ -257,6 +260,10 @@ k_conv_in3(const float* __restrict__ x, const __nv_bfloat16* __restrict__ wt, Fw
       const int u = 4 * s + 2 * h;
       af[2 * h] = static_cast<uint32_t>(p0[off[u]]) | static_cast<uint32_t>(p0[off[u + 1]]) << 16;
       af[2 * h + 1] = static_cast<uint32_t>(p1[off[u]]) | static_cast<uint32_t>(p1[off[u + 1]]) << 16;
+      if (u == 6) {
+        af[2 * h] &= tail;
+        af[2 * h + 1] &= tail;
+      }
     }
 #pragma unroll
     for (int nt = 0; nt < BN / 8; ++nt) {

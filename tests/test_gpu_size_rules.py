@@ -108,6 +108,26 @@ def test_convolution_forward(api, N, H, W, cin, cout, stride):
     assert float((y.double() - ref).norm()) <= 5e-6 * float(ref.norm())
 
 
+@pytest.mark.parametrize("cin,cout,stride", [(3, 8, 1), (3, 40, 2), (16, 8, 1), (48, 33, 2), (20, 8, 1)])
+def test_convolution_of_infinities(api, cin, cout, stride):
+    """Infinite pixels: infinities of the weights' signs (NaN where two signs meet), as direct summation gives
+    them; no padded entry of a kernel's K or halo turns them into NaN."""
+    x, wt = _bf16_exact((1, 20, 36, cin), 13), _bf16_exact((cout, 3, 3, cin), 14)
+    for i, j, c, v in ((0, 0, 0, np.inf), (5, 7, cin - 1, np.inf), (5, 8, cin - 1, -np.inf), (19, 35, cin - 1, -np.inf),
+                       (12, 20, 1, np.inf)):
+        x[0, i, j, c] = v
+    assert bool((wt != 0).all())
+    y = api.conv3x3(x, wt, None, stride=stride).cpu().double()
+    ref = torch.nn.functional.conv2d(x.cpu().double().permute(0, 3, 1, 2), wt.cpu().double().permute(0, 3, 1, 2),
+                                     stride=stride, padding=1).permute(0, 2, 3, 1)
+    assert bool(ref.isinf().any()) and torch.equal(y.isnan(), ref.isnan())
+    inf = ref.isinf()
+    assert torch.equal(y[inf], ref[inf]) and torch.equal(y.isinf(), inf)
+    ok = ref.isfinite()
+    # exact products, FP32 sums of at most 9 * 48 of them
+    assert float((y[ok] - ref[ok]).norm()) <= 5e-6 * float(ref[ok].norm())
+
+
 @pytest.mark.parametrize("cin", [16, 48])
 def test_convolution_kernels_agree(api, cin):
     """An input on no 16-byte boundary runs the general kernel: the tile kernel's bits."""
