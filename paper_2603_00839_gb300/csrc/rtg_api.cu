@@ -465,6 +465,7 @@ struct SolvePlan {
   int launches_setup = 0;                                         // reset and Theta, part of the prologue
   int launches_restart = 0;   // one restart sequence (graph: per restart; direct: every step)
   int direct_steps = 0;                                           // steps launched by the last direct solve
+  int body_steps = 1;                                             // steps of the graph's loop body
   int* stop_host = nullptr;                                       // pinned: ctl->stop read back per direct step
   bool ext_desc = false;  // desc/info live in a batch's buffers (not owned)
   // lock-step batch (w.b.n problems in one launch per kernel): the problems'
@@ -1078,7 +1079,8 @@ rtg_status build_graph(SolvePlan& P) {
   // 267 -> 255 us; Golub-Kahan 512 x 512: 752 -> 718; FP64 64 x 64: 326 -> 316;
   // 256 x 256 x 3 x 32 video: 2539 -> 2495).  Not in batches: a waiting kernel
   // would hold SMs that the other branches could use.
-  const rtg_status st = build_branch(P, g, ChainLink{}, P.w.cycles == 1 && P.w.m >= 8 ? 2 : 1, 1);
+  P.body_steps = P.w.cycles == 1 && P.w.m >= 8 ? 2 : 1;
+  const rtg_status st = build_branch(P, g, ChainLink{}, P.body_steps, 1);
   if (st != RTG_OK) {
     cudaGraphDestroy(g);
     return st;
@@ -1369,7 +1371,9 @@ void fill_info(const SolvePlan& P, const InfoDev& I, int mode, int n_mu, bool us
   info->elapsed_ms = ms;
   info->device_status = I.status;
   info->tile_config = P.w.upcfg;
-  info->launches = P.launches_pro + P.launches_epi + (use_graph ? I.iters : P.direct_steps) * P.launches_step +
+  // whole bodies: a solve that stops in a body's first step launches the second step's kernels too
+  const int graph_steps = (I.iters + P.body_steps - 1) / P.body_steps * P.body_steps;
+  info->launches = P.launches_pro + P.launches_epi + (use_graph ? graph_steps : P.direct_steps) * P.launches_step +
                    (use_graph ? I.restarts : P.direct_steps) * P.launches_restart;
   for (int k = 0; k < RTG_PHASE_COUNT; ++k) {
     info->phase_ms[k] = 0.0;

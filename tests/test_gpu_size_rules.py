@@ -211,6 +211,24 @@ def test_two_steps_a_loop_body_equal_direct_launches(api, h, dtype, m, stop_at):
         assert torch.equal(Xg, X) and np.array_equal(g.rho, r.rho)
 
 
+def test_launch_count_of_half_used_bodies(api, h):
+    """A solve that stops in the first step of a two-step body has launched the second step's kernels too."""
+    t = np.array([0.2, 1.0, 0.3])
+    A = [api.banded(1, 40, t), api.banded(2, 36, t)]
+    Cd = api.to_device(np.random.default_rng(2).standard_normal((40, 36)).astype(np.float32))
+    _, full = h.gmres_solve(Cd, 12, (20, 18), 3, 0.0, A_factors=A, use_graph=False)
+    count = {}
+    for k in (4, 5, 6, 7, 8):
+        kw = dict(A_factors=A, tol=float(full.rho[k - 1]) * (1 + 1e-9))
+        _, d = h.gmres_solve(Cd, 12, (20, 18), 3, 0.0, use_graph=False, **kw)
+        _, g = h.gmres_solve(Cd, 12, (20, 18), 3, 0.0, **kw)
+        assert d.iters == g.iters == k
+        count[k] = (d.launches, g.launches)
+    step = count[6][0] - count[5][0]   # direct launches stop at the step that stopped
+    assert step > 0 and all(d == count[4][0] + step * (k - 4) for k, (d, _) in count.items())
+    assert all(g == count[k + k % 2][0] for k, (_, g) in count.items() if k < 8)
+
+
 # ------------------------------------------------------------------------ Theta
 
 @pytest.mark.parametrize("dtype", [np.float32, np.float64])
