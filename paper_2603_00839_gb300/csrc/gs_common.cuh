@@ -100,36 +100,6 @@ __device__ __forceinline__ FF ff_warp_sum(FF v) {
   }
   return v;
 }
-// Product of two pairs, about 2^-46 relative; the low part may overlap the
-// high part's last bits (as in ff_add_lazy).
-__device__ __forceinline__ FF ff_mul(FF a, FF b) {
-  const float p = __fmul_rn(a.hi, b.hi);
-  const float e = __fmaf_rn(a.hi, b.hi, -p);
-  return {p, __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, e))};
-}
-__device__ __forceinline__ FF ff_twice(FF a) { return {2.f * a.hi, 2.f * a.lo}; }
-__device__ __forceinline__ FF ff_sub(FF a, FF b) { return ff_add_lazy(a, {-b.hi, -b.lo}); }
-__device__ __forceinline__ FF ff_mac(FF a, FF b, FF c) { return ff_add_lazy(c, ff_mul(a, b)); }   // a b + c
-__device__ __forceinline__ bool ff_finite(FF a) { return isfinite(a.hi) && isfinite(a.lo); }
-// The pair as the nearest float and the remainder.
-__device__ __forceinline__ FF ff_norm(FF v) {
-  const float s = __fadd_rn(v.hi, v.lo);
-  return {s, __fsub_rn(v.lo, __fsub_rn(s, v.hi))};
-}
-// Square root (v >= 0, normalised) and reciprocal, one Newton correction of
-// the FP32 value each: the relative error is that of the square of an FP32
-// rounding, about 2^-46.
-__device__ __forceinline__ FF ff_sqrt(FF v) {
-  const float r = __fsqrt_rn(v.hi);
-  if (!(r > 0.f)) return {r, 0.f};
-  const float e = __fadd_rn(__fmaf_rn(-r, r, v.hi), v.lo);
-  return ff_norm({r, __fdiv_rn(e, 2.f * r)});
-}
-__device__ __forceinline__ FF ff_recip(FF v) {
-  const float r = __frcp_rn(v.hi);
-  const float e = __fmaf_rn(-v.lo, r, __fmaf_rn(-v.hi, r, 1.f));
-  return ff_norm({r, __fmul_rn(r, e)});
-}
 __device__ __forceinline__ double ff_to_double(FF v) {
   return static_cast<double>(v.hi) + static_cast<double>(v.lo);
 }
@@ -159,7 +129,6 @@ struct Sum<float> {
   using V = FF;
   static __device__ __forceinline__ V zero() { return {0.f, 0.f}; }
   static __device__ __forceinline__ V add(V a, V b) { return ff_add_lazy(a, b); }
-  static __device__ __forceinline__ double dbl(V a) { return ff_to_double(a); }
   static __device__ __forceinline__ V ldcg(const V* p) {
     const float2 f = __ldcg(reinterpret_cast<const float2*>(p));
     return {f.x, f.y};
@@ -170,7 +139,6 @@ struct Sum<double> {
   using V = double;
   static __device__ __forceinline__ V zero() { return 0.0; }
   static __device__ __forceinline__ V add(V a, V b) { return a + b; }
-  static __device__ __forceinline__ double dbl(V a) { return a; }
   static __device__ __forceinline__ V ldcg(const V* p) { return __ldcg(p); }
 };
 
@@ -450,20 +418,20 @@ __device__ __forceinline__ typename Sum<T>::V column_share(const typename Sum<T>
 }
 
 // Ticket: returns true in every thread of the last block to finish, after
-// tot[0..ncols) holds the sum of all blocks' entries of each column (float-
-// float for T = float, FP64 for double; 256 threads).  The order is fixed, so
-// the result is deterministic.  FP32 data: a column is summed by G
+// tot[0..ncols) holds the sum of all blocks' entries of each column (summed in
+// float-float for T = float, in FP64 for double; 256 threads).  The order is
+// fixed, so the result is deterministic.  FP32 data: a column is summed by G
 // neighbouring lanes (a power of two), each taking every G-th entry with as
 // many loads in flight as it has entries (up to 16), and a shuffle tree adds
-// the lanes.  FP64 data: G = 256 / columns groups (at most 32), each with
+// the lanes; the total is converted once.  FP64 data: G = 256 / columns groups (at most 32), each with
 // every G-th entry, then one thread per column adds the groups' sums in a
 // pairwise tree (scratch: >= blockDim doubles).  The counter wraps back to
 // zero by itself.  pre (optional): called by every thread of the last block
 // right after the ticket, before its loads, e.g. to start asynchronous copies
 // that the caller needs after the combine.
 template <typename T, typename Pre = void (*)()>
-__device__ inline bool last_block_combine(const Work& w, int ncols, typename Sum<T>::V* tot, int* am_last,
-                                          double* scratch, Pre pre = nullptr) {
+__device__ inline bool last_block_combine(const Work& w, int ncols, double* tot, int* am_last, double* scratch,
+                                          Pre pre = nullptr) {
   using A = Sum<T>;
   using V = typename A::V;
   __syncthreads();
@@ -495,7 +463,7 @@ __device__ inline bool last_block_combine(const Work& w, int ncols, typename Sum
         other.lo = __shfl_xor_sync(0xffffffffu, acc.lo, o);
         acc = A::add(acc, other);
       }
-      if (g == 0 && c < ncols) tot[c] = ff_norm(acc);
+      if (g == 0 && c < ncols) tot[c] = ff_to_double(acc);
     }
     __syncthreads();
   } else {
@@ -548,11 +516,10 @@ __device__ __forceinline__ void set_inverse(Ctl* ctl, double d) {
 }
 
 // Start of a process (one thread): beta = ||R_0||_Theta = sqrt(s . s).
-template <typename T>
-__device__ inline void gs_finish_start(const Work& w, const StepOpts& o, const typename Sum<T>::V* tot) {
+__device__ inline void gs_finish_start(const Work& w, const StepOpts& o, const double* tot) {
   Ctl* ctl = w.ctl;
   const double tol = o.desc_tol ? *o.desc_tol : o.tol;
-  const double beta = sqrt(Sum<T>::dbl(tot[0]));
+  const double beta = sqrt(tot[0]);
   if (ctl->status != 0) {
     ctl->stop = 1;
   } else if (!isfinite(beta)) {
@@ -592,7 +559,7 @@ __device__ inline void gs_stage_gram_async(const Work& w, int J, double* sh) {
   const int n = J + 1;
   if (J < 1 || n > kGramSmemRows) return;
   const int lg = gram_smem_ld(n), ldg = gram_ld(w.m), pairs = (J + 1) / 2;
-  double* Gs = sh + (kMaxK + 2) + 4;   // (a float-float pair is as wide as a double)
+  double* Gs = sh + (kMaxK + 2) + 4;
   for (int e = threadIdx.x; e < J * pairs; e += blockDim.x) {
     const int p = e % pairs, k = e / pairs;
     const unsigned sa = static_cast<unsigned>(__cvta_generic_to_shared(&Gs[k * lg + 2 * p]));
@@ -608,8 +575,9 @@ __device__ inline void gs_stage_gram_async(const Work& w, int J, double* sh) {
 // the Gram matrix G = Q^T Q of the stored sketched basis so that a single
 // pass over Q suffices: h1 = Q^T s, h2 = Q^T (s - Q h1) = h1 - G h1,
 // h = h1 + h2 and h_{j+1,j}^2 = ||s - Q h||^2 = s.s - 2 h.h1 + h.(G h), all
-// in FP64 (FP64 data; gs_finish_gram_ff is FP32 data's).  Writes the Hessenberg column, h_{j+1,j} (0 on breakdown), the
-// breakdown and non-finite flags, and advances j.  The Givens update of
+// in FP64 (FP64 data; gs_finish_gram_f32 is FP32 data's).  Writes the
+// Hessenberg column, h_{j+1,j} (0 on breakdown), the breakdown and non-finite
+// flags, and advances j.  The Givens update of
 // Eq. 11S, rho_j and the stop rule follow in givens_step, off this
 // kernel's critical path.  Up to kGramSmemRows rows the Gram matrix is
 // staged in shared memory and every warp takes part in the two products
@@ -752,34 +720,40 @@ __device__ inline void gs_finish_gram(const Work& w, const StepOpts& o, int J, c
   }
 }
 
-// The step finish of FP32 data, in float-float arithmetic: the partial sums
-// are float-float already, and on this GPU an FP64 addition returns after 60
-// to 150 cycles and a conversion to FP32 after about 1000, against some 30 for
-// a float-float multiply-add.  G is stored as float-float pairs.  As
-// gs_finish_gram, with h_{j+1,j}^2 = s.s - h.(2 h1 - G h) in one sum; the
-// column also goes out as pairs for the update, and 1 / h_{j+1,j} with it.
-// What follows the second product is one warp's work (no block barrier).
-// Sketch group of one step (both contractions, dots and this chain; FP64
-// arithmetic, row-major partial sums and two separate sums before):
-// 512 x 512 x 3 28.6 -> 24.2 us, 1024 x 1024 x 3 40.4 -> 33.8 us,
-// 256 x 256 x 3 x 64 (1728 blocks to combine) 149 -> 107 us; the error of
-// solves against 64 bits is the same to two digits, ill-conditioned ones too.
-__device__ inline void gs_finish_gram_ff(const Work& w, const StepOpts& o, int J, const FF* tot, double* sh) {
+// The step finish of FP32 data: the same in FP64, from totals summed in
+// float-float, with h_{j+1,j}^2 = s.s - h.(2 h1 - G h) in one sum.  The column
+// also goes out as float-float pairs (48 bits) for the basis update, and
+// 1 / h_{j+1,j} with it.  On this GPU an FP64 addition returns after 60 to 150
+// cycles, so what follows the second product runs on several warps beside each
+// other without a block barrier: warps 0 and 1 both form the sum, warp 0 the
+// root and the flags, warp 1 the reciprocal, the others write the column.
+// The same chain in float-float (2^-46 a product) was no faster: 1024 x 1024,
+// 12 steps, 861 us in pairs and 846 so; 512 x 512 268 and 267; queue of 48
+// 2932 and 2885; video 2488 and 2467.
+__device__ inline void gs_finish_gram_f32(const Work& w, const StepOpts& o, int J, const double* tot, double* sh) {
   Ctl* ctl = w.ctl;
   const int ld = w.m + 1, ldg = gram_ld(w.m);
   const double bd_tol = o.desc_bd_tol ? *o.desc_bd_tol : o.bd_tol;   // loaded early, used at the end
-  const FF* h1 = tot;
-  const FF s2 = tot[J + 1];
-  const FF* grow = tot + J + 2;
-  FF* col = reinterpret_cast<FF*>(sh);   // h
-  FF* ext = col + (kMaxK + 2);          // 4 values
-  FF* G = reinterpret_cast<FF*>(w.G);
+  const double* h1 = tot;
+  const double s2 = tot[J + 1];
+  const double* grow = tot + J + 2;
+  double* col = sh;                     // h
+  double* G = w.G;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int n = J + 1;
   const bool small = n <= kGramSmemRows;
   const int lg = gram_smem_ld(n);
-  FF* Gs = ext + 4;                     // n x n, symmetric
-  FF* pr = Gs + n * lg;                 // [nw][n] partial products
+  double* Gs = col + (kMaxK + 2) + 4;   // n x n, symmetric (gs_stage_gram_async)
+  double* pr = Gs + n * lg;             // [nw][n] partial products
+  double* row = Gs;                     // beyond kGramSmemRows: h_i (2 h1 - G h)_i per row
+  auto psum = [&](int i) {   // the warps' partial rows as a fixed tree
+    if (nw == 8)
+      return ((pr[i] + pr[n + i]) + (pr[2 * n + i] + pr[3 * n + i])) +
+             ((pr[4 * n + i] + pr[5 * n + i]) + (pr[6 * n + i] + pr[7 * n + i]));
+    double u = 0.0;
+    for (int v = 0; v < nw; ++v) u += pr[v * n + i];
+    return u;
+  };
   if (small) {
     // G staged in shared memory (even row stride); each product G x runs
     // on every warp: warp w takes a slice of the columns, lane the rows
@@ -797,33 +771,18 @@ __device__ inline void gs_finish_gram_ff(const Work& w, const StepOpts& o, int J
     __syncthreads();
     const int ks = (n + nw - 1) / nw;
     const int k0 = warp * ks, k1 = (k0 + ks < n) ? k0 + ks : n;
-    auto gmul = [&](const FF* x) {   // pr[w][i] = sum over the warp's columns of G(k, i) x_k
+    auto gmul = [&](const double* x) {   // pr[w][i] = sum over the warp's columns of G(k, i) x_k
       for (int i = lane; i < n; i += 32) {
-        FF u = FF{0.f, 0.f};
-        for (int k = k0; k < k1; ++k) u = ff_mac(Gs[k * lg + i], x[k], u);
+        double u = 0.0;
+        for (int k = k0; k < k1; ++k) u = fma(Gs[k * lg + i], x[k], u);
         pr[warp * n + i] = u;
       }
     };
     gmul(h1);
     __syncthreads();
-    auto psum = [&](int i) {   // the warps' partial rows as a fixed tree
-      if (nw == 8)
-        return ff_add_lazy(ff_add_lazy(ff_add_lazy(pr[i], pr[n + i]), ff_add_lazy(pr[2 * n + i], pr[3 * n + i])),
-                      ff_add_lazy(ff_add_lazy(pr[4 * n + i], pr[5 * n + i]), ff_add_lazy(pr[6 * n + i], pr[7 * n + i])));
-      FF u = FF{0.f, 0.f};
-      for (int v = 0; v < nw; ++v) u = ff_add_lazy(u, pr[v * n + i]);
-      return u;
-    };
-    for (int i = threadIdx.x; i < n; i += blockDim.x) col[i] = ff_norm(ff_sub(ff_twice(h1[i]), psum(i)));
+    for (int i = threadIdx.x; i < n; i += blockDim.x) col[i] = 2.0 * h1[i] - psum(i);
     __syncthreads();
     gmul(col);
-    __syncthreads();
-    if (warp == 0) {
-      FF t = FF{0.f, 0.f};
-      for (int i = lane; i < n; i += 32) t = ff_mac(col[i], ff_sub(ff_twice(h1[i]), psum(i)), t);
-      t = ff_warp_sum(t);
-      if (lane == 0) ext[0] = t;
-    }
   } else {
     for (int i = threadIdx.x; i <= J; i += blockDim.x) {
       G[i + static_cast<int64_t>(ldg) * J] = grow[i];
@@ -832,52 +791,55 @@ __device__ inline void gs_finish_gram_ff(const Work& w, const StepOpts& o, int J
     __syncthreads();
     // h = 2 h1 - G h1: one warp per row, lanes across the columns
     for (int i = warp; i <= J; i += nw) {
-      FF gh = FF{0.f, 0.f};
-      for (int k = lane; k <= J; k += 32) gh = ff_mac(Sum<float>::ldcg(G + i + static_cast<int64_t>(ldg) * k), h1[k], gh);
-      gh = ff_warp_sum(gh);
-      if (lane == 0) col[i] = ff_norm(ff_sub(ff_twice(h1[i]), gh));
+      double gh = 0.0;
+      for (int k = lane; k <= J; k += 32) gh = fma(__ldcg(G + i + static_cast<int64_t>(ldg) * k), h1[k], gh);
+      gh = warp_sum(gh);
+      if (lane == 0) col[i] = 2.0 * h1[i] - gh;
     }
     __syncthreads();
-    FF* row = ext + 4;                  // h_i (2 h1 - G h)_i per row
     for (int i = warp; i <= J; i += nw) {
-      FF gh = FF{0.f, 0.f};
-      for (int k = lane; k <= J; k += 32) gh = ff_mac(Sum<float>::ldcg(G + i + static_cast<int64_t>(ldg) * k), col[k], gh);
-      gh = ff_warp_sum(gh);
-      if (lane == 0) row[i] = ff_mul(col[i], ff_sub(ff_twice(h1[i]), gh));
-    }
-    __syncthreads();
-    if (warp == 0) {
-      FF t = FF{0.f, 0.f};
-      for (int i = lane; i <= J; i += 32) t = ff_add_lazy(t, row[i]);
-      t = ff_warp_sum(t);
-      if (lane == 0) ext[0] = t;
+      double gh = 0.0;
+      for (int k = lane; k <= J; k += 32) gh = fma(__ldcg(G + i + static_cast<int64_t>(ldg) * k), col[k], gh);
+      gh = warp_sum(gh);
+      if (lane == 0) row[i] = col[i] * (2.0 * h1[i] - gh);
     }
   }
+  __syncthreads();
   double* Hc = w.H + static_cast<int64_t>(ld) * J;
-  if (warp != 0) {   // the column for the later kernels, beside warp 0's scalars
-    for (int i = static_cast<int>(threadIdx.x) - 32; i <= J; i += blockDim.x - 32) {
-      Hc[i] = ff_to_double(col[i]);
-      reinterpret_cast<float2*>(w.hf)[i] = make_float2(col[i].hi, col[i].lo);
+  if (warp > 1) {   // the column for the later kernels, beside the scalars
+    for (int i = static_cast<int>(threadIdx.x) - 64; i <= J; i += blockDim.x - 64) {
+      const FF h = double_split_rn(col[i]);
+      Hc[i] = col[i];
+      reinterpret_cast<float2*>(w.hf)[i] = make_float2(h.hi, h.lo);
     }
-    for (int i = J + 2 + static_cast<int>(threadIdx.x) - 32; i < ld; i += blockDim.x - 32) Hc[i] = 0.0;
+    for (int i = J + 2 + static_cast<int>(threadIdx.x) - 64; i < ld; i += blockDim.x - 64) Hc[i] = 0.0;
     return;
   }
+  double t = 0.0;
   bool bad = false;
-  for (int i = lane; i <= J; i += 32) bad |= !ff_finite(col[i]);
+  for (int i = lane; i <= J; i += 32) {
+    t = small ? fma(col[i], 2.0 * h1[i] - psum(i), t) : t + row[i];
+    bad |= !isfinite(col[i]);
+  }
+  t = warp_sum(t);
   bad = __any_sync(0xffffffffu, bad);
   if (lane != 0) return;
-  const FF t = ext[0];
-  const bool finite = ff_finite(s2) && ff_finite(t) && !bad;
-  const FF hn2 = ff_norm(ff_sub(s2, t));
-  const FF p2 = hn2.hi > 0.f ? hn2 : FF{0.f, 0.f};
-  const FF root = ff_sqrt(p2), inv = ff_recip(root);
-  const double hn = ff_to_double(root);
-  // h_{j+1,j} <= bd_tol ||S(Phi V_j)||, compared in squares
-  const bool breakdown = finite && ff_to_double(p2) <= bd_tol * bd_tol * ff_to_double(s2);
-  ctl->inv_hi = inv.hi;
-  ctl->inv_lo = inv.lo;
+  const double hn2 = s2 - t;
+  const double hn2p = hn2 > 0.0 ? hn2 : 0.0;
+  if (warp == 1) {   // (a breakdown's value is not used)
+    const double r = rsqrt(hn2p);
+    const FF f = double_split_rn(r);
+    ctl->inv = r;
+    ctl->inv_hi = f.hi;
+    ctl->inv_lo = f.lo;
+    return;
+  }
+  const bool finite = isfinite(s2) && isfinite(t) && !bad;
+  const double hn = sqrt(hn2p);
+  // h_{j+1,j} <= bd_tol ||S(Phi V_j)||, compared in squares (one square root fewer)
+  const bool breakdown = finite && (hn2p <= bd_tol * bd_tol * s2);
   Hc[J + 1] = breakdown ? 0.0 : hn;
-  ctl->pre2 = ff_to_double(s2);
+  ctl->pre2 = s2;
   ctl->hnext = hn;
   ctl->j = J + 1;
   if (!finite) ctl->status = RTG_ERR_NONFINITE;

@@ -973,15 +973,15 @@ k_sk_inner_tc(PtrRef Xr, int in_blocked, float* __restrict__ out, int64_t L, int
   // the reduction scratch reuses the dynamic shared memory
   __syncthreads();
   double(*red2)[kRedCols] = reinterpret_cast<double(*)[kRedCols]>(smem);
-  FF* tot = reinterpret_cast<FF*>(smem) + GS_MAXW * kRedCols;
+  double* tot = reinterpret_cast<double*>(smem) + GS_MAXW * kRedCols;
   block_partials<float, ITEMS>(w, vals, ix, ITEMS, J, red2);
   double* fin_sh = &red2[0][0];
   auto stage = [&]() { if (dots_pass > 0) gs_stage_gram_async(w, J, fin_sh); };
   if (!last_block_combine<float>(w, gs_ncols(J), tot, &am_last, fin_sh, stage)) return;
   if (dots_pass == 0) {
-    if (tid == 0) gs_finish_start<float>(w, o, tot);
+    if (tid == 0) gs_finish_start(w, o, tot);
   } else {
-    gs_finish_gram_ff(w, o, J, tot, fin_sh);
+    gs_finish_gram_f32(w, o, J, tot, fin_sh);
   }
 }
 

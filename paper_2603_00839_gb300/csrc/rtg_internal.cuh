@@ -195,7 +195,7 @@ struct Work {
   double* sn;                  // Givens sines (m)
   double* g;                   // rotated right-hand side (m+1)
   double* G;                   // (m+1) x (m+1) Gram matrix of the stored sketched basis, leading
-                               // dimension gram_ld(m) (float-float pairs for FP32 data)
+                               // dimension gram_ld(m)
   double* rho_hist;            // (m) per cycle
   double* y;                   // solution coefficients (m)
   double* gcv;                 // GCV values (kMaxMu)

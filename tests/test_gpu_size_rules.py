@@ -303,6 +303,22 @@ def test_fp32_finish_rows(api, h, m, dims, sk):
     kr.close()
 
 
+def test_fp32_finish_is_fp64(api, h):
+    """h_{j+1,j}^2 = s.s - h.(2 h1 - G h) far below s.s, from sums that float-float holds exactly: one rounding
+    at 2^-53 of s.s is left (2e-6 of the result); products kept to 48 bits would leave 1e-5."""
+    k = 2 * np.random.default_rng(1).integers(-2, 3, 256)
+    k[0] += 2 - int(k.sum()) % 4   # the mean of k is an odd multiple of 2^-7
+    dims = (256, 16)
+    kr = api.Krylov(h, dims, torch.float32, 2, dims, 3, A_factors=[api.dense(1, np.diag(1 + k * 2.0 ** -18))])
+    kr.start(api.to_device(np.ones(dims, dtype=np.float32)))   # beta = 64, every entry of V_0 and Q_0 2^-6
+    kr.step()
+    view, H = kr.query()
+    kr.close()
+    mean, square = float(k.mean()), float((k * k).mean())
+    assert view.beta == 64.0 and H[0, 0] == 1 + mean * 2.0 ** -18
+    assert H[1, 0] ** 2 == pytest.approx((square - mean * mean) * 2.0 ** -36, rel=3e-6, abs=0.0)
+
+
 @pytest.mark.parametrize("dims", [(64, 16, 3, 37), (8, 5, 3, 2), (136, 33, 3, 11), (256, 256, 3, 10), (60, 17, 1, 40)])
 @pytest.mark.parametrize("bf16", [False, True])
 def test_video_apply_chunks(api, h, dims, bf16):
