@@ -637,6 +637,7 @@ __device__ inline void gs_finish_gram(const Work& w, const StepOpts& o, int J, c
     };
     for (int i = threadIdx.x; i < n; i += blockDim.x) col[i] = 2.0 * h1[i] - wsum(i);
     __syncthreads();
+    pdl_trigger();
     gmul(col);
     __syncthreads();
     if (warp < 4) {   // a = h . h1 (warps 0, 1), b = h . (G h) (warps 2, 3) over the n <= 64 rows
@@ -782,6 +783,7 @@ __device__ inline void gs_finish_gram_f32(const Work& w, const StepOpts& o, int 
     __syncthreads();
     for (int i = threadIdx.x; i < n; i += blockDim.x) col[i] = 2.0 * h1[i] - psum(i);
     __syncthreads();
+    pdl_trigger();
     gmul(col);
   } else {
     for (int i = threadIdx.x; i <= J; i += blockDim.x) {

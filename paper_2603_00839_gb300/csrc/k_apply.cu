@@ -58,7 +58,6 @@ k_apply_fused(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, FusedArgs a, Bat
   Zr = Zr.at(bi.off);
   stop = bsh(stop, bi.off);
   if (stop != nullptr && *stop) return;
-  pdl_trigger();
   const T* X = Xr.get<const T>();
   T* __restrict__ Y = Yr.get<T>();
   const T* Z = Zr.get<const T>();
@@ -107,6 +106,7 @@ k_apply_fused(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, FusedArgs a, Bat
         acc[c][k] = s;
       }
     }
+    if (slab + bi.nz >= a.nslab) pdl_trigger();
 #pragma unroll
     for (int k = 0; k < FTY / 4; ++k) {                                // mode-3 mix + store
       const int64_t gx = x0 + tx, gy = y0 + ty + 4 * k;
@@ -195,7 +195,6 @@ k_apply_reg(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, FusedArgs a,
   Zr = Zr.at(bi.off);
   stop = bsh(stop, bi.off);
   if (stop != nullptr && *stop) return;
-  pdl_trigger();
   const T* X = Xr.get<const T>();
   T* __restrict__ Y = Yr.get<T>();
   const T* Z = Zr.get<const T>();
@@ -303,6 +302,7 @@ k_apply_reg(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, FusedArgs a,
       }
     }
     __syncthreads();
+    if (slab + bi.nz >= a.nslab) pdl_trigger();
     // mode 1 (along x): 4 consecutive outputs of one row per thread and channel
     T acc[NC][M1];
 #pragma unroll
@@ -393,7 +393,6 @@ k_apply_small64(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, FusedArgs a, B
   Zr = Zr.at(bi.off);
   stop = bsh(stop, bi.off);
   if (stop != nullptr && *stop) return;
-  pdl_trigger();
   const double* X = Xr.get<const double>();
   double* __restrict__ Y = Yr.get<double>();
   const double* Z = Zr.get<const double>();
@@ -415,6 +414,7 @@ k_apply_small64(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, FusedArgs a, B
       in_s[c][yy][xx] = v ? __ldcg(Xs + c * plane + static_cast<int64_t>(gy) * I1 + gx) : 0.0;
     }
     __syncthreads();
+    if (slab + bi.nz >= a.nslab) pdl_trigger();
     for (int e = threadIdx.x; e < NC * STY64 * Wd; e += ST64_THREADS) {   // mode 2, every staged column
       const int row = e / Wd, xx = e - row * Wd, c = row / STY64, y = row - c * STY64;
       double s = 0.0;
@@ -553,7 +553,6 @@ k_apply_st(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, StArgs a, const __g
   Zr = Zr.at(bi.off);
   stop = bsh(stop, bi.off);
   if (stop != nullptr && *stop) return;
-  pdl_trigger();
   const TI* X = Xr.get<const TI>();
   TO* __restrict__ Y = Yr.get<TO>();
   const float* Z = Zr.get<const float>();
@@ -664,6 +663,7 @@ k_apply_st(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, StArgs a, const __g
         __syncthreads();
       }
       if (u + 1 < uend) load_frame(u + 1, buf ^ 1);   // in flight during the filters
+      if (u + 1 >= uend) pdl_trigger();
       // mode 2 first over every staged column of every channel: task = (channel, column pair, 4 output rows)
       const TI* ins = in_s + buf * PITCH;
       for (int task = threadIdx.x; task < TASKS; task += ST_THREADS) {
@@ -782,7 +782,6 @@ __global__ void k_pass_band(PtrRef Xr, PtrRef Yr, int64_t L, int64_t I, int64_t 
   Yr = Yr.at(bo);
   stop = bsh(stop, bo);
   if (stop != nullptr && *stop) return;
-  pdl_trigger();
   const T* X = Xr.get<const T>();
   T* __restrict__ Y = Yr.get<T>();
   const int64_t total = L * I * R;
@@ -809,7 +808,6 @@ __global__ void k_pass_dense(PtrRef Xr, PtrRef Yr, int64_t L, int64_t I, int64_t
   Yr = Yr.at(bo);
   stop = bsh(stop, bo);
   if (stop != nullptr && *stop) return;
-  pdl_trigger();
   const T* X = Xr.get<const T>();
   T* __restrict__ Y = Yr.get<T>();
   const int64_t total = L * I * R;
@@ -834,7 +832,6 @@ __global__ void k_axpby(PtrRef Ar, PtrRef Yr, PtrRef Zr, double alpha, double be
   Zr = Zr.at(bo);
   stop = bsh(stop, bo);
   if (stop != nullptr && *stop) return;
-  pdl_trigger();
   const T* A = Ar.get<const T>();
   T* Y = Yr.get<T>();
   const T* Z = Zr.get<const T>();

@@ -49,7 +49,6 @@ __global__ void __launch_bounds__(GS_THREADS) k_gs_pass(Work w0, int pass, StepO
   const StepOpts o = o0.at(bo);
   Ctl* ctl = w.ctl;
   gate = bsh(gate, bo);
-  pdl_trigger();
   pdl_wait();
   if (gate != nullptr && *gate) return;
   if (ctl->stop) return;

@@ -39,7 +39,6 @@ __device__ __forceinline__ double gk_coef(const Work& w, int phase) {
 template <typename T>
 __global__ void __launch_bounds__(GK_THREADS) k_gk_norm(Work w, int phase, StepOpts o) {
   Ctl* ctl = w.ctl;
-  pdl_trigger();
   pdl_wait();
   if (ctl->stop) return;
   __shared__ double red[GS_MAXW][kRedCols];
@@ -70,6 +69,7 @@ __global__ void __launch_bounds__(GK_THREADS) k_gk_norm(Work w, int phase, StepO
     w.part[static_cast<int64_t>(threadIdx.x) * w.part_rows + blockIdx.x] =
         warps_total(red, blockDim.x >> 5, threadIdx.x);
   if (!last_block_combine<double>(w, 2, tot, &am_last, &red[0][0])) return;
+  pdl_trigger();
   if (threadIdx.x != 0) return;
   const double nrm = sqrt(tot[0] > 0.0 ? tot[0] : 0.0);
   const double pre = sqrt(tot[1] > 0.0 ? tot[1] : 0.0);

@@ -518,7 +518,6 @@ k_sk_first_umma(PtrRef Xr, float* __restrict__ out, int64_t I, int64_t R, int64_
     pdl_wait();
     return;
   }
-  pdl_trigger();
   __syncthreads();
   auto rows_of = [&](int kb) {
     const int64_t i0 = static_cast<int64_t>(kb) * 64;
@@ -711,6 +710,7 @@ k_sk_first_umma(PtrRef Xr, float* __restrict__ out, int64_t I, int64_t R, int64_
   tc_fence_after();
   const uint32_t tmem = tmem_holder;
   bad = failed();
+  pdl_trigger();
   // the blocked layout of the next stage with M = 1 (no unsketched mode in
   // between): whole rows of 20 floats, contiguous for consecutive columns of
   // one r2, leave as bulk stores (the scratch tensors are 16-byte aligned)
@@ -847,7 +847,6 @@ k_sk_inner_tc(PtrRef Xr, int in_blocked, float* __restrict__ out, int64_t L, int
     pdl_wait();
     return;
   }
-  pdl_trigger();
   const float* X = Xr.get<const float>();
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t bar;
@@ -924,6 +923,7 @@ k_sk_inner_tc(PtrRef Xr, int in_blocked, float* __restrict__ out, int64_t L, int
     }
     __syncthreads();
   }
+  if (dots_pass < 0) pdl_trigger();   // (with the dots, the finish does)
   if (!ok) {   // timed out: zeros where the solve records the timeout (the CTA still takes
                // part in the dots), else NaN (never a silent partial sum)
     const float fill = poison ? __int_as_float(0x7fc00000) : 0.f;
@@ -1008,7 +1008,6 @@ __global__ void k_sketch_mode(PtrRef Xr, T* __restrict__ Y, int64_t L, int64_t I
     bits = bsh(bits, bo);
     stop = bsh(stop, bo);
   }
-  pdl_trigger();
   pdl_wait();
   if (stop != nullptr && *stop) return;
   const T* X = Xr.get<const T>();

@@ -342,10 +342,18 @@ inline cudaError_t set_smem(K* kernel, size_t bytes) {
 void record_error(const char* msg);
 
 // Programmatic dependent launch, for the kernels of an Arnoldi or Golub-Kahan
-// step of a plan that runs alone: the sketch, norm and update kernels start
-// while their predecessor still runs (it has called pdl_trigger, or its last
-// CTAs have ended), set up their barriers, and pdl_wait for it to complete
-// before they touch anything a kernel of this step writes.  Every CTA of a
+// step of a stand-alone plan: the sketch, norm and update kernels start
+// while their predecessor still runs (all its CTAs have called pdl_trigger or
+// ended), set up their barriers, and pdl_wait for it to complete
+// before they touch anything a kernel of this step writes.  A waiting CTA holds
+// its shared memory, registers and tensor memory, which the kernels of other
+// solves in flight could use: so a kernel triggers late, when its last phase
+// starts (the launch takes 1 to 2 us), and one whose last phase a single block
+// runs (a step's finish) triggers from that block.  512 x 512, 12 steps, several
+// solves submitted on streams of their own, us a solve with triggers at the
+// kernels' start / late / without dependents: one 480 / 466 / 488, two 374 / 294
+// / 322, four 266 / 213 / 230, eight 226 / 190 / 202; 1024 x 1024, four: 524 /
+// 469 / 473, eight 483 / 477 / 467.  333 x 517, 8 steps, alone: 514 / 500 / 517.  Every CTA of a
 // kernel launched so waits before it ends, also where it returns at once, so a
 // kernel's end still means that all before it have ended.  The step's operator
 // kernel is launched plainly: what earlier steps and the setup wrote (the stop

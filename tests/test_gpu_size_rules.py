@@ -229,6 +229,43 @@ def test_launch_count_of_half_used_bodies(api, h):
     assert all(g == count[k + k % 2][0] for k, (_, g) in count.items() if k < 8)
 
 
+# (dims, sketch, dtype, dense factor, BF16 basis): the kernel chains that run as dependent launches
+@pytest.mark.parametrize("dims,sk,dtype,dense,bf16", [
+    ((40, 36), (20, 36), np.float32, False, False),          # one mode sketched: the Gram-Schmidt pass is a kernel
+    ((40, 36), (20, 36), np.float64, False, False),
+    ((40, 36), (40, 36), np.float32, False, False),          # nothing sketched: a copy in the sketch's place
+    ((41, 37), (20, 18), np.float32, False, False),          # rows on no 16 bytes: register kernels, 4-byte copies
+    ((40, 36, 5), (20, 18, 5), np.float32, True, False),     # an operator of several kernels
+    ((64, 40, 3, 9), (24, 20, 3, 4), np.float32, False, True),
+    ((512, 448, 3), (128, 128, 3), np.float32, False, False),   # many blocks a kernel
+    ((333, 517, 3), (128, 128, 3), np.float32, False, False),
+    ((256, 232, 3), (40, 40, 3), np.float64, False, False),
+])
+def test_dependent_launches_equal_direct_launches(api, h, dims, sk, dtype, dense, bf16):
+    """Kernels of a step that start before their predecessor has ended, alone and with three other solves in
+    flight on streams of their own, give the bits of plain launches that the host waits for."""
+    rng = np.random.default_rng(dims[1])
+    t = np.array([0.2, 1.0, 0.3])
+    A = [api.banded(k + 1, n, t) for k, n in enumerate(dims) if n > 5]
+    B = [api.dense(3, np.eye(5) + 0.1 * rng.standard_normal((5, 5)))] if dense else []
+    Cd = api.to_device(np.asfortranarray(rng.standard_normal(dims).astype(dtype)))
+    kw = dict(A_factors=A, B_factors=B)
+    for solve in (h.gmres_solve,) if bf16 else (h.gmres_solve, h.gk_solve):
+        if bf16:
+            kw["bf16_basis"] = True
+        X, r = solve(Cd, 9, sk, 3, 1e-2, use_graph=False, **kw)
+        for _ in range(3):
+            Xg, g = solve(Cd, 9, sk, 3, 1e-2, **kw)
+            assert g.iters == r.iters == 9 and torch.equal(Xg, X) and np.array_equal(g.rho, r.rho)
+    X, r = h.gmres_solve(Cd, 9, sk, 3, 1e-2, use_graph=False, **kw)
+    streams = [torch.cuda.Stream() for _ in range(4)]
+    torch.cuda.synchronize()
+    for _ in range(2):
+        pend = [h.gmres_submit(Cd, 9, sk, 3, 1e-2, slot=i, stream=s, **kw) for i, s in enumerate(streams)]
+        for Xg, g in [h.gmres_wait(p) for p in pend]:
+            assert torch.equal(Xg, X) and np.array_equal(g.rho, r.rho)
+
+
 # ------------------------------------------------------------------------ Theta
 
 @pytest.mark.parametrize("dtype", [np.float32, np.float64])
