@@ -151,6 +151,14 @@ struct RegGeom {
   static constexpr int OFF = RA - RR;
   static constexpr int Wd = RTX + 2 * RA;
   static constexpr int Ht = RTY + 2 * RR;
+  // Channels that share the two barriers: all, where the second tile of all of
+  // them leaves the SM its CTAs; FP64 at radii 10 to 16 goes channel by channel
+  // (512 x 512 x 3, mixed, radius 12 / 16: 127 / 169 us so, 136 / 175 all at once).
+  template <int NC>
+  static constexpr int group = sizeof(T) == 4 || RR <= 9 ? NC : 1;
+  // halo tiles, mode-2 results, room to align them to 128 bytes
+  template <int NC>
+  static constexpr size_t smem = size_t(NC * Ht + group<NC> * RTY) * Wd * sizeof(T) + 128;
 };
 
 // Paired FP32 FMA (fma.rn.f32x2): two lanes of independent multiply-adds
@@ -204,6 +212,8 @@ k_apply_reg(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, FusedArgs a,
   constexpr int NPAIR = Wd / 2;                 // mode-2 pass: column pairs
   constexpr int V2 = 4;                          // mode-2 pass: output rows per task
   constexpr int M1 = 4;                          // mode-1 pass: outputs per thread
+  constexpr int CG = G::template group<NC>;      // channels between barriers
+  static_assert(NC % CG == 0, "whole groups of channels");
   static_assert(Wd % 2 == 0, "mode-2 tasks");
   static_assert(RTY * (RTX / M1) == FTHREADS, "mode-1 tasks: one per thread");
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -212,7 +222,7 @@ k_apply_reg(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, FusedArgs a,
   // there explicitly (the launch adds 128 bytes of slack)
   const uint32_t raw = static_cast<uint32_t>(__cvta_generic_to_shared(smem_raw));
   T* in_s = reinterpret_cast<T*>(smem_raw + (((raw + 127u) & ~127u) - raw));   // NC x Ht x Wd
-  T* tmp = in_s + NC * Ht * Wd;                  // NC x RTY x Wd
+  T* tmp = in_s + NC * Ht * Wd;                  // CG x RTY x Wd
   const int x0 = blockIdx.x * RTX;
   const int y0 = blockIdx.y * RTY;
   const int I1 = static_cast<int>(a.I1), I2 = static_cast<int>(a.I2);
@@ -272,69 +282,73 @@ k_apply_reg(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, FusedArgs a,
     }
     asm volatile("cp.async.wait_all;\n" ::: "memory");
     __syncthreads();
-    // mode 2 first (along y, all Wd staged columns of all channels): task =
-    // (channel, column pair, 4 output rows), paired FMAs over the two columns, tap
-    // by tap over a sliding window of rows: one copy of a tap serves the four outputs
-    for (int task = threadIdx.x; task < NC * NPAIR * (RTY / V2); task += FTHREADS) {
-      const int pr = task % NPAIR, cg = task / NPAIR, g = cg % (RTY / V2), c = cg / (RTY / V2);
-      const T* col = in_s + (c * Ht + g * V2) * Wd + 2 * pr;
-      Pair<T> win[V2], s[V2];
-#pragma unroll
-      for (int o = 0; o < V2; ++o) {
-        win[o] = load_pair(col + o * Wd);
-        s[o] = {static_cast<T>(0), static_cast<T>(0)};
-      }
-#pragma unroll
-      for (int t = 0; t < NT; ++t) {
-#pragma unroll
-        for (int o = 0; o < V2; ++o) s[o] = pfma(t2(t), win[(o + t) % V2], s[o]);
-        if (t + 1 < NT) win[t % V2] = load_pair(col + (t + V2) * Wd);
-      }
-      T* q = tmp + (c * RTY + g * V2) * Wd + 2 * pr;
-#pragma unroll
-      for (int o = 0; o < V2; ++o) {
-        if constexpr (sizeof(T) == 4) {
-          *reinterpret_cast<float2*>(q + o * Wd) = make_float2(s[o].x, s[o].y);
-        } else {
-          q[o * Wd] = s[o].x;
-          q[o * Wd + 1] = s[o].y;
-        }
-      }
-    }
-    __syncthreads();
-    if (slab + bi.nz >= a.nslab) pdl_trigger();
-    // mode 1 (along x): 4 consecutive outputs of one row per thread and channel
     T acc[NC][M1];
 #pragma unroll
-    for (int c = 0; c < NC; ++c) {
+    for (int c0 = 0; c0 < NC; c0 += CG) {   // channels c0 .. c0 + CG - 1
+      if (c0 > 0) __syncthreads();            // (the channel before is done with tmp)
+      // mode 2 first (along y, all Wd staged columns of the channels): task =
+      // (channel, column pair, 4 output rows), paired FMAs over the two columns, tap
+      // by tap over a sliding window of rows: one copy of a tap serves the four outputs
+      for (int task = threadIdx.x; task < CG * NPAIR * (RTY / V2); task += FTHREADS) {
+        const int pr = task % NPAIR, cg = task / NPAIR, g = cg % (RTY / V2), c = cg / (RTY / V2);
+        const T* col = in_s + ((c0 + c) * Ht + g * V2) * Wd + 2 * pr;
+        Pair<T> win[V2], s[V2];
 #pragma unroll
-      for (int o = 0; o < M1; ++o) acc[c][o] = 0;
-      T win[M1 + 2 * RR];
-      if (sizeof(T) == 4) {
-        // aligned 16-byte loads covering the window, which starts OFF & 3 floats in
-        constexpr int A0 = OFF & ~3, SH = OFF & 3;
-        constexpr int NV = (SH + M1 + 2 * RR + 3) / 4;
-        const float4* rp = reinterpret_cast<const float4*>(tmp + (c * RTY + oy) * Wd + ox + A0);
-        float buf[NV * 4];
-#pragma unroll
-        for (int v4 = 0; v4 < NV; ++v4) {
-          const float4 q = rp[v4];
-          buf[4 * v4] = q.x;
-          buf[4 * v4 + 1] = q.y;
-          buf[4 * v4 + 2] = q.z;
-          buf[4 * v4 + 3] = q.w;
+        for (int o = 0; o < V2; ++o) {
+          win[o] = load_pair(col + o * Wd);
+          s[o] = {static_cast<T>(0), static_cast<T>(0)};
         }
 #pragma unroll
-        for (int u = 0; u < M1 + 2 * RR; ++u) win[u] = static_cast<T>(buf[SH + u]);
-      } else {
-        const T* row = tmp + (c * RTY + oy) * Wd + ox + OFF;
+        for (int t = 0; t < NT; ++t) {
 #pragma unroll
-        for (int u = 0; u < M1 + 2 * RR; ++u) win[u] = row[u];
+          for (int o = 0; o < V2; ++o) s[o] = pfma(t2(t), win[(o + t) % V2], s[o]);
+          if (t + 1 < NT) win[t % V2] = load_pair(col + (t + V2) * Wd);
+        }
+        T* q = tmp + (c * RTY + g * V2) * Wd + 2 * pr;
+#pragma unroll
+        for (int o = 0; o < V2; ++o) {
+          if constexpr (sizeof(T) == 4) {
+            *reinterpret_cast<float2*>(q + o * Wd) = make_float2(s[o].x, s[o].y);
+          } else {
+            q[o * Wd] = s[o].x;
+            q[o * Wd + 1] = s[o].y;
+          }
+        }
       }
+      __syncthreads();
+      if (c0 + CG == NC && slab + bi.nz >= a.nslab) pdl_trigger();
+      // mode 1 (along x): 4 consecutive outputs of one row per thread and channel
 #pragma unroll
-      for (int t = 0; t < NT; ++t)
+      for (int c = 0; c < CG; ++c) {
 #pragma unroll
-        for (int o = 0; o < M1; ++o) acc[c][o] += t1(t) * win[o + t];
+        for (int o = 0; o < M1; ++o) acc[c0 + c][o] = 0;
+        T win[M1 + 2 * RR];
+        if (sizeof(T) == 4) {
+          // aligned 16-byte loads covering the window, which starts OFF & 3 floats in
+          constexpr int A0 = OFF & ~3, SH = OFF & 3;
+          constexpr int NV = (SH + M1 + 2 * RR + 3) / 4;
+          const float4* rp = reinterpret_cast<const float4*>(tmp + (c * RTY + oy) * Wd + ox + A0);
+          float buf[NV * 4];
+#pragma unroll
+          for (int v4 = 0; v4 < NV; ++v4) {
+            const float4 q = rp[v4];
+            buf[4 * v4] = q.x;
+            buf[4 * v4 + 1] = q.y;
+            buf[4 * v4 + 2] = q.z;
+            buf[4 * v4 + 3] = q.w;
+          }
+#pragma unroll
+          for (int u = 0; u < M1 + 2 * RR; ++u) win[u] = static_cast<T>(buf[SH + u]);
+        } else {
+          const T* row = tmp + (c * RTY + oy) * Wd + ox + OFF;
+#pragma unroll
+          for (int u = 0; u < M1 + 2 * RR; ++u) win[u] = row[u];
+        }
+#pragma unroll
+        for (int t = 0; t < NT; ++t)
+#pragma unroll
+          for (int o = 0; o < M1; ++o) acc[c0 + c][o] += t1(t) * win[o + t];
+      }
     }
     const int gy = y0 + oy;
     if (gy < I2) {
@@ -977,7 +991,7 @@ static cudaError_t apply_t(const OpPlan& op, PtrRef X, PtrRef Y, double alpha, d
 #define RTG_REG_CASE(NC, RR)                                                                          \
   if (a.nc == NC && rr == RR) {                                                                       \
     using Gm = RegGeom<RR, T>;                                                                        \
-    const size_t smem = static_cast<size_t>(NC) * (Gm::Ht + RTY) * Gm::Wd * sizeof(T) + 128;             \
+    const size_t smem = Gm::template smem<NC>;                                                        \
     e = set_smem(k_apply_reg<T, NC, RR>, smem);                                                       \
     if (e != cudaSuccess) return e;                                                                   \
     CUtensorMap xm;                                                                                   \

@@ -170,6 +170,12 @@ def test_fp64_apply_tiles(api, h, dims, radius, mix):
     assert _rel(got.cpu().numpy(), ref) < 1e-13
 
 
+# three mixed channels at the radii whose channels go one by one
+@pytest.mark.parametrize("dims,radius", [((200, 100, 3), 10), ((70, 33, 3), 16)])
+def test_fp64_apply_tiles_of_mixed_channels(api, h, dims, radius):
+    test_fp64_apply_tiles(api, h, dims, radius, True)
+
+
 @pytest.mark.parametrize("m", [1, 3, 20])
 def test_fp64_gram_schmidt_shared_columns(api, h, m):
     """Steps whose column count is below, at and above the blocks that share a slice of the sketch."""
