@@ -170,8 +170,10 @@ def test_fp64_apply_tiles(api, h, dims, radius, mix):
     assert _rel(got.cpu().numpy(), ref) < 1e-13
 
 
-# three mixed channels at the radii whose channels go one by one
-@pytest.mark.parametrize("dims,radius", [((200, 100, 3), 10), ((70, 33, 3), 16)])
+# three mixed channels: the small tiles' last size and the first of the large ones, and the radii whose
+# channels go one by one
+@pytest.mark.parametrize("dims,radius", [((384, 320, 3), 9), ((384, 352, 3), 9), ((384, 384, 3), 3), ((200, 100, 3), 10),
+                                         ((70, 33, 3), 16)])
 def test_fp64_apply_tiles_of_mixed_channels(api, h, dims, radius):
     test_fp64_apply_tiles(api, h, dims, radius, True)
 
