@@ -103,7 +103,9 @@ typedef struct rtg_opts {
                                         restarts from its least-squares iterate;
                                         m * (max_restarts + 1) <= RTG_MAX_KRYLOV */
     double breakdown_tol;            /* breakdown if h_{j+1,j} <= breakdown_tol * ||S(Phi V_j)||;
-                                        0 selects 1e-12 (F64) / 1e-6 (F32) */
+                                        0 selects 1e-12 (F64) / 1e-6 (F32); FP32 tensors are
+                                        rounded at 2^-24, so levels below about 1e-6 of
+                                        ||S(Phi V_j)|| are rounding for them */
     int32_t flags;                   /* RTG_FLAG_* */
     int32_t slot;                    /* workspace slot, 0..RTG_MAX_SLOTS-1: solves that may be
                                         in flight at the same time on different streams must use

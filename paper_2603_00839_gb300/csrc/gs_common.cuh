@@ -186,33 +186,13 @@ __device__ __forceinline__ T coef_as(double x) {
 // Gram matrix G = Q^T Q).  The start of a process (J = -1) has only s . s.
 __device__ __forceinline__ int gs_ncols(int J) { return J < 0 ? 1 : 2 * J + 3; }
 
-// Reduce-scatter of 32 float-float values across a warp: in five halving
-// rounds each lane keeps one half of its values and hands the other half
-// to its partner, adding what it receives; afterwards v[0] of lane l is the
-// warp total of value l.  31 exchanges per lane instead of 32 x 5 for 32
-// separate warp sums, and the adds of a round are independent.  The tree
+// Reduce-scatter of NV = 2, 4, ..., 32 float-float values across a warp: in
+// log2(NV) halving rounds inside aligned groups of NV lanes each lane keeps one
+// half of its values and hands the other half to its partner, adding what it
+// receives; then butterfly sums across the groups; afterwards v[0] of lane l is
+// the warp total of value l % NV.  NV = 32: 31 exchanges per lane instead of 32
+// x 5 for separate warp sums, and the adds of a round are independent.  The tree
 // is fixed, so the sums are deterministic.
-__device__ __forceinline__ void ff_reduce_scatter32(FF (&v)[32]) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int r = 0; r < 5; ++r) {
-    const int half = 16 >> r;          // also the partner's lane offset
-    const bool up = (lane & half) != 0;
-#pragma unroll
-    for (int k = 0; k < half; ++k) {
-      const FF give = up ? v[k] : v[k + half];
-      const FF keep = up ? v[k + half] : v[k];
-      FF got;
-      got.hi = __shfl_xor_sync(0xffffffffu, give.hi, half);
-      got.lo = __shfl_xor_sync(0xffffffffu, give.lo, half);
-      v[k] = ff_add_lazy(keep, got);
-    }
-  }
-}
-
-// The same for NV = 2, 4, ..., 32 values: log2(NV) halving rounds inside
-// aligned groups of NV lanes, then butterfly sums across the groups;
-// afterwards v[0] of lane l is the warp total of value l % NV.
 template <int NV>
 __device__ __forceinline__ void ff_reduce_scatter(FF (&v)[NV]) {
   const int lane = threadIdx.x & 31;

@@ -627,8 +627,8 @@ cudaError_t launch_start(const Work& w, PtrRef src, const StepOpts& o, bool fuse
   return cudaGetLastError();
 }
 
-// FP64: up to sixteen blocks share the columns of one slice of the sketch, as
-// many as two waves of the GPU hold (64 x 64 x 3, 7 steps: the pass 23.7 us
+// FP64: up to sixteen blocks share the columns of one slice of the sketch, while
+// there are two or fewer an SM (64 x 64 x 3, 7 steps: the pass 23.7 us
 // with one, 14.3 us with the finish's staging and splitting as they are now).
 cudaError_t launch_pass1(const Work& w, const StepOpts& o, cudaStream_t s) {
   const int slices = gs_grid(w.d);

@@ -8,17 +8,10 @@
 #include <cuda_bf16.h>
 
 #include "nn_internal.cuh"
+#include "nn_mma.cuh"
 
 namespace rtg {
 namespace nn {
-
-__device__ __forceinline__ void mma16816(float* c, const uint32_t* a, uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-      "{%0,%1,%2,%3};\n"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
 
 static unsigned grid_of(int64_t n) {
   int64_t b = (n + 255) / 256;
@@ -160,7 +153,7 @@ k_conv_fwd(const float* __restrict__ x, const __nv_bfloat16* __restrict__ wt, co
       for (int nt = 0; nt < BN / 8; ++nt) {
         const uint32_t b0 = *reinterpret_cast<const uint32_t*>(&Bs[buf][nt * 8 + gid][kk + tig * 2]);
         const uint32_t b1 = *reinterpret_cast<const uint32_t*>(&Bs[buf][nt * 8 + gid][kk + tig * 2 + 8]);
-        mma16816(acc[nt], af, b0, b1);
+        mma_k16(acc[nt], af, b0, b1);
       }
     }
     if (more) {

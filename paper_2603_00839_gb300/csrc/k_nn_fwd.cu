@@ -47,8 +47,7 @@ __device__ __forceinline__ void fwd_store(const FwdEpilogue& ep, float v, int c,
 // multiplied; all operands go through ldmatrix.  Eight warps, 4 along the
 // pixels x 2 along the channels (8 x 1 for BN = 8).  SPLIT: K is cut every
 // `kchunk` values and the slices are added in a second accumulator.
-// 512 x 512, c = 32 (bound by the tensor pipe's mma.sync rate and shared-memory
-// reads of the operands): see conv_tile for both sides.
+// Bound by the tensor pipe's mma.sync rate and the operands' shared-memory reads.
 template <int BN, bool SPLIT>
 __global__ void __launch_bounds__(256)
 k_conv_tile(const float* __restrict__ x, const __nv_bfloat16* __restrict__ wt, FwdEpilogue ep, int H, int W, int C,

@@ -94,7 +94,6 @@ const char* make_sketch_plan(int order, const int64_t* dims, const int64_t* sdim
     sp.stage_first[t] = (L == 1) ? 1 : 0;
     sp.stage_kt[t] = static_cast<int>((I + 15) / 16);
     sp.stage_out[t] = L * s * R;
-    sp.stage_split[t] = 1;
     if (dtype == RTG_F32) {
       sp.frag_off[t] = frag;
       if (sp.stage_first[t]) {
@@ -135,7 +134,6 @@ const char* make_sketch_plan(int order, const int64_t* dims, const int64_t* sdim
     }
   }
   sp.part_elems = part;
-  sp.last_split = 1;
   sp.tmp_elems = part;
   sp.fused_dots = (dtype == RTG_F32 && sp.nstage > 0 && !sp.stage_first[sp.nstage - 1]) ? 1 : 0;
   sp.dots_blocks = 0;

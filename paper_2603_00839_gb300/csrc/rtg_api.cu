@@ -1068,17 +1068,21 @@ rtg_status build_graph(SolvePlan& P) {
   cudaGraph_t g = nullptr;
   CK(cudaGraphCreate(&g, 0));
   // Two steps a body where a solve may take many: starting a WHILE body again
-  // costs 4 to 5 us, the idle kernels of a half-used last body about 15, so
-  // from 8 steps on (odd stops included) the pair wins.  1024 x 1024, 12 steps:
-  // 902 -> 875 us; 333 x 517, 20 steps: 1013 -> 977; at 5 to 7 steps no
-  // difference.  Batches keep one step (their branches fill each other's
+  // costs 4 to 5 us, the idle kernels of a half-used last body 8 (GMRES) to 15
+  // (Golub-Kahan).  How many steps a solve takes is not known here; m >= 8 stands
+  // for many.  512 x 512, m = 50, stopped after k = 1, 2, ..., 8 steps, one / two a
+  // body, us: GMRES 129 / 136, 167 / 153, 199 / 197, 229 / 215, 264 / 258, 297 /
+  // 276, 327 / 318, 366 / 340; Golub-Kahan 182 / 190, 233 / 227, 293 / 299, 357 /
+  // 341, 418 / 415, 471 / 454, 531 / 526, 593 / 567: the pair loses where a solve
+  // stops after its first step (Golub-Kahan: or third) and wins or ties at every
+  // other stop.  Batches keep one step (their branches fill each other's
   // gaps: 48 problems took 3769 us both ways), and so do restarted solves,
   // whose restart stands at the end of each body.
   // Programmatic dependents within a step: a launch gap of a kernel that waits
-  // for its predecessor's end costs 1 to 2 us, three to four a step (512 x 512:
-  // 267 -> 255 us; Golub-Kahan 512 x 512: 752 -> 718; FP64 64 x 64: 326 -> 316;
-  // 256 x 256 x 3 x 32 video: 2539 -> 2495).  Not in batches: a waiting kernel
-  // would hold SMs that the other branches could use.
+  // for its predecessor's end costs 1 to 2 us, three to four a step (512 x 512,
+  // 12 steps: 488 -> 466 us; Golub-Kahan 512 x 512, 8 steps: 612 -> 570; 128 x 128,
+  // 12 steps: 407 -> 390).  Also where several solves are in flight (figures at
+  // pdl_wait).  Not in batches, whose branches are always many.
   P.body_steps = P.w.cycles == 1 && P.w.m >= 8 ? 2 : 1;
   const rtg_status st = build_branch(P, g, ChainLink{}, P.body_steps, 1);
   if (st != RTG_OK) {

@@ -254,7 +254,6 @@ struct SketchPlan {
   int nstage;
   int stage_mode[kMaxOrder];
   int stage_first[kMaxOrder];  // 1: L == 1 (first-mode tensor-core kernel)
-  int stage_split[kMaxOrder];  // K split (partial outputs)
   int stage_kt[kMaxOrder];     // K tiles of 16
   int stage_ntile[kMaxOrder];  // 128-row tiles (L == 1 stages, tcgen05) or n8 tiles (later stages) of the sketch size
   int stage_kb[kMaxOrder];     // K blocks of 64 (tcgen05 stages)
@@ -274,7 +273,6 @@ struct SketchPlan {
   int64_t frag_off[kMaxOrder];    // uint32 offset of the stage's Theta images (tcgen05) or fragments (mma.sync)
   int64_t frag_words;
   int64_t part_elems;             // elements of each scratch tensor
-  int last_split;                 // partial copies of the final sketch (1)
   int fused_dots;                 // the last stage can run the first Gram-Schmidt pass
   int64_t dots_blocks;            // CTAs of that last stage (rows of partial sums)
 };

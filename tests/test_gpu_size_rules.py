@@ -382,6 +382,19 @@ def test_fp32_finish_rows(api, h, m, dims, sk):
     kr.close()
 
 
+@pytest.mark.parametrize("k", [1, 2, 4])
+@pytest.mark.parametrize("sk", [(64, 60), (64, 24), (32, 30)])
+def test_fp32_breakdown_after_k_steps(api, h, k, sk):
+    """An operator with k distinct eigenvalues: the Krylov space is invariant after k steps, and the remainder of
+    the k-th (roundings at 2^-24 of the operator's norm, a few of them a step) is below the level asked for."""
+    dims = (64, 60)
+    A = [api.dense(1, np.diag(1.0 + np.arange(64) % k))]
+    Cd = api.to_device(np.random.default_rng(k).standard_normal(dims).astype(np.float32))
+    for kw in (dict(), dict(use_graph=False)):
+        _, r = h.gmres_solve(Cd, 12, sk, 3, 0.0, A_factors=A, breakdown_tol=1e-5, **kw)
+        assert r.breakdown and r.converged and r.iters == k
+
+
 def test_fp32_finish_is_fp64(api, h):
     """h_{j+1,j}^2 = s.s - h.(2 h1 - G h) far below s.s, from sums that float-float holds exactly: one rounding
     at 2^-53 of s.s is left (2e-6 of the result); products kept to 48 bits would leave 1e-5."""
