@@ -106,7 +106,7 @@ k_apply_fused(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, FusedArgs a, Bat
         acc[c][k] = s;
       }
     }
-    if (slab + bi.nz >= a.nslab) pdl_trigger();
+    pdl_trigger();
 #pragma unroll
     for (int k = 0; k < FTY / 4; ++k) {                                // mode-3 mix + store
       const int64_t gx = x0 + tx, gy = y0 + ty + 4 * k;
@@ -316,7 +316,7 @@ k_apply_reg(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, FusedArgs a,
         }
       }
       __syncthreads();
-      if (c0 + CG == NC && slab + bi.nz >= a.nslab) pdl_trigger();
+      if (c0 + CG == NC) pdl_trigger();
       // mode 1 (along x): 4 consecutive outputs of one row per thread and channel
 #pragma unroll
       for (int c = 0; c < CG; ++c) {
@@ -428,7 +428,7 @@ k_apply_small64(PtrRef Xr, PtrRef Yr, PtrRef Zr, const int* stop, FusedArgs a, B
       in_s[c][yy][xx] = v ? __ldcg(Xs + c * plane + static_cast<int64_t>(gy) * I1 + gx) : 0.0;
     }
     __syncthreads();
-    if (slab + bi.nz >= a.nslab) pdl_trigger();
+    pdl_trigger();
     for (int e = threadIdx.x; e < NC * STY64 * Wd; e += ST64_THREADS) {   // mode 2, every staged column
       const int row = e / Wd, xx = e - row * Wd, c = row / STY64, y = row - c * STY64;
       double s = 0.0;
