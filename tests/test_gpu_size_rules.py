@@ -428,3 +428,9 @@ def test_video_apply_chunks(api, h, dims, bf16):
     got = h.operator_apply(X, A).float().cpu().double().numpy()
     # at most 9 + 13 + 5 FP32 roundings along a chain (6e-8 each); BF16: one rounding of the result (2^-9)
     assert _rel(got, ref) < (3e-3 if bf16 else 1e-6)
+
+
+# frames by the hundred, in one chunk a frame and in chunks of several
+@pytest.mark.parametrize("dims", [(8, 5, 1, 300), (8, 5, 1, 700), (64, 16, 3, 311)])
+def test_video_apply_many_frames(api, h, dims):
+    test_video_apply_chunks(api, h, dims, False)
