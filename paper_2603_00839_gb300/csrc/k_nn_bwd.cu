@@ -471,11 +471,14 @@ k_conv_dx(const __nv_bfloat16* __restrict__ dzb, const __nv_bfloat16* __restrict
 
 cudaError_t conv_dx(const __nv_bfloat16* dzb, const __nv_bfloat16* w, const float* addend, float* dx, int N, int H,
                     int W, int C, int stride, int cout, bool up2, cudaStream_t s) {
-  const int bn = C <= 32 ? 32 : (C <= 64 ? 64 : 128);
+  int bn = C <= 32 ? 32 : (C <= 64 ? 64 : 128);
   int kp = (cout + 15) / 16 * 16;
   if (kp > 128) kp = 128;
   const int Ho = H / stride, Wo = W / stride;
   const int ta = (Ho + DX_TA - 1) / DX_TA, tb = (Wo + DX_TB - 1) / DX_TB;
+  // fewer input channels per CTA where all of them leave most SMs idle (4 x 4 pixels,
+  // 1024 channels: 8 CTAs of 128); the result does not depend on it
+  while (bn > 32 && int64_t(ta) * tb * stride * stride * N * ((C + bn - 1) / bn) < 76) bn /= 2;
   const size_t smem = (size_t(DX_PIX) * (kp + 8) + size_t(2) * kp * (bn + 8)) * 2;
   const int vecw = C % 8 == 0 && aligned16(w) ? 1 : 0, u = up2 ? 1 : 0;
   const int per = 65535 / (stride * stride);   // images of one launch (the grid's z limit)

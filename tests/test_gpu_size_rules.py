@@ -90,6 +90,12 @@ def test_convolution_gradients(api, N, H, W, cin, cout, stride):
         assert float((got.double() - ref).norm()) <= 5e-6 * float(ref.norm()) + 1e-12
 
 
+# enough tiles for all input channels in one CTA: 100 of them at 64 and 128 channels, and a class of stride 2
+@pytest.mark.parametrize("N,H,W,cin,cout,stride", [(1, 80, 160, 128, 16, 1), (1, 79, 157, 64, 8, 1), (2, 80, 160, 128, 8, 2)])
+def test_convolution_gradients_of_large_grids(api, N, H, W, cin, cout, stride):
+    test_convolution_gradients(api, N, H, W, cin, cout, stride)
+
+
 @pytest.mark.parametrize("N,H,W,cin,cout,stride", [
     (1, 1, 1, 3, 1, 1),          # the three-channel kernel's smallest
     (2, 18, 34, 3, 40, 2),       # and its stride 2, ragged, 64 output channels at a time
