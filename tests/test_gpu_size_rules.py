@@ -361,6 +361,28 @@ def test_tikhonov_of_one_column_is_as_exact_as_plain_operations(api, h):
     assert np.mean(got_err) <= 1.25 * np.mean(plain_err) + 1e-17
 
 
+@pytest.mark.parametrize("lam", [1e-2, -1.0])
+@pytest.mark.parametrize("e", [-470, 470])
+def test_tikhonov_of_extreme_operators(api, h, e, lam):
+    """Operator and observation times 2^e and mu times 2^2e leave the solution: squares outside 2^+-900 take the
+    plain operations, which differ from the refined ones by a rounding each."""
+    dims = (24, 20)
+    t = np.exp(-0.5 * (np.arange(-4, 5) / 1.7) ** 2)
+    t /= t.sum()
+    C = np.random.default_rng(3).standard_normal(dims)
+    grid = np.array([1e-3, 1e-2, 1e-1])
+    out = []
+    for f in (0, e):
+        A = [api.banded(1, 24, t * 2.0 ** f), api.banded(2, 20, t)]
+        kw = dict(mu_grid=grid * 4.0 ** f) if lam < 0 else {}
+        X, r = h.gk_solve(api.to_device(np.asfortranarray(C * 2.0 ** f)), 6, (12, 10), 3,
+                          lam if lam < 0 else lam * 4.0 ** f, A_factors=A, **kw)
+        assert r.iters == 6 and r.device_status == 0
+        out.append((X.cpu().numpy(), r.mu / 4.0 ** f))
+    # roundings of six reflections and of the rotations, times the condition of R_mu (below 1e2)
+    assert out[0][1] == out[1][1] and _rel(out[1][0], out[0][0]) < 1e-12
+
+
 # ------------------------------------------------------------------------ FP32 step finish, video apply
 
 # the finish keeps up to 56 rows of the Gram matrix in shared memory (J + 1 <= 56)
